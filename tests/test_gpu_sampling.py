@@ -96,3 +96,48 @@ def test_surface_samples_equal_the_oracle_and_the_mesh_bucket_runs(orc):
     u = sc["lr_vel"][n_g:, :3]
     np.testing.assert_allclose(x1[n_g:, :3] - x0[n_g:, :3], 4 / 60.0 * u, atol=1e-5)
     ctx.close()
+
+
+def _near_surface(V, T, rng, n):
+    """Candidates at 1e-2 .. 1e-10 of the mesh's size from its faces, edges and vertices, and some far away."""
+    size = float((V.max(0) - V.min(0)).max())
+    t = rng.integers(0, len(T), n)
+    bary = rng.dirichlet((1.0, 1.0, 1.0), n)
+    bary[: n // 3, 2] = 0.0                     # on an edge
+    bary[: n // 9] = (1.0, 0.0, 0.0)            # on a vertex
+    bary /= bary.sum(1, keepdims=True)
+    p = (V[T[t]] * bary[:, :, None]).sum(1)
+    d = rng.normal(size=(n, 3))
+    d *= size * 10.0 ** rng.uniform(-10, -2, (n, 1)) / np.linalg.norm(d, axis=1, keepdims=True)
+    far = V.mean(0) + size * rng.uniform(-50.0, 50.0, (16, 3))
+    return np.concatenate([p + d, far])
+
+
+@pytest.mark.parametrize("scale, shift", [(1.0, 0.0), (1e-12, 0.0), (1e9, 0.0), (1.0, 1e3)])
+@pytest.mark.parametrize("mesh", ["castle", "sphere", "open_box"])
+def test_inside_decisions_near_the_surface_equal_the_oracle(orc, mesh, scale, shift):
+    # the single-precision evaluation may decide only what double precision
+    # decides too: equality, no tolerance (offsets stay far above the double
+    # evaluation's own rounding, also after a shift by 1e3)
+    rng = np.random.default_rng(31)
+    if mesh == "castle":
+        V, T = scenes.castle_mesh()
+    elif mesh == "sphere":
+        V, T = scenes.icosphere((0.1, 0.2, 0.3), 0.15, 3)     # 1280 triangles: several staging rounds, a remainder
+        T = T[: len(T) - 77]                                   # and not closed
+    else:
+        V, T = scenes.box_mesh((0, 0, 0), (1, 0.5, 0.25))
+        T = T[2:]
+    V = V * scale + shift
+    cand = _near_surface(V, T, rng, 20000)
+    if shift:
+        cand = cand[: 20000][np.linalg.norm(cand[: 20000] - shift, axis=1) > 0]
+    import paper_2308_01629_gb300 as gs
+    orc.set_threads(orc.max_threads())
+    r = 0.02 * float((V.max(0) - V.min(0)).max())
+    rc, sel, inside = gs.gs_sample_volume(V, T, cand, r)
+    ref_sel, ref_inside = orc.sample_volume(V, T, cand, r)
+    orc.set_threads(1)
+    assert rc == gs.GS_OK
+    np.testing.assert_array_equal(inside, ref_inside)
+    np.testing.assert_array_equal(sel, ref_sel)
