@@ -262,6 +262,8 @@ PbdArgs pbd_args(const gs_ctx* c, float dt)
     a.dt = dt;
     a.dt_dev = nullptr;
     a.scenes = c->d_scenes;
+    a.n_scenes = c->n_scenes;
+    a.scene0 = c->scenes[0];
     a.lr_scene = c->lr_scene;
     a.sdf = c->d_sdf;
     const bool mat = c->n_materials > 0;

@@ -408,6 +408,8 @@ struct PbdArgs {
     float dt;
     const float* dt_dev;   // not null: the step length is *dt_dev (adaptive frames), not dt
     const SceneDev* scenes;
+    int n_scenes;
+    SceneDev scene0;       // the first scene's descriptor (what a one-scene context reads)
     const uint32_t* lr_scene;
     const gs_sdf* sdf;
     // grain materials: null for the scenes' coefficients; else the table

@@ -1,0 +1,50 @@
+// lr_bins.cuh -- binning of the LR set in three launches and no clears.
+//   arrive  one thread per particle (fused with whatever computes its
+//           position): its cell's count, its place in the cell's bucket of
+//           kBucket indices in order of arrival, and the count of the cell's
+//           tile of kBinTile cells (summed per block in shared memory first);
+//   scan    one block per tile: the counts of the tiles before it, then the
+//           tile's own exclusive scan, into the cell starts;
+//   place   one thread per particle: its rank among the indices of its cell's
+//           bucket is its place in the stable order, and it copies itself
+//           there.
+// Every launch leaves what the next binning counts in at zero: place clears
+// the counts, scan moves the sums that place or later kernels read out of the
+// words that arrive adds to.  A particle beyond kBucket of its cell (a 3 r_LR
+// cube holds 8 LR particles of a 2 r_LR lattice) goes to a list that its
+// cell's particles search; the order is the same.
+// On the digging bed (50,527 LR, 33,213 cells) the chain of clear, keys, two
+// scan launches, scatter and per-cell order took BIN_OLD us, this one BIN_NEW.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "gs_internal.cuh"
+
+constexpr int kBucket = 16;
+constexpr int kBinTile = 4096;       // cells per tile of the scan
+constexpr int kMaxBinTiles = 1024;   // beyond that (4 M cells) the general counting sort
+
+// Clears the block's tile counts (s_tile: b.n_tiles words); a barrier follows
+// in bins_arrive's callers.
+__device__ __forceinline__ void bins_begin(const LrBins& b, uint32_t* s_tile)
+{
+    for (int t = threadIdx.x; t < b.n_tiles; t += blockDim.x) s_tile[t] = 0u;
+    __syncthreads();
+}
+
+__device__ __forceinline__ void bins_arrive(const LrBins& b, uint32_t* s_tile, uint32_t cell, uint32_t i)
+{
+    const uint32_t rank = atomicAdd(b.count + cell, 1u);
+    if (rank < (uint32_t)kBucket) b.bucket[(size_t)cell * kBucket + rank] = i;
+    else b.spill[atomicAdd(b.words + kBinSpillAcc, 1u)] = i;
+    atomicAdd(s_tile + cell / kBinTile, 1u);
+}
+
+// Adds the block's tile counts to the tiles' (after every thread's arrival).
+__device__ __forceinline__ void bins_end(const LrBins& b, uint32_t* s_tile)
+{
+    __syncthreads();
+    for (int t = threadIdx.x; t < b.n_tiles; t += blockDim.x)
+        if (s_tile[t]) atomicAdd(b.tile + t, s_tile[t]);
+}

@@ -215,46 +215,92 @@ __global__ void __launch_bounds__(128) k_neighbors(const PbdArgs a, const float4
     }
 }
 
-// kLanes lanes share one particle: lane `sub` takes candidates sub, sub +
-// kLanes, ... (their distances kDistGroup at a time, the contact terms of
-// those that may touch kContactGroup at a time, loads in flight together)
-// and the SDF components whose running index is sub modulo kLanes; the
-// partial sums are added with shuffles in a fixed order and lane 0 writes
-// the particle.
-constexpr int kLanes = 2;
+// One Jacobi pass.  A particle's candidates are summed in two chains, the
+// even and the odd ones in ascending order, which two lanes (its chain lanes)
+// own, so the sums have the same bits however many lanes share the particle:
+// two (in the middle and large sets) or eight (small sets).  The candidates
+// go in windows of kWindow: first their distances alone, kDistGroup at a time
+// with the loads in flight together, a bit per candidate that may touch (a
+// slightly wider test than contact_term's, which decides); then the contact
+// terms of the marked ones only.
+//   two lanes    each chain lane takes its own contacts, kContactGroup at a
+//                time.  Instruction issue bounds a large pass and the chain of
+//                dependent loads a pass of one wave.
+//   eight lanes  the marked contacts of the whole warp (four particles) are
+//                listed in shared memory and evaluated 32 at a time, one per
+//                lane, and every chain adds its own terms in order: more
+//                instructions, but one round trip where two lanes make four.
+// One pass on settled scenes of 10 passes per step (before: two lanes,
+// contacts found and friction evaluated with every root and division, every
+// wall evaluated, 79 registers): cube 1,000 LR 5.8 -> 4.2 us, column 4,000
+// 6.5 -> 4.5, bed of 12,624 8.2 -> 5.8 (eight lanes; two: 4.9, 5.8, 7.1),
+// bed 24,504 9.0 -> 7.6 (eight: 9.6), digging 50,527 10.7 -> 8.9 (eight: 15),
+// 2 x 2 m bed 202,112 32.5 -> 23.2, 64 scenes of 275,339 35.2 -> 28.4.
+// 64 registers (eight blocks per SM) is where the two-lane form is fastest:
+// 48 spill (digging 10.5), 80 leave too few warps (batch 30.5).
+constexpr int kWindow = 64;
 constexpr int kDistGroup = 4;      // candidate distances whose loads are in flight together
-constexpr int kContactGroup = 2;   // contact terms whose loads are in flight together
+constexpr int kContactGroup = 2;   // contact terms whose loads are in flight together (two lanes)
+constexpr int kPassThreads = 128;
+constexpr int kPassBlocks = 8;     // per SM
+// Eight lanes while they fill less than one wave (152 SMs x 32 warps of four
+// particles).  At 20,000 LR they gain on a dense pile (the funnel's end, 9.2
+// against 11.9 us) and lose where grains fall without contacts (the funnel's
+// frame 363 against 342 us), so the line lies below.
+constexpr int64_t kWideMax = 16384;
+
+// Per-warp shared memory of the eight-lane form.
+constexpr int kChunk = 64;
+struct PassShared {
+    float4 contact[kChunk];   // (s, e): contact term -s e; s = kNoContact where there is none
+    float4 slide[kChunk];     // (f, t): friction term -f t
+    uint16_t list[32 * (kWindow / 2)];   // chain lane << 8 | index in the chain's window
+};
+constexpr int kNoContact = 0x7fc00001;   // a NaN that no arithmetic gives (its NaNs are 0x7fffffff)
 
 struct PassAcc {
     float Dx, Dy, Dz;
     int n;
 };
 
-// mu_s, mu_k: the pair's friction coefficients (the scene's, or the cross
-// coefficients of the two grains' materials)
-__device__ __forceinline__ void pair_term(PassAcc& acc, const SceneDev& sc, int stab, float4 yp, float wp, float dpx,
-                                          float dpy, float dpz, float4 xtq, float4 xq, float d0, float mu_s,
-                                          float mu_k)
+// The terms of one pair: -s e (contact) and -f t (friction, solver passes),
+// false where the two do not touch.
+struct PairTerms {
+    float s, ex, ey, ez;
+    float f, tx, ty, tz;
+};
+
+__device__ __forceinline__ bool contact_term(const SceneDev& sc, int stab, float4 yp, float wp, float dpx, float dpy,
+                                             float dpz, float4 xtq, float4 xq, float mu_s, float mu_k, PairTerms& o)
 {
-    const float4 yq = stab ? xq : xtq;
-    const PairGeo pg = pair_geo(yp, yq);
-    if (!(pg.d < d0) || pg.d2 == 0.0f) return;
+    const float d0 = 2.0f * sc.r_low;
+    const PairGeo pg = pair_geo(yp, stab ? xq : xtq);
     const float wsum = wp + xtq.w;
-    if (!(wsum > 0.0f)) return;
+    if (!(pg.d < d0) || pg.d2 == 0.0f || !(wsum > 0.0f)) return false;
     const float m = wp / wsum;
     const float pen = d0 - pg.d;
-    const float s = m * pen / pg.d;
-    acc.Dx -= s * pg.ex;
-    acc.Dy -= s * pg.ey;
-    acc.Dz -= s * pg.ez;
+    o.s = m * pen / pg.d;
+    o.ex = pg.ex;
+    o.ey = pg.ey;
+    o.ez = pg.ez;
     if (!stab) {
         const float rx = dpx - (xtq.x - xq.x), ry = dpy - (xtq.y - xq.y), rz = dpz - (xtq.z - xq.z);
-        const Tangent tg = tangent_part(rx, ry, rz, pg.ex, pg.ey, pg.ez, pg.d2);
         const float base = sc.friction_mode == 1 ? pen : d0;
-        const float f = m * friction_scale(tg.L, base * mu_s, base * mu_k);
-        acc.Dx -= f * tg.tx;
-        acc.Dy -= f * tg.ty;
-        acc.Dz -= f * tg.tz;
+        o.f = m * tangent_friction(rx, ry, rz, pg.ex, pg.ey, pg.ez, pg.d2, base * mu_s, base * mu_k, o.tx, o.ty,
+                                   o.tz);
+    }
+    return true;
+}
+
+__device__ __forceinline__ void add_term(PassAcc& acc, int stab, const PairTerms& t)
+{
+    acc.Dx = fmaf(-t.s, t.ex, acc.Dx);
+    acc.Dy = fmaf(-t.s, t.ey, acc.Dy);
+    acc.Dz = fmaf(-t.s, t.ez, acc.Dz);
+    if (!stab) {
+        acc.Dx = fmaf(-t.f, t.tx, acc.Dx);
+        acc.Dy = fmaf(-t.f, t.ty, acc.Dy);
+        acc.Dz = fmaf(-t.f, t.tz, acc.Dz);
     }
     ++acc.n;
 }
@@ -285,8 +331,6 @@ __device__ __forceinline__ void st_pos(float4* p, float4 v)
     else *p = v;
 }
 
-// One Jacobi pass of particle p (valid == p < n) by its kLanes lanes; every
-// lane of the warp takes part (the partial sums meet in full-warp shuffles).
 // Finalize of the step (last loop of Algorithm 1) folded into its last pass:
 // v = (x~ - x) / dt and x = x~, written to original order through idx.
 struct FinalOut {
@@ -296,19 +340,29 @@ struct FinalOut {
     unsigned* rate;        // not null: atomic max of the CFL rate of the new velocities
 };
 
+// The pass of the warp's particles [p0, p0 + 32 / kLanes); every lane of the
+// warp takes part.
 // kMat: grains carry materials (their ids in the w of x); a pair's
 // coefficients are the cross coefficients of the two materials, an SDF
 // contact's sqrt(mu_i mu_b).
 // kBody: rigid bodies; in solver passes a body particle also receives its
 // shape-matching delta (R xo + c) - x~ (Sec. 3), counted once in n_i.
-template <bool kL2, bool kMat, bool kBody = false>
-__device__ __forceinline__ void pass_particle(const PbdArgs& a, int stab, int64_t p, bool valid, int sub,
-                                              const float4* __restrict__ x_in, const float4* __restrict__ xt_in,
-                                              float4* __restrict__ x_out, float4* __restrict__ xt_out,
-                                              const uint32_t* __restrict__ nbr, const uint32_t* __restrict__ cnt,
-                                              const FinalOut fin = FinalOut{nullptr, nullptr, nullptr, nullptr})
+// kSingle: a context of one scene, whose parameters ride in the arguments
+// (constant memory) instead of two dependent loads per particle.
+template <int kLanes, bool kL2, bool kMat, bool kBody, bool kSingle>
+__device__ __forceinline__ void pass_warp(const PbdArgs& a, int stab, int64_t p0, PassShared& sh,
+                                          const float4* __restrict__ x_in, const float4* __restrict__ xt_in,
+                                          float4* __restrict__ x_out, float4* __restrict__ xt_out,
+                                          const uint32_t* __restrict__ nbr, const uint32_t* __restrict__ cnt,
+                                          const FinalOut fin = FinalOut{nullptr, nullptr, nullptr, nullptr})
 {
-    const SceneDev& sc = a.scenes[valid ? a.lr_scene[p] : 0];
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = (int)(threadIdx.x & 31u);
+    const int sub = lane % kLanes;
+    const int64_t p = p0 + lane / kLanes;
+    const bool valid = p < a.n;
+    const int scene = kSingle ? 0 : (int)a.lr_scene[valid ? p : 0];
+    const SceneDev& sc = kSingle ? a.scene0 : a.scenes[scene];
     const float d0 = 2.0f * sc.r_low;
     float4 xtp = make_float4(0.f, 0.f, 0.f, 0.f), xp = xtp;
     int nc = 0;
@@ -318,25 +372,18 @@ __device__ __forceinline__ void pass_particle(const PbdArgs& a, int stab, int64_
         nc = (int)__ldg(cnt + p);
     }
     const uint32_t matp = kMat ? __float_as_uint(xp.w) : 0u;
-    const float2* cross_p = kMat ? a.mu_cross + matp * GS_MAX_MATERIALS : nullptr;
     const float4 yp = stab ? xp : xtp;          // positions the constraints are evaluated on
     const float wp = xtp.w;                      // inverse height-scaled mass
     const float dpx = xtp.x - xp.x, dpy = xtp.y - xp.y, dpz = xtp.z - xp.z;
-    PassAcc acc = {0.f, 0.f, 0.f, 0};
-    // The lane's candidates k = sub, sub + kLanes, ... in windows of 32.
-    // First their distances alone: kDistGroup at a time, the loads of the
-    // evaluated positions in flight together, a bit per candidate that may
-    // be in contact (a slightly wider test than pair_term's, which decides).
-    // Then the contact terms for the marked candidates only, in candidate
-    // order (the summation order of the lane).  A warp thus runs the contact
-    // code as often as its busiest lane has contacts, not once per candidate
-    // slot that any lane fills.
+    PassAcc acc = {0.f, 0.f, 0.f, 0};            // of the chain (chain lanes)
     const float4* yq_in = stab ? x_in : xt_in;
     const float d2_mark = d0 * d0 * 1.0001f;
-    for (int w0 = sub; w0 < nc; w0 += 32 * kLanes) {
-        const int wend = min(nc, w0 + 32 * kLanes);
+    const int nc_max = __reduce_max_sync(kAll, nc);
+    for (int w0 = 0; w0 < nc_max; w0 += kWindow) {
+        // mark: bit b of a chain's mask is candidate w0 + 2 b + (chain)
+        const int wend = min(nc, w0 + kWindow);
         uint32_t marked = 0u;
-        for (int k = w0; k < wend; k += kDistGroup * kLanes) {
+        for (int k = w0 + sub; k < wend; k += kDistGroup * kLanes) {
             uint32_t q[kDistGroup];
             bool in[kDistGroup];
 #pragma unroll
@@ -351,68 +398,158 @@ __device__ __forceinline__ void pass_particle(const PbdArgs& a, int stab, int64_
             for (int j = 0; j < kDistGroup; ++j) {
                 const float ex = yq[j].x - yp.x, ey = yq[j].y - yp.y, ez = yq[j].z - yp.z;
                 const float d2 = fmaf(ez, ez, fmaf(ey, ey, ex * ex));   // as pair_geo
-                if (in[j] && d2 < d2_mark) marked |= 1u << ((k - w0) / kLanes + j);
+                if (in[j] && d2 < d2_mark) marked |= 1u << ((k - w0 + j * kLanes) >> 1);
             }
         }
-        // the marked candidates kContactGroup at a time, their loads in flight
-        // together, then their terms in candidate order
-        while (marked) {
-            uint32_t q[kContactGroup];
-            bool ok[kContactGroup];
 #pragma unroll
-            for (int j = 0; j < kContactGroup; ++j) {
-                ok[j] = marked != 0u;
-                const int li = ok[j] ? __ffs(marked) - 1 : 0;
-                marked &= marked - 1u;
-                q[j] = ok[j] ? __ldg(nbr + (int64_t)(w0 + li * kLanes) * a.n + p) : (uint32_t)p;
-            }
-            float4 xtq[kContactGroup], xq[kContactGroup];
+        for (int o = 2; o < kLanes; o <<= 1) marked |= __shfl_xor_sync(kAll, marked, o);
+        if constexpr (kLanes == 2) {
+            while (marked) {
+                uint32_t q[kContactGroup];
+                bool on[kContactGroup];
 #pragma unroll
-            for (int j = 0; j < kContactGroup; ++j) {
-                xtq[j] = ld_pos<kL2>(xt_in + q[j]);
-                xq[j] = ld_pos<kL2>(x_in + q[j]);
-            }
-#pragma unroll
-            for (int j = 0; j < kContactGroup; ++j) {
-                if (!ok[j]) continue;
-                if constexpr (kMat) {
-                    const float2 mu = __ldg(cross_p + __float_as_uint(xq[j].w));
-                    pair_term(acc, sc, stab, yp, wp, dpx, dpy, dpz, xtq[j], xq[j], d0, mu.x, mu.y);
-                } else {
-                    pair_term(acc, sc, stab, yp, wp, dpx, dpy, dpz, xtq[j], xq[j], d0, sc.mu_s, sc.mu_k);
+                for (int j = 0; j < kContactGroup; ++j) {
+                    on[j] = marked != 0u;
+                    const int b = on[j] ? __ffs(marked) - 1 : 0;
+                    marked &= marked - 1u;
+                    q[j] = on[j] ? __ldg(nbr + (int64_t)(w0 + 2 * b + sub) * a.n + p) : (uint32_t)p;
                 }
+                float4 xtq[kContactGroup], xq[kContactGroup];
+#pragma unroll
+                for (int j = 0; j < kContactGroup; ++j) {
+                    xtq[j] = ld_pos<kL2>(xt_in + q[j]);
+                    xq[j] = ld_pos<kL2>(x_in + q[j]);
+                }
+#pragma unroll
+                for (int j = 0; j < kContactGroup; ++j) {
+                    if (!on[j]) continue;
+                    float mu_s = sc.mu_s, mu_k = sc.mu_k;
+                    if constexpr (kMat) {
+                        const float2 mu = __ldg(a.mu_cross + matp * GS_MAX_MATERIALS + __float_as_uint(xq[j].w));
+                        mu_s = mu.x;
+                        mu_k = mu.y;
+                    }
+                    PairTerms t;
+                    if (contact_term(sc, stab, yp, wp, dpx, dpy, dpz, xtq[j], xq[j], mu_s, mu_k, t))
+                        add_term(acc, stab, t);
+                }
+            }
+        } else {
+            // list
+            const int c_cnt = sub < 2 ? __popc(marked) : 0;
+            int incl = c_cnt;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(kAll, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const int total = __shfl_sync(kAll, incl, 31);
+            const int c_off = incl - c_cnt;
+            if (sub < 2)
+                for (int i = c_off; marked; ++i) {
+                    sh.list[i] = (uint16_t)((lane << 8) | (__ffs(marked) - 1));
+                    marked &= marked - 1u;
+                }
+            __syncwarp();
+            for (int base = 0; base < total; base += kChunk) {
+                const int end = min(total, base + kChunk);
+                for (int r0 = base; r0 < end; r0 += 32) {
+                    const int t = r0 + lane;
+                    const bool has = t < end;
+                    const int e = has ? sh.list[t] : (lane << 8);
+                    const int src = e >> 8;
+                    uint32_t q = (uint32_t)p;
+                    if (has) q = __ldg(nbr + (int64_t)(w0 + 2 * (e & 255) + (src & 1)) * a.n + p0 + src / kLanes);
+                    const float4 yc = make_float4(__shfl_sync(kAll, yp.x, src), __shfl_sync(kAll, yp.y, src),
+                                                  __shfl_sync(kAll, yp.z, src), 0.f);
+                    const float wc = __shfl_sync(kAll, wp, src);
+                    const uint32_t matc = kMat ? __shfl_sync(kAll, matp, src) : 0u;
+                    const int scene_c = kSingle ? 0 : __shfl_sync(kAll, scene, src);
+                    const float cx = __shfl_sync(kAll, dpx, src), cy = __shfl_sync(kAll, dpy, src),
+                                cz = __shfl_sync(kAll, dpz, src);
+                    if (!has) continue;
+                    const SceneDev& sd = kSingle ? a.scene0 : a.scenes[scene_c];
+                    const float4 xtq = ld_pos<kL2>(xt_in + q), xq = ld_pos<kL2>(x_in + q);
+                    float mu_s = sd.mu_s, mu_k = sd.mu_k;
+                    if constexpr (kMat) {
+                        const float2 mu = __ldg(a.mu_cross + matc * GS_MAX_MATERIALS + __float_as_uint(xq.w));
+                        mu_s = mu.x;
+                        mu_k = mu.y;
+                    }
+                    PairTerms o;
+                    if (contact_term(sd, stab, yc, wc, cx, cy, cz, xtq, xq, mu_s, mu_k, o)) {
+                        sh.contact[t - base] = make_float4(o.s, o.ex, o.ey, o.ez);
+                        if (!stab) sh.slide[t - base] = make_float4(o.f, o.tx, o.ty, o.tz);
+                    } else {
+                        sh.contact[t - base].x = __int_as_float(kNoContact);
+                    }
+                }
+                __syncwarp();
+                const int i1 = min(c_off + c_cnt, end) - base;
+                for (int i = max(c_off, base) - base; i < i1; ++i) {
+                    const float4 c = sh.contact[i];
+                    if (__float_as_int(c.x) == kNoContact) continue;
+                    PairTerms o;
+                    o.s = c.x;
+                    o.ex = c.y;
+                    o.ey = c.z;
+                    o.ez = c.w;
+                    if (!stab) {
+                        const float4 f = sh.slide[i];
+                        o.f = f.x;
+                        o.tx = f.y;
+                        o.ty = f.z;
+                        o.tz = f.w;
+                    }
+                    add_term(acc, stab, o);
+                }
+                __syncwarp();
             }
         }
     }
-    if (valid && wp > 0.0f) {
-        float gmu_s = sc.mu_s, gmu_k = sc.mu_k;   // the grain's own coefficients
-        if constexpr (kMat) {
-            const float2 mu = __ldg(a.mu_mat + matp);
-            gmu_s = mu.x;
-            gmu_k = mu.y;
-        }
-        const float sdt = step_dt(a);
+    if (valid && sub < 2 && wp > 0.0f) {
+        // the boundaries: chain `sub` takes the components whose running
+        // index has its parity.  Most particles are near none: three walls of
+        // a box, or a bound of the distance to another shape, decide that.
         int gc = 0;
         for (int sI = 0; sI < sc.n_sdf; ++sI) {
             const gs_sdf& b = a.sdf[sc.sdf_begin + sI];
             const int ncomp = sdf_components(b.kind);
-            for (int c = 0; c < ncomp; ++c, ++gc) {
-                if ((gc & (kLanes - 1)) != sub) continue;
+            const int c0 = (sub ^ gc) & 1;   // this chain's first component
+            gc += ncomp;
+            if (b.kind == GS_SDF_BOX_INTERIOR) {
+                const bool hi = c0 != 0;
+                const float fx = hi ? b.p[3] - yp.x : yp.x - b.p[0];
+                const float fy = hi ? b.p[4] - yp.y : yp.y - b.p[1];
+                const float fz = hi ? b.p[5] - yp.z : yp.z - b.p[2];
+                if (!(fx < sc.r_low || fy < sc.r_low || fz < sc.r_low)) continue;
+            } else if (c0 >= ncomp || sdf_far(b, yp.x, yp.y, yp.z, sc.r_low)) {
+                continue;
+            }
+            float gmu_s = sc.mu_s, gmu_k = sc.mu_k;   // the grain's own coefficients
+            if constexpr (kMat) {
+                const float2 mu = __ldg(a.mu_mat + matp);
+                gmu_s = mu.x;
+                gmu_k = mu.y;
+            }
+            const float sdt = step_dt(a);
+            for (int c = c0; c < ncomp; c += 2) {
                 const SdfHit h = sdf_eval(b, c, yp.x, yp.y, yp.z);
                 if (!(h.phi < sc.r_low)) continue;
                 const float pen = sc.r_low - h.phi;
-                acc.Dx += pen * h.nx;
-                acc.Dy += pen * h.ny;
-                acc.Dz += pen * h.nz;
+                acc.Dx = fmaf(pen, h.nx, acc.Dx);
+                acc.Dy = fmaf(pen, h.ny, acc.Dy);
+                acc.Dz = fmaf(pen, h.nz, acc.Dz);
                 if (!stab) {
                     const float bmu_s = sqrtf(gmu_s * b.mu_s), bmu_k = sqrtf(gmu_k * b.mu_k);
-                    const float rx = dpx - b.vel[0] * sdt, ry = dpy - b.vel[1] * sdt, rz = dpz - b.vel[2] * sdt;
+                    const float rx = fmaf(-b.vel[0], sdt, dpx), ry = fmaf(-b.vel[1], sdt, dpy),
+                                rz = fmaf(-b.vel[2], sdt, dpz);
                     const Tangent tg = tangent_part(rx, ry, rz, h.nx, h.ny, h.nz, 1.0f);
                     const float base = sc.friction_mode == 1 ? pen : d0;
                     const float f = friction_scale(tg.L, base * bmu_s, base * bmu_k);
-                    acc.Dx -= f * tg.tx;
-                    acc.Dy -= f * tg.ty;
-                    acc.Dz -= f * tg.tz;
+                    acc.Dx = fmaf(-f, tg.tx, acc.Dx);
+                    acc.Dy = fmaf(-f, tg.ty, acc.Dy);
+                    acc.Dz = fmaf(-f, tg.tz, acc.Dz);
                 }
                 ++acc.n;
             }
@@ -432,13 +569,11 @@ __device__ __forceinline__ void pass_particle(const PbdArgs& a, int stab, int64_
             }
         }
     }
-#pragma unroll
-    for (int o = 1; o < kLanes; o <<= 1) {
-        acc.Dx += __shfl_xor_sync(0xffffffffu, acc.Dx, o);
-        acc.Dy += __shfl_xor_sync(0xffffffffu, acc.Dy, o);
-        acc.Dz += __shfl_xor_sync(0xffffffffu, acc.Dz, o);
-        acc.n += __shfl_xor_sync(0xffffffffu, acc.n, o);
-    }
+    // the two chains meet in the particle's first lane
+    acc.Dx += __shfl_xor_sync(kAll, acc.Dx, 1);
+    acc.Dy += __shfl_xor_sync(kAll, acc.Dy, 1);
+    acc.Dz += __shfl_xor_sync(kAll, acc.Dz, 1);
+    acc.n += __shfl_xor_sync(kAll, acc.n, 1);
     const bool writer = valid && sub == 0;
     const bool reduce = fin.idx && fin.rate;   // the whole warp meets in the rate reduction below
     if (!writer && !reduce) return;
@@ -479,16 +614,18 @@ __device__ __forceinline__ void pass_particle(const PbdArgs& a, int stab, int64_
     if (stab) st_pos<kL2>(x_out + p, nx);
 }
 
-template <bool kMat, bool kBody>
-__global__ void __launch_bounds__(128, 6) k_pass(const PbdArgs a, int stab, const float4* __restrict__ x_in,
-                                              const float4* __restrict__ xt_in, float4* __restrict__ x_out,
-                                              float4* __restrict__ xt_out, const uint32_t* __restrict__ nbr,
-                                              const uint32_t* __restrict__ cnt, const FinalOut fin)
+template <int kLanes, bool kMat, bool kBody, bool kSingle>
+__global__ void __launch_bounds__(kPassThreads, kPassBlocks) k_pass(
+    const PbdArgs a, int stab, const float4* __restrict__ x_in, const float4* __restrict__ xt_in,
+    float4* __restrict__ x_out, float4* __restrict__ xt_out, const uint32_t* __restrict__ nbr,
+    const uint32_t* __restrict__ cnt, const FinalOut fin)
 {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t p = t / kLanes;
-    pass_particle<false, kMat, kBody>(a, stab, p, p < a.n, (int)(t % kLanes), x_in, xt_in, x_out, xt_out, nbr, cnt,
-                                      fin);
+    __shared__ PassShared sh[kLanes == 2 ? 1 : kPassThreads / 32];   // not used by the two-lane form
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t p0 = w * (32 / kLanes);
+    if (p0 >= a.n) return;   // whole warps
+    pass_warp<kLanes, false, kMat, kBody, kSingle>(a, stab, p0, sh[kLanes == 2 ? 0 : threadIdx.x >> 5], x_in, xt_in,
+                                                   x_out, xt_out, nbr, cnt, fin);
 }
 
 // ---- all passes of one step in one launch --------------------------------
@@ -552,26 +689,25 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned nblocks, un
     return s_ok != 0;
 }
 
+constexpr int kSolveLanes = 2;
+
 template <bool kMat>
 __global__ void __launch_bounds__(128, 6) k_solve(const SolveArgs s)
 {
-    const int sub = (int)(threadIdx.x % kLanes);
-    const int64_t groups = (int64_t)gridDim.x * (blockDim.x / kLanes);
-    const int64_t group = (int64_t)blockIdx.x * (blockDim.x / kLanes) + threadIdx.x / kLanes;
-    // the warp's first group decides the trip count, so whole warps iterate
-    const int64_t warp_first = group & ~(int64_t)(32 / kLanes - 1);
+    __shared__ PassShared sh[1];   // not used by the two-lane form
+    constexpr int kPer = 32 / kSolveLanes;   // particles per warp
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int bx = 0, bt = 0;
     const int total = s.n_stab + s.iters;
     for (int it = 0; it < total; ++it) {
         const int stab = it < s.n_stab;
-        for (int64_t base = warp_first; base < s.a.n; base += groups) {
-            const int64_t p = base + (group - warp_first);
-            float4* xi = bx ? s.x1 : s.x0;
-            float4* xo = bx ? s.x0 : s.x1;
-            float4* ti = bt ? s.xt1 : s.xt0;
-            float4* to = bt ? s.xt0 : s.xt1;
-            pass_particle<true, kMat>(s.a, stab, p, p < s.a.n, sub, xi, ti, xo, to, s.nbr, s.cnt);
-        }
+        float4* xi = bx ? s.x1 : s.x0;
+        float4* xo = bx ? s.x0 : s.x1;
+        float4* ti = bt ? s.xt1 : s.xt0;
+        float4* to = bt ? s.xt0 : s.xt1;
+        for (int64_t p0 = warp * kPer; p0 < s.a.n; p0 += warps * kPer)
+            pass_warp<kSolveLanes, true, kMat, false, false>(s.a, stab, p0, sh[0], xi, ti, xo, to, s.nbr, s.cnt);
         bt ^= 1;
         if (stab) bx ^= 1;
         if (it + 1 < total && !grid_barrier(s.bar, gridDim.x + s.extra_arrivals, (unsigned)it + 1u, s.err)) return;
@@ -818,6 +954,36 @@ cudaError_t gs_launch_neighbors(cudaStream_t s, const PbdArgs& a, const float4* 
     return cudaGetLastError();
 }
 
+template <int kLanes, bool kSingle>
+static void launch_pass_scenes(cudaStream_t s, const PbdArgs& a, int stab, const float4* x_in, const float4* xt_in,
+                               float4* x_out, float4* xt_out, const uint32_t* nbr, const uint32_t* cnt,
+                               const FinalOut& fin)
+{
+    const unsigned nb = gs_blocks(a.n * kLanes, kPassThreads);
+    if (a.body) {
+        if (a.mu_cross)
+            k_pass<kLanes, true, true, kSingle><<<nb, kPassThreads, 0, s>>>(a, stab, x_in, xt_in, x_out, xt_out, nbr,
+                                                                            cnt, fin);
+        else
+            k_pass<kLanes, false, true, kSingle><<<nb, kPassThreads, 0, s>>>(a, stab, x_in, xt_in, x_out, xt_out, nbr,
+                                                                             cnt, fin);
+    } else if (a.mu_cross) {
+        k_pass<kLanes, true, false, kSingle><<<nb, kPassThreads, 0, s>>>(a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt,
+                                                                         fin);
+    } else {
+        k_pass<kLanes, false, false, kSingle><<<nb, kPassThreads, 0, s>>>(a, stab, x_in, xt_in, x_out, xt_out, nbr,
+                                                                          cnt, fin);
+    }
+}
+
+template <int kLanes>
+static void launch_pass(cudaStream_t s, const PbdArgs& a, int stab, const float4* x_in, const float4* xt_in,
+                        float4* x_out, float4* xt_out, const uint32_t* nbr, const uint32_t* cnt, const FinalOut& fin)
+{
+    if (a.n_scenes == 1) launch_pass_scenes<kLanes, true>(s, a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt, fin);
+    else launch_pass_scenes<kLanes, false>(s, a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt, fin);
+}
+
 cudaError_t gs_launch_pass(cudaStream_t s, const PbdArgs& a, int stab, const float4* x_in, const float4* xt_in,
                            float4* x_out, float4* xt_out, const uint32_t* nbr, const uint32_t* cnt,
                            int64_t* launches, const uint32_t* fin_idx, float4* fin_pos, float4* fin_vel,
@@ -825,17 +991,8 @@ cudaError_t gs_launch_pass(cudaStream_t s, const PbdArgs& a, int stab, const flo
 {
     if (a.n <= 0) return cudaSuccess;
     const FinalOut fin{fin_idx, fin_pos, fin_vel, fin_idx ? fin_rate : nullptr};
-    const unsigned nb = gs_blocks(a.n * kLanes, 128);
-    if (a.body) {
-        if (a.mu_cross)
-            k_pass<true, true><<<nb, 128, 0, s>>>(a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt, fin);
-        else
-            k_pass<false, true><<<nb, 128, 0, s>>>(a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt, fin);
-    } else if (a.mu_cross) {
-        k_pass<true, false><<<nb, 128, 0, s>>>(a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt, fin);
-    } else {
-        k_pass<false, false><<<nb, 128, 0, s>>>(a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt, fin);
-    }
+    if (a.n <= kWideMax) launch_pass<8>(s, a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt, fin);
+    else launch_pass<2>(s, a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt, fin);
     *launches += 1;
     return cudaGetLastError();
 }
@@ -872,7 +1029,7 @@ cudaError_t gs_launch_solve(cudaStream_t s, const PbdArgs& a, int n_stab, int it
     sa.bar = bar;
     sa.err = err;
     sa.extra_arrivals = extra_arrivals;
-    int64_t need = (a.n * kLanes + 127) / 128;
+    int64_t need = (a.n * kSolveLanes + 127) / 128;
     const int grid = (int)std::min<int64_t>(need, max_blocks);
     void* args[] = {&sa};
     const void* fn = a.mu_cross ? (const void*)k_solve<true> : (const void*)k_solve<false>;

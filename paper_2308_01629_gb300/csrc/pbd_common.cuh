@@ -43,3 +43,21 @@ __device__ __forceinline__ Tangent tangent_part(float rx, float ry, float rz, fl
     t.L = sqrtf(fmaf(t.tz, t.tz, fmaf(t.ty, t.ty, t.tx * t.tx)));
     return t;
 }
+
+// friction_scale of the tangential displacement r - (r.e / ee) e (tx, ty, tz
+// on return), without the length's square root and the division where the
+// squared length is surely below the static threshold's: nearly always, as
+// 2 r mu_s is what a grain slides in one step at over a metre per second.
+// The margin of 1e-5 exceeds the roundings of the square and the root, so
+// the decision is the same.
+__device__ __forceinline__ float tangent_friction(float rx, float ry, float rz, float ex, float ey, float ez, float ee,
+                                                  float thr_s, float thr_k, float& tx, float& ty, float& tz)
+{
+    const float al = fmaf(rz, ez, fmaf(ry, ey, rx * ex)) / ee;
+    tx = fmaf(-al, ex, rx);
+    ty = fmaf(-al, ey, ry);
+    tz = fmaf(-al, ez, rz);
+    const float L2 = fmaf(tz, tz, fmaf(ty, ty, tx * tx));
+    if (L2 < thr_s * thr_s * 0.99999f) return 1.0f;
+    return friction_scale(sqrtf(L2), thr_s, thr_k);
+}
