@@ -244,17 +244,6 @@ cudaError_t launch_hr_load(gs_ctx* c, const float4* src, float4* dst, int set_id
     return cudaGetLastError();
 }
 
-int bin_low_at(gs_ctx* c, const float4* positions)
-{
-    const int64_t n = c->n_low;
-    CK(gs_count_sort_cells(c->stream, positions, n, c->d_scenes, c->lr_scene, c->n_cell_total, c->lr_keys[0],
-                           c->lr_vals[0], c->lr_keys[1], c->lr_vals[1], c->lr_cell_start, c->scan_aux, &c->launches),
-       "bin by cell");
-    c->lr_sorted_keys = c->lr_keys[1];
-    c->lr_sorted_idx = c->lr_vals[1];
-    return GS_OK;
-}
-
 PbdArgs pbd_args(const gs_ctx* c, float dt)
 {
     PbdArgs a;
@@ -448,6 +437,14 @@ int create_impl(int S, const gs_scene* scenes, const float* r_low, const float* 
     A(dalloc(&c->step_cell_start, cells + 1));
     A(dalloc(&c->d_sdf_pend, std::max<size_t>(c->sdf_host.size(), 1)));
     A(dalloc(&c->scan_aux, gs_scan_aux_words(cells + 1)));
+    c->bins.n_tiles = gs_bins_tiles(cells);
+    if (c->bins.n_tiles > 0) {
+        A(dalloc(&c->bins.count, gs_bins_count_words(cells)));
+        A(dalloc(&c->bins.bucket, gs_bins_bucket_words(cells)));
+        A(dalloc(&c->bins.tile, c->bins.n_tiles));
+        A(dalloc(&c->bins.spill, N));
+        A(dalloc(&c->bins.words, kBinWords));
+    }
     A(dalloc(&c->lr_spos, N));
     A(dalloc(&c->lr_svel, N));
     A(dalloc(&c->lr_xt, N));
@@ -516,6 +513,11 @@ int create_impl(int S, const gs_scene* scenes, const float* r_low, const float* 
     Z(cudaMemsetAsync(c->d_cfl, 0, sizeof(CflState), c->stream));
     Z(cudaMemsetAsync(c->tmp4, 0, std::max<int64_t>(std::max(NM, MR), 1) * sizeof(float4), c->stream));
     Z(cudaMemsetAsync(c->lr_cell_start, 0, (cells + 2) * sizeof(uint32_t), c->stream));
+    if (c->bins.count) {
+        Z(cudaMemsetAsync(c->bins.count, 0, gs_bins_count_words(cells) * sizeof(uint32_t), c->stream));
+        Z(cudaMemsetAsync(c->bins.tile, 0, c->bins.n_tiles * sizeof(uint32_t), c->stream));
+        Z(cudaMemsetAsync(c->bins.words, 0, kBinWords * sizeof(uint32_t), c->stream));
+    }
     if (z) Z(launch_hr_load(c, c->tmp4, c->hr_pos[0], 1));
     if (z) Z(launch_hr_load(c, c->tmp4, c->hr_vel[0], 0));
     if (z) Z(cudaStreamSynchronize(c->stream));
@@ -580,15 +582,26 @@ int bin_low_impl(gs_ctx* c)
     // of rigid bodies for the gather (the binning reads every position
     // anyway); body particles enter the gather's view with w = 0
     const uint32_t* body = c->n_bodies > 0 ? c->lr_body : nullptr;
-    CK(gs_cs_clear(c->stream, c->lr_cell_start, c->n_cell_total, 1), "clear counts");
-    CK(gs_cs_keys(c->stream, c->lr_pos, c->n_low, c->d_scenes, c->lr_scene, c->lr_keys[0], c->lr_vals[0],
-                  c->lr_cell_start, &c->launches, c->lr_cell_start + c->n_cell_total + 1, body),
-       "cell keys");
     CsExtras ex;
     ex.ga_solid = body;
-    CK(gs_cs_finish(c->stream, c->n_low, c->n_cell_total, c->lr_keys[0], c->lr_vals[0], c->lr_keys[1], c->lr_vals[1],
-                    c->lr_cell_start, c->scan_aux, c->lr_pos, c->lr_vel, c->lr_spos, c->lr_svel, &c->launches, ex),
-       "bin by cell");
+    unsigned* flag = c->lr_cell_start + c->n_cell_total + 1;
+    if (c->bins.count) {
+        CK(gs_bins_keys(c->stream, c->bins, c->lr_pos, c->n_low, c->d_scenes, c->lr_scene, c->lr_keys[0], &c->launches,
+                        1, body),
+           "cell keys");
+        CK(gs_bins_finish(c->stream, c->bins, c->n_low, c->n_cell_total, c->lr_keys[0], c->lr_keys[1], c->lr_vals[1],
+                          c->lr_cell_start, c->lr_pos, c->lr_vel, c->lr_spos, c->lr_svel, &c->launches, ex, flag),
+           "bin by cell");
+    } else {
+        CK(gs_cs_clear(c->stream, c->lr_cell_start, c->n_cell_total, 1), "clear counts");
+        CK(gs_cs_keys(c->stream, c->lr_pos, c->n_low, c->d_scenes, c->lr_scene, c->lr_keys[0], c->lr_vals[0],
+                      c->lr_cell_start, &c->launches, flag, body),
+           "cell keys");
+        CK(gs_cs_finish(c->stream, c->n_low, c->n_cell_total, c->lr_keys[0], c->lr_vals[0], c->lr_keys[1],
+                        c->lr_vals[1], c->lr_cell_start, c->scan_aux, c->lr_pos, c->lr_vel, c->lr_spos, c->lr_svel,
+                        &c->launches, ex),
+           "bin by cell");
+    }
     c->lr_sorted_keys = c->lr_keys[1];
     c->lr_sorted_idx = c->lr_vals[1];
     c->lr_binned = true;
@@ -661,6 +674,34 @@ int upsample_impl(gs_ctx* c, float dt)
     return GS_OK;
 }
 
+// The beginning of an LR step: prediction fused with the counting stage of
+// the binning of x~, the binning (whose last stage copies x and x~ into cell
+// order, X and XT; cell starts in `start`), and the candidate lists.
+int step_begin(gs_ctx* c, const PbdArgs& a, float4* X, float4* XT, uint32_t* start, uint32_t* nbr, uint32_t* cnt)
+{
+    const int64_t N = c->n_low;
+    if (c->bins.count) {
+        CK(gs_launch_predict_bins(c->stream, a, c->bins, c->lr_pos, c->lr_vel, c->lr_xt, c->lr_keys[0], &c->launches),
+           "predict");
+        CK(gs_bins_finish(c->stream, c->bins, N, c->n_cell_total, c->lr_keys[0], c->lr_keys[1], c->lr_vals[1], start,
+                          c->lr_xt, c->lr_pos, XT, X, &c->launches, step_extras(c, a)),
+           "bin by cell");
+    } else {
+        CK(gs_cs_clear(c->stream, start, c->n_cell_total), "clear counts");
+        CK(gs_launch_predict_keys(c->stream, a, c->lr_pos, c->lr_vel, c->lr_xt, c->lr_keys[0], c->lr_vals[0], start,
+                                  &c->launches),
+           "predict");
+        CK(gs_cs_finish(c->stream, N, c->n_cell_total, c->lr_keys[0], c->lr_vals[0], c->lr_keys[1], c->lr_vals[1],
+                        start, c->scan_aux, c->lr_xt, c->lr_pos, XT, X, &c->launches, step_extras(c, a)),
+           "bin by cell");
+    }
+    c->lr_sorted_keys = c->lr_keys[1];
+    c->lr_sorted_idx = c->lr_vals[1];
+    CK(gs_launch_neighbors(c->stream, a, XT, c->lr_sorted_keys, start, nbr, cnt, c->nbr_cap, c->d_err, &c->launches),
+       "neighbours");
+    return GS_OK;
+}
+
 // dt_dev (adaptive frames): the step length is read from device memory
 // instead of dt; rate: the finalize's atomic max of |v| / (2 r_LR).
 int step_low_impl(gs_ctx* c, float dt, int iters, const float* dt_dev = nullptr, unsigned* rate = nullptr)
@@ -670,21 +711,8 @@ int step_low_impl(gs_ctx* c, float dt, int iters, const float* dt_dev = nullptr,
     Timed t(c, GS_TIMER_STEP_LOW);
     PbdArgs a = pbd_args(c, dt);
     a.dt_dev = dt_dev;
-    // prediction fused with the counting stage of the binning of x~; the
-    // binning's last stage copies x~ and x into cell order
-    CK(gs_cs_clear(c->stream, c->step_cell_start, c->n_cell_total), "clear counts");
-    CK(gs_launch_predict_keys(c->stream, a, c->lr_pos, c->lr_vel, c->lr_xt, c->lr_keys[0], c->lr_vals[0],
-                              c->step_cell_start, &c->launches),
-       "predict");
-    CK(gs_cs_finish(c->stream, N, c->n_cell_total, c->lr_keys[0], c->lr_vals[0], c->lr_keys[1], c->lr_vals[1],
-                    c->step_cell_start, c->scan_aux, c->lr_xt, c->lr_pos, c->s_xt[0], c->s_x[0], &c->launches,
-                    step_extras(c, a)),
-       "bin by cell");
-    c->lr_sorted_keys = c->lr_keys[1];
-    c->lr_sorted_idx = c->lr_vals[1];
-    CK(gs_launch_neighbors(c->stream, a, c->s_xt[0], c->lr_sorted_keys, c->step_cell_start, c->n_cell_total, c->nbr, c->nbr_cnt,
-                           c->nbr_cap, c->d_err, &c->launches),
-       "neighbours");
+    int st = step_begin(c, a, c->s_x[0], c->s_xt[0], c->step_cell_start, c->nbr, c->nbr_cnt);
+    if (st) return st;
     int bx = 0, bt = 0;   // buffers holding the current x and xt
     if (c->use_solver && c->solve_blocks > 0 && c->n_bodies == 0) {
         // all passes in one cooperative launch; the buffers alternate as in
@@ -1165,7 +1193,8 @@ void gs_destroy(gs_ctx* c)
                     c->step_cell_start, c->d_sdf_pend, c->stage_in, c->lr_mat, c->d_mu, c->d_cfl, c->lr_body, c->lr_xo, c->body_members,
                     c->body_start, c->body_xf, c->lr_slot, c->hr_bin_start, c->hr_big, c->hr_scan_aux,
                     c->async_in[0], c->async_in[1], c->async_in[2], c->async_in[3],
-                    c->async_out[0], c->async_out[1], c->async_out[2], c->async_out[3], c->slab_stage};
+                    c->async_out[0], c->async_out[1], c->async_out[2], c->async_out[3], c->slab_stage,
+                    c->bins.count, c->bins.bucket, c->bins.tile, c->bins.spill, c->bins.words};
     for (void* b : bufs)
         if (b) cudaFree(b);
     free_tapes(c);
@@ -2538,13 +2567,8 @@ static int step_low_record_into(gs_ctx* c, float dt, int iters, float4* X, float
     int st = flag_solid(c, (const float*)c->lr_pos, N);
     if (st) return st;
     PbdArgs a = pbd_args(c, dt);
-    CK(gs_launch_predict(c->stream, a, c->lr_pos, c->lr_vel, c->lr_xt, &c->launches), "predict");
-    st = bin_low_at(c, c->lr_xt);
+    st = step_begin(c, a, X, XT, c->step_cell_start, nbr, cnt);
     if (st) return st;
-    CK(gs_launch_step_gather(c->stream, N, c->lr_sorted_idx, c->lr_xt, c->lr_pos, XT, X, &c->launches), "gather");
-    CK(gs_launch_neighbors(c->stream, a, XT, c->lr_sorted_keys, c->lr_cell_start, c->n_cell_total, nbr, cnt,
-                           c->nbr_cap, c->d_err, &c->launches),
-       "neighbours");
     for (int it = 0; it < total; ++it) {
         const int stab = it < c->n_stab;
         CK(gs_launch_pass(c->stream, a, stab, X + (size_t)std::min(it, c->n_stab) * N, XT + (size_t)it * N,

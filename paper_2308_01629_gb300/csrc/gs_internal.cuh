@@ -85,6 +85,17 @@ struct CflState {
     float log[GS_MAX_SUBSTEPS];      // the frame's step lengths
 };
 
+// Scratch of the LR binning (lr_bins.cuh); all counts zero between binnings.
+enum { kBinSpillAcc = 0, kBinSpill = 1, kBinSolidAcc = 2, kBinWords = 4 };
+struct LrBins {
+    uint32_t* count = nullptr;    // per cell, padded to whole tiles; null: the general counting sort
+    uint32_t* bucket = nullptr;   // [n_cell][kBucket] particles of a cell in order of arrival
+    uint32_t* tile = nullptr;     // [n_tiles] particles per tile of cells
+    uint32_t* spill = nullptr;    // [n] particles beyond their cell's bucket
+    uint32_t* words = nullptr;    // spilled so far, spilled (of this binning), flag of solid particles so far
+    int n_tiles = 0;
+};
+
 struct gs_ctx {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
@@ -133,6 +144,7 @@ struct gs_ctx {
     uint32_t* lr_cell_start = nullptr;            // n_cell_total + 1 (upsampling view)
     uint32_t* step_cell_start = nullptr;          // n_cell_total + 1 (binning of x~ in the LR step)
     uint32_t* scan_aux = nullptr;                 // tile sums of the cell-start scan
+    LrBins bins;                                  // counts, buckets and tile sums of the LR binning
     float4* lr_spos = nullptr;                    // cell-ordered LR position (upsampling view)
     float4* lr_svel = nullptr;                    // cell-ordered LR velocity
     bool lr_binned = false;
@@ -314,9 +326,8 @@ cudaError_t gs_launch_cell_keys(cudaStream_t s, const float4* pos, int64_t n, Gr
 // Stable counting sort of n items by the cell of their position (coarse
 // keys): out_keys / out_idx in ascending (cell, item) order and cell_start
 // (n_cell + 1 entries) the start of every cell.  aux holds
-// gs_scan_aux_words(n_cell + 1) words.
+// gs_scan_aux_words(n_cell + 1) words.  In stages:
 size_t gs_scan_aux_words(int64_t total);
-// The same sort in stages, so that the keys can come from a fused kernel:
 // clear the counts, count (keys + arrival ranks; gs_cs_keys or a kernel
 // that does the same with grid_cell_of), then scan + scatter + per-cell
 // order; finish also copies ga / gb (when not null) into cell order.
@@ -351,10 +362,20 @@ cudaError_t gs_cs_finish(cudaStream_t s, int64_t n, int64_t n_cell, const uint32
                          uint32_t* out_keys, uint32_t* out_idx, uint32_t* cell_start, uint32_t* aux, const float4* ga,
                          const float4* gb, float4* ga_out, float4* gb_out, int64_t* launches,
                          const CsExtras& ex = CsExtras{});
-cudaError_t gs_count_sort_cells(cudaStream_t s, const float4* pos, int64_t n, const SceneDev* scenes,
-                                const uint32_t* tag, int64_t n_cell, uint32_t* keys, uint32_t* rank,
-                                uint32_t* out_keys, uint32_t* out_idx, uint32_t* cell_start, uint32_t* aux,
-                                int64_t* launches);
+// The LR binning by buckets (lr_bins.cuh): arrivals of given positions (the
+// LR step's prediction has its own), then scan and place.  start: n_cell + 1
+// cell starts; solid_flag (optional) receives the flag that the arrivals
+// raised (see gs_cs_keys).  ga / gb are copied into cell order as by
+// gs_cs_finish.
+int gs_bins_tiles(int64_t n_cell);             // tiles, or 0 where the grid is too large for buckets
+size_t gs_bins_bucket_words(int64_t n_cell);
+size_t gs_bins_count_words(int64_t n_cell);
+cudaError_t gs_bins_keys(cudaStream_t s, const LrBins& b, const float4* pos, int64_t n, const SceneDev* scenes,
+                         const uint32_t* tag, uint32_t* keys, int64_t* launches, int flag_solid, const uint32_t* body);
+cudaError_t gs_bins_finish(cudaStream_t s, const LrBins& b, int64_t n, int64_t n_cell, const uint32_t* keys,
+                           uint32_t* out_keys, uint32_t* out_idx, uint32_t* start, const float4* ga, const float4* gb,
+                           float4* ga_out, float4* gb_out, int64_t* launches, const CsExtras& ex,
+                           unsigned* solid_flag = nullptr);
 // vals[i] = i, or with count not null the arrival rank of slot i in its
 // key's counter (count[key] += 1), for a counting sort by key.
 cudaError_t gs_launch_scene_keys(cudaStream_t s, const float4* pos, int64_t n, const SceneDev* scenes,
@@ -428,13 +449,9 @@ struct PbdArgs {
     const float4* body_xf;
     const uint32_t* sorted_idx;
 };
-cudaError_t gs_launch_predict(cudaStream_t s, const PbdArgs& a, const float4* pos, const float4* vel, float4* xt,
-                              int64_t* launches);
-cudaError_t gs_launch_step_gather(cudaStream_t s, int64_t n, const uint32_t* idx, const float4* xt,
-                                  const float4* pos, float4* s_xt, float4* s_x, int64_t* launches);
 cudaError_t gs_launch_neighbors(cudaStream_t s, const PbdArgs& a, const float4* s_xt, const uint32_t* skeys,
-                                const uint32_t* cell_start, int64_t n_cell, uint32_t* nbr, uint32_t* cnt, int cap,
-                                int* err, int64_t* launches);
+                                const uint32_t* cell_start, uint32_t* nbr, uint32_t* cnt, int cap, int* err,
+                                int64_t* launches);
 // One Jacobi pass.  With fin_idx not null the pass is the step's last: it
 // writes the finalized position and velocity to original order (fin_pos,
 // fin_vel through fin_idx) instead of x_out / xt_out.
@@ -447,6 +464,9 @@ cudaError_t gs_launch_pass(cudaStream_t s, const PbdArgs& a, int stab, const flo
 // Prediction + cell keys + arrival ranks (the counting stage of the binning).
 cudaError_t gs_launch_predict_keys(cudaStream_t s, const PbdArgs& a, const float4* pos, const float4* vel,
                                    float4* xt, uint32_t* keys, uint32_t* rank, uint32_t* cnt, int64_t* launches);
+// The same with the arrivals of the LR binning by buckets.
+cudaError_t gs_launch_predict_bins(cudaStream_t s, const PbdArgs& a, const LrBins& b, const float4* pos,
+                                   const float4* vel, float4* xt, uint32_t* keys, int64_t* launches);
 // All n_stab + iters passes of one step in one cooperative launch of at most
 // max_blocks blocks (gs_solve_blocks: the blocks that fit on the GPU at
 // once), with grid barriers between passes.  bar: two words of scratch.

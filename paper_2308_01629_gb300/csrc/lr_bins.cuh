@@ -13,8 +13,11 @@
 // words that arrive adds to.  A particle beyond kBucket of its cell (a 3 r_LR
 // cube holds 8 LR particles of a 2 r_LR lattice) goes to a list that its
 // cell's particles search; the order is the same.
-// On the digging bed (50,527 LR, 33,213 cells) the chain of clear, keys, two
-// scan launches, scatter and per-cell order took BIN_OLD us, this one BIN_NEW.
+// A binning is a chain of dependent launches, so their number and each one's
+// latency bound it: clear, keys, two scan launches, scatter and a per-cell
+// order that copied cell by cell in one thread before.  With the candidate
+// search they took 30 us of an LR step on the digging bed (50,527 LR, 33,213
+// cells) and take 15; gs_bin_low by itself 31 us, now 17 (launches included).
 #pragma once
 
 #include <cuda_runtime.h>

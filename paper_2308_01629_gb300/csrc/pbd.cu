@@ -25,6 +25,7 @@
 
 #include "grid.cuh"
 #include "gs_internal.cuh"
+#include "lr_bins.cuh"
 #include "pbd_common.cuh"
 #include "sdf.cuh"
 
@@ -41,23 +42,6 @@ __device__ __forceinline__ unsigned cfl_rate_bits(float vx, float vy, float vz, 
 {
     const float s = __fadd_rn(__fadd_rn(__fmul_rn(vx, vx), __fmul_rn(vy, vy)), __fmul_rn(vz, vz));
     return __float_as_uint(__fdiv_rn(__fsqrt_rn(s), __fmul_rn(2.0f, r_low)));
-}
-
-__global__ void k_predict(const PbdArgs a, const float4* __restrict__ pos, const float4* __restrict__ vel,
-                          float4* __restrict__ xt)
-{
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.n) return;
-    const SceneDev& sc = a.scenes[a.lr_scene[i]];
-    const float dt = step_dt(a);
-    float4 x = pos[i], v = vel[i];
-    // particles of infinite mass (1/m = 0: sampled boundaries, rigid bodies)
-    // keep their prescribed velocity
-    const float gdt = x.w > 0.0f ? dt : 0.0f;
-    float vx = v.x + gdt * sc.gx, vy = v.y + gdt * sc.gy, vz = v.z + gdt * sc.gz;
-    // 1/m* = (1/m) e^{h(x)}, h = k (z - ground), at the start-of-step position
-    float ws = x.w * expf(sc.mass_k * (x.z - sc.ground_z));
-    xt[i] = make_float4(x.x + dt * vx, x.y + dt * vy, x.z + dt * vz, ws);
 }
 
 // Prediction fused with the first stage of the binning: x~ as above, then
@@ -81,137 +65,117 @@ __global__ void k_predict_keys(const PbdArgs a, const float4* __restrict__ pos, 
     rank[i] = atomicAdd(cnt + cell, 1u);
 }
 
-__global__ void k_step_gather(int64_t n, const uint32_t* __restrict__ idx, const float4* __restrict__ xt,
-                              const float4* __restrict__ pos, float4* __restrict__ s_xt, float4* __restrict__ s_x)
+__global__ void __launch_bounds__(256) k_predict_bins(const PbdArgs a, const LrBins b,
+                                                      const float4* __restrict__ pos,
+                                                      const float4* __restrict__ vel, float4* __restrict__ xt,
+                                                      uint32_t* __restrict__ keys)
 {
-    int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    uint32_t i = idx[p];
-    s_xt[p] = xt[i];
-    s_x[p] = pos[i];   // w carries the inverse mass
+    __shared__ uint32_t s_tile[kMaxBinTiles];
+    bins_begin(b, s_tile);
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < a.n) {
+        const SceneDev& sc = a.scenes[a.lr_scene[i]];
+        const float dt = step_dt(a);
+        float4 x = pos[i], v = vel[i];
+        const float gdt = x.w > 0.0f ? dt : 0.0f;   // no gravity for 1/m = 0
+        float vx = v.x + gdt * sc.gx, vy = v.y + gdt * sc.gy, vz = v.z + gdt * sc.gz;
+        float ws = x.w * expf(sc.mass_k * (x.z - sc.ground_z));
+        const float4 p = make_float4(x.x + dt * vx, x.y + dt * vy, x.z + dt * vz, ws);
+        xt[i] = p;
+        const uint32_t cell = grid_cell_of(sc, p.x, p.y, p.z);
+        keys[i] = cell;
+        bins_arrive(b, s_tile, cell, (uint32_t)i);
+    }
+    bins_end(b, s_tile);
 }
 
 // Candidate partners of every particle within the neighbour radius, in
-// ascending sorted index row by row of the 27 surrounding cells.  The
-// particles of a cell share their 27-cell candidate set, so one warp walks
-// it once, 32 candidates at a time (lane j takes flat candidate j of the
-// concatenated row ranges), and for each particle of the cell a ballot keeps
-// its accepted candidates in ascending order.  Two ways to hand out cells,
-// with the same lists: on a dense grid one warp per cell (empty cells leave
-// at once); on a sparse grid (many small scenes) warp w takes the cells whose
-// first sorted particle lies in [kNbrGroup w, kNbrGroup (w + 1)), so empty
-// cells cost nothing.
-constexpr int kNbrGroup = 8;
+// ascending sorted index row by row of the 3 x 3 rows of cells around its own
+// (each row's three cells are one run of slots).  kGroup lanes share a
+// particle: they test kGroup slots of a row at a time, the loads of
+// kNbrAhead such rounds in flight together, and a ballot gives the accepted
+// ones their places in order.  The particles of a cell read the same runs at
+// the same time, so the loads are broadcasts.
+constexpr int kNbrAhead = 4;
+// Four lanes while they fit one wave or so: the rest of an LR step besides its
+// passes takes 11 us with four lanes and 23 with one at 4,000 LR, 15 and 25 at
+// 50,527; 35 and 23 at 202,112, where the ballots count.  A warp per cell, as
+// before, took 120 instructions per particle for its 86 candidates (58 us at
+// 202,112 LR against 21).
+constexpr int64_t kNbrGroupMax = 65536;
 
-__device__ __forceinline__ void neighbors_of_cell(const PbdArgs& a, const float4* __restrict__ s_xt,
-                                                  const uint32_t* __restrict__ cell_start, int64_t cell,
-                                                  uint32_t* __restrict__ nbr, uint32_t* __restrict__ cnt, int cap,
-                                                  int* err, int lane)
-{
-    const uint32_t pb = __ldg(cell_start + cell), pe = __ldg(cell_start + cell + 1);
-    const SceneDev& sc = a.scenes[a.lr_scene[pb]];
-    const GridDev& g = sc.g;
-    const uint32_t c = (uint32_t)(cell - sc.cell_off);
-    const int cx = (int)(c % (uint32_t)g.dx);
-    const int cy = (int)((c / (uint32_t)g.dx) % (uint32_t)g.dy);
-    const int cz = (int)(c / ((uint32_t)g.dx * (uint32_t)g.dy));
-    const float rc2 = sc.rc * sc.rc;
-    const int x0 = cx > 0 ? cx - 1 : 0, x1 = cx + 1 < g.dx ? cx + 1 : g.dx - 1;
-    // lane r < 9 fetches row r = (z, y) of the 3 x 3 rows around the cell
-    uint32_t rb = 0, len = 0;
-    if (lane < 9) {
-        const int z = cz - 1 + lane / 3, y = cy - 1 + lane % 3;
-        if (z >= 0 && z < g.dz && y >= 0 && y < g.dy) {
-            const int64_t row = (int64_t)sc.cell_off + ((int64_t)z * g.dy + y) * g.dx;
-            rb = __ldg(cell_start + row + x0);
-            len = __ldg(cell_start + row + x1 + 1) - rb;
-        }
-    }
-    uint32_t incl = len;
-#pragma unroll
-    for (int o = 1; o < 16; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    const uint32_t excl = incl - len;
-    const uint32_t total = __shfl_sync(0xffffffffu, incl, 8);
-    const unsigned lt = (1u << lane) - 1u;
-    for (uint32_t i0 = pb; i0 < pe; i0 += 32) {       // the cell's particles, 32 at a time
-        const uint32_t mine = i0 + (uint32_t)lane;
-        const bool own = mine < pe;
-        const float4 xo = own ? s_xt[mine] : make_float4(0.f, 0.f, 0.f, 0.f);
-        int k = 0;                                      // lane j: count of particle i0 + j
-        const int np = (int)min(pe - i0, 32u);
-        for (uint32_t base = 0; base < total; base += 32) {
-            const uint32_t f = base + (uint32_t)lane;
-            // row of flat index f: last row whose exclusive prefix is <= f
-            int r = 0;
-#pragma unroll
-            for (int step = 8; step > 0; step >>= 1) {
-                const uint32_t e = __shfl_sync(0xffffffffu, excl, (r + step) & 31);
-                if (r + step < 9 && e <= f) r += step;
-            }
-            const uint32_t q = __shfl_sync(0xffffffffu, rb, r) + (f - __shfl_sync(0xffffffffu, excl, r));
-            const bool in = f < total;
-            const float4 xq = in ? s_xt[q] : make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int j = 0; j < np; ++j) {
-                const float px = __shfl_sync(0xffffffffu, xo.x, j);
-                const float py = __shfl_sync(0xffffffffu, xo.y, j);
-                const float pz = __shfl_sync(0xffffffffu, xo.z, j);
-                const float dx = xq.x - px, dy = xq.y - py, dz = xq.z - pz;
-                const bool take = in && q != i0 + (uint32_t)j && dx * dx + dy * dy + dz * dz < rc2;
-                const unsigned bal = __ballot_sync(0xffffffffu, take);
-                const int kj = __shfl_sync(0xffffffffu, k, j);
-                if (take) {
-                    const int pos = kj + __popc(bal & lt);
-                    if (pos < cap) nbr[(int64_t)pos * a.n + i0 + j] = q;
-                }
-                if (lane == j) k += __popc(bal);
-            }
-        }
-        if (own) {
-            if (k > cap) {
-                atomicOr(err, GS_DEVERR_NEIGHBOR_CAP);
-                k = cap;
-            }
-            cnt[mine] = (uint32_t)k;
-        }
-    }
-}
-
-__global__ void __launch_bounds__(128) k_neighbors_cells(const PbdArgs a, const float4* __restrict__ s_xt,
-                                                         const uint32_t* __restrict__ cell_start, int64_t n_cell,
-                                                         uint32_t* __restrict__ nbr, uint32_t* __restrict__ cnt,
-                                                         int cap, int* err)
-{
-    const int lane = (int)(threadIdx.x & 31u);
-    const int64_t cell = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (cell >= n_cell) return;   // whole warps leave together
-    if (__ldg(cell_start + cell) == __ldg(cell_start + cell + 1)) return;
-    neighbors_of_cell(a, s_xt, cell_start, cell, nbr, cnt, cap, err, lane);
-}
-
+template <int kGroup, bool kSingle>
 __global__ void __launch_bounds__(128) k_neighbors(const PbdArgs a, const float4* __restrict__ s_xt,
                                                    const uint32_t* __restrict__ skeys,
                                                    const uint32_t* __restrict__ cell_start,
                                                    uint32_t* __restrict__ nbr, uint32_t* __restrict__ cnt, int cap,
                                                    int* err)
 {
-    const int lane = (int)(threadIdx.x & 31u);
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t p = w * kNbrGroup + lane;
-    bool head = false;
-    uint32_t key = 0;
-    if (lane < kNbrGroup && p < a.n) {
-        key = __ldg(skeys + p);
-        head = p == 0 || __ldg(skeys + p - 1) != key;   // the first particle of its cell
+    const int lane = (int)(threadIdx.x & 31u), sub = lane % kGroup;
+    const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kGroup;
+    const bool own = p < a.n;
+    if (__ballot_sync(0xffffffffu, own) == 0u) return;   // whole warps
+    const int64_t pp = own ? p : a.n - 1;   // lanes past the end repeat the last particle and write nothing
+    const SceneDev& sc = kSingle ? a.scene0 : a.scenes[a.lr_scene[pp]];
+    const GridDev& g = sc.g;
+    const uint32_t c = __ldg(skeys + pp) - sc.cell_off;
+    const float4 x = s_xt[pp];
+    const int cx = (int)(c % (uint32_t)g.dx);
+    const int cy = (int)((c / (uint32_t)g.dx) % (uint32_t)g.dy);
+    const int cz = (int)(c / ((uint32_t)g.dx * (uint32_t)g.dy));
+    const float rc2 = sc.rc * sc.rc;
+    const int x0 = cx > 0 ? cx - 1 : 0, x1 = cx + 1 < g.dx ? cx + 1 : g.dx - 1;
+    uint32_t rb[9], re[9];
+#pragma unroll
+    for (int r = 0; r < 9; ++r) {
+        const int z = cz - 1 + r / 3, y = cy - 1 + r % 3;
+        rb[r] = re[r] = 0u;
+        if (z >= 0 && z < g.dz && y >= 0 && y < g.dy) {
+            const uint32_t* row = cell_start + (int64_t)sc.cell_off + ((int64_t)z * g.dy + y) * g.dx;
+            rb[r] = __ldg(row + x0);
+            re[r] = __ldg(row + x1 + 1);
+        }
     }
-    unsigned heads = __ballot_sync(0xffffffffu, head);
-    while (heads) {                                    // warp-uniform
-        const int j = __ffs(heads) - 1;
-        heads &= heads - 1u;
-        const int64_t cell = (int64_t)__shfl_sync(0xffffffffu, key, j);
-        neighbors_of_cell(a, s_xt, cell_start, cell, nbr, cnt, cap, err, lane);
+    const unsigned mine = kGroup == 32 ? 0xffffffffu : ((1u << (kGroup & 31)) - 1u) << (lane - sub);
+    const unsigned below = mine & ((1u << lane) - 1u);
+    int k = 0;
+    uint32_t* out = nbr + pp;
+#pragma unroll
+    for (int r = 0; r < 9; ++r) {
+        for (uint32_t q0 = rb[r]; kGroup > 1 ? __any_sync(0xffffffffu, q0 < re[r]) : q0 < re[r];
+             q0 += kNbrAhead * kGroup) {
+            float4 y[kNbrAhead];
+            bool in[kNbrAhead];
+#pragma unroll
+            for (int j = 0; j < kNbrAhead; ++j) {
+                const uint32_t q = q0 + (uint32_t)(j * kGroup + sub);
+                in[j] = q < re[r] && q != (uint32_t)pp;
+                y[j] = s_xt[in[j] ? q : (uint32_t)pp];
+            }
+#pragma unroll
+            for (int j = 0; j < kNbrAhead; ++j) {
+                const float dx = y[j].x - x.x, dy = y[j].y - x.y, dz = y[j].z - x.z;
+                const bool take = in[j] && fmaf(dz, dz, fmaf(dx, dx, dy * dy)) < rc2;
+                if constexpr (kGroup == 1) {
+                    if (take) {
+                        if (own && k < cap) out[(int64_t)k * a.n] = q0 + (uint32_t)j;
+                        ++k;
+                    }
+                } else {
+                    const unsigned bal = __ballot_sync(0xffffffffu, take) & mine;
+                    const int at = k + __popc(bal & below);
+                    if (take && own && at < cap) out[(int64_t)at * a.n] = q0 + (uint32_t)(j * kGroup + sub);
+                    k += __popc(bal);
+                }
+            }
+        }
+    }
+    if (own && sub == 0) {
+        if (k > cap) {
+            atomicOr(err, GS_DEVERR_NEIGHBOR_CAP);
+            k = cap;
+        }
+        cnt[p] = (uint32_t)k;
     }
 }
 
@@ -911,15 +875,6 @@ __global__ void k_cfl_pick(CflState* st, float dt_max, float cfl, int max_sub, c
 
 }  // namespace
 
-cudaError_t gs_launch_predict(cudaStream_t s, const PbdArgs& a, const float4* pos, const float4* vel, float4* xt,
-                              int64_t* launches)
-{
-    if (a.n <= 0) return cudaSuccess;
-    k_predict<<<gs_blocks(a.n, 256), 256, 0, s>>>(a, pos, vel, xt);
-    *launches += 1;
-    return cudaGetLastError();
-}
-
 cudaError_t gs_launch_predict_keys(cudaStream_t s, const PbdArgs& a, const float4* pos, const float4* vel,
                                    float4* xt, uint32_t* keys, uint32_t* rank, uint32_t* cnt, int64_t* launches)
 {
@@ -929,27 +884,33 @@ cudaError_t gs_launch_predict_keys(cudaStream_t s, const PbdArgs& a, const float
     return cudaGetLastError();
 }
 
-cudaError_t gs_launch_step_gather(cudaStream_t s, int64_t n, const uint32_t* idx, const float4* xt,
-                                  const float4* pos, float4* s_xt, float4* s_x, int64_t* launches)
+cudaError_t gs_launch_predict_bins(cudaStream_t s, const PbdArgs& a, const LrBins& b, const float4* pos,
+                                   const float4* vel, float4* xt, uint32_t* keys, int64_t* launches)
 {
-    if (n <= 0) return cudaSuccess;
-    k_step_gather<<<gs_blocks(n, 256), 256, 0, s>>>(n, idx, xt, pos, s_xt, s_x);
+    if (a.n <= 0) return cudaSuccess;
+    k_predict_bins<<<gs_blocks(a.n, 256), 256, 0, s>>>(a, b, pos, vel, xt, keys);
     *launches += 1;
     return cudaGetLastError();
 }
 
+template <int kGroup>
+static void launch_neighbors(cudaStream_t s, const PbdArgs& a, const float4* s_xt, const uint32_t* skeys,
+                             const uint32_t* cell_start, uint32_t* nbr, uint32_t* cnt, int cap, int* err)
+{
+    const unsigned nb = gs_blocks(a.n * kGroup, 128);
+    if (a.n_scenes == 1)
+        k_neighbors<kGroup, true><<<nb, 128, 0, s>>>(a, s_xt, skeys, cell_start, nbr, cnt, cap, err);
+    else
+        k_neighbors<kGroup, false><<<nb, 128, 0, s>>>(a, s_xt, skeys, cell_start, nbr, cnt, cap, err);
+}
+
 cudaError_t gs_launch_neighbors(cudaStream_t s, const PbdArgs& a, const float4* s_xt, const uint32_t* skeys,
-                                const uint32_t* cell_start, int64_t n_cell, uint32_t* nbr, uint32_t* cnt, int cap,
-                                int* err, int64_t* launches)
+                                const uint32_t* cell_start, uint32_t* nbr, uint32_t* cnt, int cap, int* err,
+                                int64_t* launches)
 {
     if (a.n <= 0) return cudaSuccess;
-    if (n_cell <= 2 * a.n) {
-        k_neighbors_cells<<<gs_blocks(n_cell * 32, 128), 128, 0, s>>>(a, s_xt, cell_start, n_cell, nbr, cnt, cap,
-                                                                      err);
-    } else {
-        const int64_t warps = (a.n + kNbrGroup - 1) / kNbrGroup;
-        k_neighbors<<<gs_blocks(warps * 32, 128), 128, 0, s>>>(a, s_xt, skeys, cell_start, nbr, cnt, cap, err);
-    }
+    if (a.n <= kNbrGroupMax) launch_neighbors<4>(s, a, s_xt, skeys, cell_start, nbr, cnt, cap, err);
+    else launch_neighbors<1>(s, a, s_xt, skeys, cell_start, nbr, cnt, cap, err);
     *launches += 1;
     return cudaGetLastError();
 }

@@ -19,6 +19,7 @@
 
 #include "grid.cuh"
 #include "gs_internal.cuh"
+#include "lr_bins.cuh"
 
 namespace {
 
@@ -657,6 +658,95 @@ __global__ void __launch_bounds__(kThreads) k_cs_order_big(const uint32_t* __res
     }
 }
 
+// ---- the LR binning by buckets (lr_bins.cuh) ------------------------------
+__global__ void __launch_bounds__(256) k_bins_keys(const LrBins b, const float4* __restrict__ pos, int64_t n,
+                                                   const SceneDev* __restrict__ scenes,
+                                                   const uint32_t* __restrict__ tag, uint32_t* __restrict__ keys,
+                                                   int flag_solid, const uint32_t* __restrict__ body)
+{
+    __shared__ uint32_t s_tile[kMaxBinTiles];
+    bins_begin(b, s_tile);
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) {
+        const SceneDev& sc = scenes[tag[i] & ~kPadBit];
+        const float4 p = pos[i];
+        if (flag_solid && (p.w == 0.0f || (body && body[i] != 0u))) atomicOr(b.words + kBinSolidAcc, 1u);
+        const uint32_t cell = grid_cell_of(sc, p.x, p.y, p.z);
+        keys[i] = cell;
+        bins_arrive(b, s_tile, cell, (uint32_t)i);
+    }
+    bins_end(b, s_tile);
+}
+
+// One block per tile of cells.  The tile sums before it (at most one per
+// thread) give its base, so no launch sums tiles and no block waits.
+__global__ void __launch_bounds__(kScanBlock) k_bins_scan(const LrBins b, uint32_t* __restrict__ start, int64_t total,
+                                                          unsigned* solid_flag)
+{
+    __shared__ uint32_t ws[32];
+    static_assert(kBinTile == kScanTile && kMaxBinTiles <= kScanBlock, "one word per thread");
+    const int64_t i0 = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanPer;
+    const uint4 v = *reinterpret_cast<const uint4*>(b.count + i0);   // padded to whole tiles
+    const uint32_t before = threadIdx.x < blockIdx.x ? b.tile[threadIdx.x] : 0u;
+    uint32_t base, tot;
+    block_scan(before, ws, &base);
+    const uint32_t sum = v.x + v.y + v.z + v.w;
+    uint32_t run = base + block_scan(sum, ws, &tot) - sum;
+    const uint32_t c[kScanPer] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int k = 0; k < kScanPer; ++k) {
+        if (i0 + k < total) start[i0 + k] = run;
+        run += c[k];
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {   // this binning's words, and zero for the next one's arrivals
+        b.words[kBinSpill] = b.words[kBinSpillAcc];
+        b.words[kBinSpillAcc] = 0u;
+        if (solid_flag) *solid_flag = b.words[kBinSolidAcc];
+        b.words[kBinSolidAcc] = 0u;
+    }
+}
+
+__global__ void __launch_bounds__(128) k_bins_place(const LrBins b, int64_t n, const uint32_t* __restrict__ keys,
+                                                    const uint32_t* __restrict__ start,
+                                                    uint32_t* __restrict__ out_keys, uint32_t* __restrict__ out_idx,
+                                                    const float4* __restrict__ ga, const float4* __restrict__ gb,
+                                                    float4* __restrict__ ga_out, float4* __restrict__ gb_out,
+                                                    const CsExtras ex)
+{
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (int64_t k = t; k < b.n_tiles; k += (int64_t)gridDim.x * blockDim.x) b.tile[k] = 0u;
+    if (t >= n) return;
+    const uint32_t i = (uint32_t)t;
+    const uint32_t key = keys[i];
+    float4 u = ga[i], v = gb[i];
+    const uint32_t s = start[key], c = start[key + 1] - s;
+    const uint4* bk = reinterpret_cast<const uint4*>(b.bucket + (size_t)key * kBucket);
+    uint32_t rank = 0;
+#pragma unroll
+    for (int k = 0; k < kBucket; k += 4) {
+        if ((uint32_t)k >= c) break;
+        const uint4 e = bk[k / 4];   // entries beyond the count are stale
+        rank += (e.x < i ? 1u : 0u) + (k + 1 < c && e.y < i ? 1u : 0u) + (k + 2 < c && e.z < i ? 1u : 0u) +
+                (k + 3 < c && e.w < i ? 1u : 0u);
+    }
+    if (c > (uint32_t)kBucket) {
+        const uint32_t m = b.words[kBinSpill];
+        for (uint32_t k = 0; k < m; ++k) {
+            const uint32_t j = b.spill[k];
+            if (j < i && keys[j] == key) ++rank;
+        }
+    }
+    b.count[key] = 0u;   // every particle of the cell writes the same
+    const uint32_t slot = s + rank;
+    out_keys[slot] = key;
+    out_idx[slot] = i;
+    if (ex.ga_solid && ex.ga_solid[i] != 0u) u.w = 0.0f;
+    if (ex.gb_w) v.w = __uint_as_float(ex.gb_w[i]);
+    ga_out[slot] = u;
+    gb_out[slot] = v;
+    if (ex.slot_of) ex.slot_of[i] = slot;
+}
+
 __global__ void k_cell_start(const uint32_t* __restrict__ sk, int64_t n, int64_t n_cell, uint32_t* __restrict__ start)
 {
     int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -815,17 +905,36 @@ cudaError_t gs_cs_finish(cudaStream_t s, int64_t n, int64_t n_cell, const uint32
     return cudaGetLastError();
 }
 
-cudaError_t gs_count_sort_cells(cudaStream_t s, const float4* pos, int64_t n, const SceneDev* scenes,
-                                const uint32_t* tag, int64_t n_cell, uint32_t* keys, uint32_t* rank,
-                                uint32_t* out_keys, uint32_t* out_idx, uint32_t* cell_start, uint32_t* aux,
-                                int64_t* launches)
+int gs_bins_tiles(int64_t n_cell)
 {
-    cudaError_t e = gs_cs_clear(s, cell_start, n_cell);
-    if (e == cudaSuccess) e = gs_cs_keys(s, pos, n, scenes, tag, keys, rank, cell_start, launches);
-    if (e == cudaSuccess)
-        e = gs_cs_finish(s, n, n_cell, keys, rank, out_keys, out_idx, cell_start, aux, nullptr, nullptr, nullptr,
-                         nullptr, launches);
-    return e;
+    const int64_t t = (n_cell + 1 + kBinTile - 1) / kBinTile;
+    return t <= kMaxBinTiles ? (int)t : 0;
+}
+size_t gs_bins_bucket_words(int64_t n_cell) { return (size_t)n_cell * kBucket; }
+size_t gs_bins_count_words(int64_t n_cell) { return (size_t)gs_bins_tiles(n_cell) * kBinTile; }
+
+cudaError_t gs_bins_keys(cudaStream_t s, const LrBins& b, const float4* pos, int64_t n, const SceneDev* scenes,
+                         const uint32_t* tag, uint32_t* keys, int64_t* launches, int flag_solid, const uint32_t* body)
+{
+    if (n <= 0) return cudaSuccess;
+    k_bins_keys<<<gs_blocks(n, 256), 256, 0, s>>>(b, pos, n, scenes, tag, keys, flag_solid, body);
+    *launches += 1;
+    return cudaGetLastError();
+}
+
+cudaError_t gs_bins_finish(cudaStream_t s, const LrBins& b, int64_t n, int64_t n_cell, const uint32_t* keys,
+                           uint32_t* out_keys, uint32_t* out_idx, uint32_t* start, const float4* ga, const float4* gb,
+                           float4* ga_out, float4* gb_out, int64_t* launches, const CsExtras& ex,
+                           unsigned* solid_flag)
+{
+    k_bins_scan<<<(unsigned)b.n_tiles, kScanBlock, 0, s>>>(b, start, n_cell + 1, solid_flag);
+    *launches += 1;
+    if (n > 0) {
+        k_bins_place<<<gs_blocks(n, 128), 128, 0, s>>>(b, n, keys, start, out_keys, out_idx, ga, gb, ga_out, gb_out,
+                                                       ex);
+        *launches += 1;
+    }
+    return cudaGetLastError();
 }
 
 cudaError_t gs_launch_cell_keys(cudaStream_t s, const float4* pos, int64_t n, GridDev g, int fine, uint32_t* keys,

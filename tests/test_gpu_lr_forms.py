@@ -1,0 +1,96 @@
+"""The forms of the LR step's kernels against one another: eight or two lanes
+per particle in a pass, four or one in the candidate search, one-scene
+parameters or a scene table, and the binning by buckets or by the general
+counting sort.  Which form runs depends on the sizes only, and all give the
+same bits, so the same scene is stepped alone and among copies of itself."""
+import numpy as np
+import pytest
+
+import scenes
+
+pytestmark = pytest.mark.gpu
+
+
+def _small(kind):
+    sc = scenes.cube(n_side=12, ratio=1)
+    if kind == "packed":     # over 64 candidates per particle and cells of over 16: windows and spilled buckets
+        c = sc["lr_pos"][:, :3].mean(0)
+        sc["lr_pos"][:, :3] = c + (sc["lr_pos"][:, :3] - c) * np.float32(0.45)
+    rng = np.random.default_rng(5)
+    sc["lr_vel"][:, :3] = rng.normal(0.0, 0.4, (len(sc["lr_vel"]), 3))
+    return sc
+
+
+def _states(gs, sl, frames=2, mat=None, dt=1.0 / 60.0):
+    ctx = gs.Context(sl if len(sl) > 1 else sl[0], max_neighbors=512)
+    if mat is not None:
+        ctx.set_materials(scenes.MATERIALS, np.concatenate([mat] * len(sl)))
+    for _ in range(frames):
+        ctx.frame(dt, 2, 5)
+    out = [ctx.read(f)[ctx.scene_slice(k, f)] for k in range(len(sl)) for f in (gs.GS_FIELD_LR_POS, gs.GS_FIELD_LR_VEL)]
+    ctx.close()
+    return out
+
+
+@pytest.mark.parametrize("copies", [3, 10, 39])     # 5,184 / 17,280 / 67,392 LR: on each side of both lines
+@pytest.mark.parametrize("kind", ["cube", "packed", "materials"])
+def test_lane_forms_give_the_same_bits(kind, copies):
+    import paper_2308_01629_gb300 as gs
+    sc = _small(kind)
+    mat = np.random.default_rng(6).integers(0, 3, len(sc["lr_pos"])).astype(np.uint32) if kind == "materials" else None
+    ref = _states(gs, [sc], mat=mat)
+    got = _states(gs, [sc] * copies, mat=mat)
+    for k in range(copies):
+        np.testing.assert_array_equal(got[2 * k], ref[0])
+        np.testing.assert_array_equal(got[2 * k + 1], ref[1])
+
+
+@pytest.mark.parametrize("size", [0.66, 1.17])      # 22,000 / 69,000 LR
+def test_one_scene_equals_a_scene_among_others(size):
+    import paper_2308_01629_gb300 as gs
+    sc = scenes.digging(ratio=1, size=size)
+    sc["lr_vel"][:, :3] = np.random.default_rng(7).normal(0.0, 0.2, (len(sc["lr_vel"]), 3))
+    ref = _states(gs, [sc], frames=1)
+    got = _states(gs, [sc, scenes.cube(ratio=1)], frames=1)
+    np.testing.assert_array_equal(got[0], ref[0])
+    np.testing.assert_array_equal(got[1], ref[1])
+
+
+@pytest.mark.parametrize("pile", [0, 15, 16, 17, 33, 700])
+@pytest.mark.parametrize("n_cells_x", [1, 63, 64, 65])    # with 8 x 8 more: one cell row up to past a tile of 4,096
+def test_bucket_binning_order(orc, pile, n_cells_x):
+    import paper_2308_01629_gb300 as gs
+    sc = dict(scenes.cube(ratio=1))
+    h = float(np.float32(3.0 * sc["r_low"] * (1.0 + 1.0 / 1024.0)))
+    sc["box_lo"], sc["box_hi"] = (0.0, 0.0, 0.0), (h * (n_cells_x - 0.5), 7.5 * h, 7.5 * h)
+    rng = np.random.default_rng(pile + n_cells_x)
+    ctx = None
+    for round_ in range(2):      # the second binning meets what the first one left of its counts
+        p = sc["lr_pos"].copy()
+        p[:, :3] = rng.uniform(-0.5 * h, np.asarray(sc["box_hi"]) + 0.5 * h, (len(p), 3))
+        p[rng.choice(len(p), pile, replace=False), :3] = np.asarray(sc["box_hi"]) - 0.3 * h
+        if ctx is None:
+            ctx = gs.Context(dict(sc, lr_pos=p))
+        else:
+            ctx.write(gs.GS_FIELD_LR_POS, p)
+        ctx.bin_low()
+        o, _, ih, dims = orc.grid(float(np.float32(sc["r_low"])), np.float32(sc["box_lo"]).astype(float),
+                                  np.float32(sc["box_hi"]).astype(float))
+        nc = int(np.prod(dims))
+        ref_idx, ref_start = orc.counting_sort(orc.cell_keys(p, o, ih, dims), nc)
+        np.testing.assert_array_equal(ctx.read(gs.GS_FIELD_LR_SORTED_INDEX), ref_idx)
+        np.testing.assert_array_equal(ctx.read(gs.GS_FIELD_LR_CELL_START)[:nc + 1], ref_start)
+    ctx.close()
+
+
+def test_a_grid_too_large_for_buckets_gives_the_same_steps():
+    # over four million cells take the general counting sort; the cell order
+    # of the particles is that of the small grid with the same origin
+    import paper_2308_01629_gb300 as gs
+    sc = _small("cube")
+    sc["sdfs"] = [scenes.box_interior((0, 0, 0), (0.5, 0.5, 0.5))]
+    ref = _states(gs, [sc])
+    big = dict(sc, box_hi=(5.0, 5.0, 5.0))
+    got = _states(gs, [big])
+    np.testing.assert_array_equal(got[0], ref[0])
+    np.testing.assert_array_equal(got[1], ref[1])
