@@ -590,7 +590,8 @@ int bin_low_impl(gs_ctx* c)
                         1, body),
            "cell keys");
         CK(gs_bins_finish(c->stream, c->bins, c->n_low, c->n_cell_total, c->lr_keys[0], c->lr_keys[1], c->lr_vals[1],
-                          c->lr_cell_start, c->lr_pos, c->lr_vel, c->lr_spos, c->lr_svel, &c->launches, ex, flag),
+                          c->lr_cell_start, c->lr_pos, c->lr_vel, c->lr_spos, c->lr_svel, &c->launches, ex, flag,
+                          c->d_work),
            "bin by cell");
     } else {
         CK(gs_cs_clear(c->stream, c->lr_cell_start, c->n_cell_total, 1), "clear counts");
@@ -623,9 +624,11 @@ UpsampleArgs upsample_args(const gs_ctx* c, float dt, const float4* in_pos, cons
     u.hr_tag = c->hr_scene;
     u.sdf = c->d_sdf;
     u.n_scenes = c->n_scenes;
+    u.scene0 = c->scenes[0];
     u.n_warps = c->n_warps;
     u.item_begin = 0;
     u.work = c->d_work;
+    u.clear_work = !c->bins.count;   // one gather follows each binning
     u.solid_flag = c->lr_cell_start + c->n_cell_total + 1;
     u.dt = dt;
     return u;
@@ -2035,9 +2038,10 @@ int gs_autotune(gs_ctx* c, float dt, int reps, int* warps_per_block, int* blocks
     // candidate shapes, timed on the current state written out of place
     // (the state is left unchanged)
     const int shapes[][2] = {{8, 0}, {4, 0}, {16, 0}, {8, 1}, {8, 2}, {8, 3}, {8, 4}, {4, 4},
-                             {4, 8}, {16, 1}, {16, 2}};
+                             {4, 7}, {4, 8}, {16, 1}, {16, 2}};
     const int cur = c->hr_cur;
     UpsampleArgs u = upsample_args(c, dt, c->hr_pos[cur], c->hr_vel[cur], c->hr_pos[cur ^ 1], c->hr_vel[cur ^ 1]);
+    u.clear_work = true;   // many gathers on one binning
     cudaEvent_t a, b;
     CK(cudaEventCreate(&a), "event");
     CK(cudaEventCreate(&b), "event");

@@ -280,7 +280,7 @@ struct gs_ctx {
 
     // persistent upsampling: work counter and launch shape (autotuned)
     unsigned* d_work = nullptr;
-    int tune_warps = 8;          // warps per block
+    int tune_warps = 0;          // warps per block; 0: chosen by the number of items
     int tune_blocks_per_sm = 0;  // 0: one warp item per warp (grid launch); else persistent
     int sm_count = 152;
 
@@ -375,7 +375,7 @@ cudaError_t gs_bins_keys(cudaStream_t s, const LrBins& b, const float4* pos, int
 cudaError_t gs_bins_finish(cudaStream_t s, const LrBins& b, int64_t n, int64_t n_cell, const uint32_t* keys,
                            uint32_t* out_keys, uint32_t* out_idx, uint32_t* start, const float4* ga, const float4* gb,
                            float4* ga_out, float4* gb_out, int64_t* launches, const CsExtras& ex,
-                           unsigned* solid_flag = nullptr);
+                           unsigned* solid_flag = nullptr, unsigned* clear = nullptr);   // *clear = 0 on the way
 // vals[i] = i, or with count not null the arrival rank of slot i in its
 // key's counter (count[key] += 1), for a counting sort by key.
 cudaError_t gs_launch_scene_keys(cudaStream_t s, const float4* pos, int64_t n, const SceneDev* scenes,
@@ -412,12 +412,15 @@ struct UpsampleArgs {
     const uint32_t* hr_tag;
     const gs_sdf* sdf;
     int n_scenes;
+    SceneDev scene0;           // the first scene's descriptor (what a one-scene context reads)
     int64_t n_warps;           // warp items
     int64_t item_begin;        // first item: the launch covers items [item_begin, item_begin + n_warps)
-    unsigned* work;            // persistent mode: next warp item (zeroed before the launch)
+    unsigned* work;            // persistent mode: next warp item (zero before the launch)
+    bool clear_work;           // zero it here (else the LR binning before the gather has)
     const unsigned* solid_flag;   // nonzero: some LR particle has w = 0 (set by the LR binning)
     float dt;
 };
+// warps_per_block == 0: a shape by the number of items.
 // blocks_per_sm == 0: one warp per item; else a persistent grid of
 // blocks_per_sm blocks per SM pulling items from *work (bounded loop).
 cudaError_t gs_launch_upsample(cudaStream_t s, const UpsampleArgs& a, int warps_per_block, int blocks_per_sm,

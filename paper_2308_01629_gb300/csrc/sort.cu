@@ -681,7 +681,7 @@ __global__ void __launch_bounds__(256) k_bins_keys(const LrBins b, const float4*
 // One block per tile of cells.  The tile sums before it (at most one per
 // thread) give its base, so no launch sums tiles and no block waits.
 __global__ void __launch_bounds__(kScanBlock) k_bins_scan(const LrBins b, uint32_t* __restrict__ start, int64_t total,
-                                                          unsigned* solid_flag)
+                                                          unsigned* solid_flag, unsigned* clear)
 {
     __shared__ uint32_t ws[32];
     static_assert(kBinTile == kScanTile && kMaxBinTiles <= kScanBlock, "one word per thread");
@@ -703,6 +703,7 @@ __global__ void __launch_bounds__(kScanBlock) k_bins_scan(const LrBins b, uint32
         b.words[kBinSpillAcc] = 0u;
         if (solid_flag) *solid_flag = b.words[kBinSolidAcc];
         b.words[kBinSolidAcc] = 0u;
+        if (clear) *clear = 0u;
     }
 }
 
@@ -925,9 +926,9 @@ cudaError_t gs_bins_keys(cudaStream_t s, const LrBins& b, const float4* pos, int
 cudaError_t gs_bins_finish(cudaStream_t s, const LrBins& b, int64_t n, int64_t n_cell, const uint32_t* keys,
                            uint32_t* out_keys, uint32_t* out_idx, uint32_t* start, const float4* ga, const float4* gb,
                            float4* ga_out, float4* gb_out, int64_t* launches, const CsExtras& ex,
-                           unsigned* solid_flag)
+                           unsigned* solid_flag, unsigned* clear)
 {
-    k_bins_scan<<<(unsigned)b.n_tiles, kScanBlock, 0, s>>>(b, start, n_cell + 1, solid_flag);
+    k_bins_scan<<<(unsigned)b.n_tiles, kScanBlock, 0, s>>>(b, start, n_cell + 1, solid_flag, clear);
     *launches += 1;
     if (n > 0) {
         k_bins_place<<<gs_blocks(n, 128), 128, 0, s>>>(b, n, keys, start, out_keys, out_idx, ga, gb, ga_out, gb_out,

@@ -25,11 +25,21 @@
 // it, so scenes without such particles run the plain gather.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "gs_internal.cuh"
 #include "sdf.cuh"
 
 namespace {
 
+// Launch shape where the caller sets none: blocks of four warps, one item per
+// warp, and from about two waves on (152 SMs x 28 warps) a persistent grid
+// whose warps pull items, which balances them.  Gather of a frame (before:
+// eight warps, one item each): cube 250 items 25 us (25; persistent 26),
+// funnel 15,625 94 (115), digging 63,160 157 (220; one item per warp 165),
+// 2 x 2 m bed 252,640 576 (856; 619), 64 scenes 143,255 506 (609; 538).
+constexpr int64_t kPersistentItems = 8192;
+constexpr int kAutoBlocks = 7;   // 28 warps per SM: 72 registers; 8 spill (digging 162 us), 6 are 164
 constexpr int kBuf = 64;   // staged LR per warp; flushed at >= 32
 // The staged LR set of a warp is eight arrays of kBuf floats (structure of
 // arrays): 2 w_x, 2 w_y, 2 w_z, -|w|^2 (w the LR position relative to the
@@ -118,15 +128,19 @@ __device__ __forceinline__ int sub_floor(float x, float o, float inv_h)
 }
 
 // One warp item: the 32 HR slots [32 item, 32 item + 32) of one scene.
-// st: this warp's staged LR set (kStage floats).  sol (kSolid): this warp's
-// 5 x 32 sums of solid particles (S, V, max w per lane), zero on entry and on
-// return.
-template <bool kSolid>
-__device__ __forceinline__ void upsample_item(const UpsampleArgs& a, int64_t item, float* st, float* sol, int lane)
+// st: this warp's staged LR set (kStage floats).  rows: 32 words for its rows
+// of cells.  sol (kSolid): this warp's 5 x 32 sums of solid particles (S, V,
+// max w per lane), zero on entry and on return.  kSingle: a context of one
+// scene, whose parameters ride in the arguments instead of two dependent
+// loads per item.
+template <bool kSolid, bool kSingle>
+__device__ __forceinline__ void upsample_item(const UpsampleArgs& a, int64_t item, float* st, uint32_t* rows,
+                                              float* sol, int lane)
 {
     const int64_t first = item * 32;
-    const uint32_t tag = __ldg(a.hr_tag + first);          // the first slot of an item is never padding
-    const SceneDev& sc = a.scenes[tag & ~kPadBit];
+    // the first slot of an item is never padding
+    const uint32_t scene = kSingle ? 0u : __ldg(a.hr_tag + first) & ~kPadBit;
+    const SceneDev& sc = kSingle ? a.scene0 : a.scenes[scene];
     const int64_t i = first + lane;
     const bool valid = i < sc.hr_end;
 
@@ -140,7 +154,7 @@ __device__ __forceinline__ void upsample_item(const UpsampleArgs& a, int64_t ite
 
     const float R = 3.0f * sc.r_low * (1.0f + 1.0e-5f);    // support, padded against rounding
     const float R2 = R * R;
-    const unsigned lt = (1u << lane) - 1u;
+    const unsigned lt = (1u << lane) - 1u, le = (lt << 1) | 1u;
     const float inv3r = 1.0f / (3.0f * sc.r_low);
     const int64_t coff = sc.cell_off;
 
@@ -302,21 +316,23 @@ __device__ __forceinline__ void upsample_item(const UpsampleArgs& a, int64_t ite
             }
             const uint32_t excl = incl - len;
             const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+            // the rows that hold any, in order: flat index f of the t-th is
+            // slot f + rows[t]
+            const unsigned some = __ballot_sync(0xffffffffu, len != 0u);
+            if (len != 0u) rows[__popc(some & lt)] = rb - excl;
+            __syncwarp();
+            int before = 0;   // rows that start before base
             for (uint32_t base = 0; base < total; base += 32) {
                 const uint32_t f = base + lane;
                 bool take = false;
                 float4 c = make_float4(0.f, 0.f, 0.f, 0.f), cv = c;
-                // row of flat index f: last row whose exclusive prefix is <= f
-                int lo = 0;
-#pragma unroll
-                for (int step = 16; step > 0; step >>= 1) {
-                    const uint32_t e = __shfl_sync(0xffffffffu, excl, lo + step);
-                    if (lo + step < 32 && e <= f) lo += step;
-                }
-                const uint32_t rbase = __shfl_sync(0xffffffffu, rb, lo);
-                const uint32_t rex = __shfl_sync(0xffffffffu, excl, lo);
+                // row of f: the starts in this round of 32 as bits, those up to f counted
+                const uint32_t off = excl - base;
+                const unsigned starts = __reduce_or_sync(0xffffffffu, len != 0u && off < 32u ? 1u << off : 0u);
+                const int t = before + __popc(starts & le) - 1;
+                before += __popc(starts);
                 if (f < total) {
-                    const uint32_t jj = rbase + (f - rex);
+                    const uint32_t jj = f + rows[t];
                     c = __ldg(a.lr_spos + jj);
                     cv = __ldg(a.lr_svel + jj);
                     const float ex = fmaxf(fmaxf(lx - c.x, c.x - hx), 0.0f);
@@ -334,6 +350,7 @@ __device__ __forceinline__ void upsample_item(const UpsampleArgs& a, int64_t ite
                     batch_solid = false;
                 }
             }
+            __syncwarp();   // rows is written again
         }
         if (cnt > 0) flush(cnt, batch_solid);
     }
@@ -363,20 +380,24 @@ __device__ __forceinline__ void upsample_item(const UpsampleArgs& a, int64_t ite
     const bool A = wmax <= sc.c1;
     const bool B = S > 0.0f && wmax >= sc.c2 * S;
     const float alpha = (A || B) ? 1.0f - wmax : 0.0f;
-    float nvx = (1.0f - alpha) * vtx + alpha * (v.x + a.dt * sc.gx);
-    float nvy = (1.0f - alpha) * vty + alpha * (v.y + a.dt * sc.gy);
-    float nvz = (1.0f - alpha) * vtz + alpha * (v.z + a.dt * sc.gz);
-    float nx = p.x + a.dt * nvx, ny = p.y + a.dt * nvy, nz = p.z + a.dt * nvz;
+    // multiply-adds written out, so that every instantiation rounds alike
+    // (left to the compiler they differ where a factor is a kernel argument)
+    float nvx = fmaf(1.0f - alpha, vtx, alpha * fmaf(a.dt, sc.gx, v.x));
+    float nvy = fmaf(1.0f - alpha, vty, alpha * fmaf(a.dt, sc.gy, v.y));
+    float nvz = fmaf(1.0f - alpha, vtz, alpha * fmaf(a.dt, sc.gz, v.z));
+    float nx = fmaf(a.dt, nvx, p.x), ny = fmaf(a.dt, nvy, p.y), nz = fmaf(a.dt, nvz, p.z);
     hr_boundary(nx, ny, nz, nvx, nvy, nvz, a.sdf + sc.sdf_begin, sc.n_sdf, sc.r_high);
     __stcs(a.out_pos + i, make_float4(nx, ny, nz, p.w));
     __stcs(a.out_vel + i, make_float4(nvx, nvy, nvz, 0.0f));
 }
 
-template <int WARPS, bool kSolid>
-__global__ void __launch_bounds__(WARPS * 32, 24 / WARPS) k_upsample(const UpsampleArgs a, int persistent)
+template <int WARPS, bool kSolid, bool kSingle>
+__global__ void __launch_bounds__(WARPS * 32, WARPS == 4 && !kSolid ? kAutoBlocks : 24 / WARPS)
+    k_upsample(const UpsampleArgs a, int persistent)
 {
     if ((*a.solid_flag != 0u) != kSolid) return;   // the other instantiation does the frame
     __shared__ __align__(16) float s_st[WARPS][kStage];
+    __shared__ uint32_t s_rows[WARPS][32];
     __shared__ float s_sol[kSolid ? WARPS : 1][5 * 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if constexpr (kSolid) {
@@ -409,42 +430,50 @@ __global__ void __launch_bounds__(WARPS * 32, 24 / WARPS) k_upsample(const Upsam
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(a.hr_vel + line));
             }
         }
-        upsample_item<kSolid>(a, a.item_begin + item, s_st[warp], s_sol[kSolid ? warp : 0], lane);
+        upsample_item<kSolid, kSingle>(a, a.item_begin + item, s_st[warp], s_rows[warp], s_sol[kSolid ? warp : 0], lane);
     }
 }
 
 }  // namespace
 
-template <int WARPS>
+template <int WARPS, bool kSingle>
 static cudaError_t launch_w(cudaStream_t s, const UpsampleArgs& a, int blocks_per_sm, int sm_count)
 {
     // both instantiations; the one the device flag does not select returns
-    if (blocks_per_sm <= 0) {
-        k_upsample<WARPS, false><<<gs_blocks(a.n_warps, WARPS), WARPS * 32, 0, s>>>(a, 0);
-        k_upsample<WARPS, true><<<gs_blocks(a.n_warps, WARPS), WARPS * 32, 0, s>>>(a, 0);
-    } else {
-        int64_t nb = (int64_t)blocks_per_sm * sm_count;
-        const int64_t need = (a.n_warps + WARPS - 1) / WARPS;
-        if (nb > need) nb = need;
-        k_upsample<WARPS, false><<<(unsigned)nb, WARPS * 32, 0, s>>>(a, 1);
-        k_upsample<WARPS, true><<<(unsigned)nb, WARPS * 32, 0, s>>>(a, 1);
-    }
+    // (the one for solid particles always as a persistent grid, so that a
+    // frame without them pays for few blocks: the full grid's empty blocks
+    // took 18 us on the 2 x 2 m bed)
+    const unsigned need = gs_blocks(a.n_warps, WARPS);
+    const int64_t resident = (int64_t)std::max(blocks_per_sm, 1) * sm_count;
+    const unsigned nb = (unsigned)std::min<int64_t>(resident, need);
+    if (blocks_per_sm <= 0) k_upsample<WARPS, false, kSingle><<<need, WARPS * 32, 0, s>>>(a, 0);
+    else k_upsample<WARPS, false, kSingle><<<nb, WARPS * 32, 0, s>>>(a, 1);
+    const unsigned nb_solid = (unsigned)std::min<int64_t>((int64_t)(24 / WARPS) * sm_count, need);
+    k_upsample<WARPS, true, kSingle><<<nb_solid, WARPS * 32, 0, s>>>(a, 1);
     return cudaGetLastError();
+}
+
+template <int WARPS>
+static cudaError_t launch_scenes(cudaStream_t s, const UpsampleArgs& a, int blocks_per_sm, int sm_count)
+{
+    return a.n_scenes == 1 ? launch_w<WARPS, true>(s, a, blocks_per_sm, sm_count)
+                           : launch_w<WARPS, false>(s, a, blocks_per_sm, sm_count);
 }
 
 cudaError_t gs_launch_upsample(cudaStream_t s, const UpsampleArgs& a, int warps_per_block, int blocks_per_sm,
                                int sm_count, int64_t* launches)
 {
     if (a.n_warps <= 0) return cudaSuccess;
-    if (blocks_per_sm > 0) {
-        cudaError_t e = cudaMemsetAsync(a.work, 0, sizeof(unsigned), s);
-        if (e != cudaSuccess) return e;
+    cudaError_t e = a.clear_work ? cudaMemsetAsync(a.work, 0, sizeof(unsigned), s) : cudaSuccess;
+    if (e != cudaSuccess) return e;
+    if (warps_per_block == 0) {   // by the number of items
+        warps_per_block = 4;
+        blocks_per_sm = a.n_warps >= kPersistentItems ? kAutoBlocks : 0;
     }
-    cudaError_t e;
     switch (warps_per_block) {
-    case 4: e = launch_w<4>(s, a, blocks_per_sm, sm_count); break;
-    case 16: e = launch_w<16>(s, a, blocks_per_sm, sm_count); break;
-    default: e = launch_w<8>(s, a, blocks_per_sm, sm_count); break;
+    case 4: e = launch_scenes<4>(s, a, blocks_per_sm, sm_count); break;
+    case 16: e = launch_scenes<16>(s, a, blocks_per_sm, sm_count); break;
+    default: e = launch_scenes<8>(s, a, blocks_per_sm, sm_count); break;
     }
     *launches += 2;   // the two instantiations
     return e;

@@ -94,3 +94,27 @@ def test_a_grid_too_large_for_buckets_gives_the_same_steps():
     got = _states(gs, [big])
     np.testing.assert_array_equal(got[0], ref[0])
     np.testing.assert_array_equal(got[1], ref[1])
+
+
+@pytest.mark.parametrize("solid", [False, True])
+@pytest.mark.parametrize("ratio", [3, 12])      # 4,700 / 18,900 warp items: on each side of the persistent grid's line
+def test_gather_shapes_and_scene_forms_give_the_same_bits(ratio, solid):
+    import paper_2308_01629_gb300 as gs
+    sc = scenes.stir(scenes.digging(ratio=ratio), seed=9)
+    if solid:
+        sc["lr_pos"][::97, 3] = 0.0
+
+    def run(sl, shape):
+        ctx = gs.Context(sl if len(sl) > 1 else sl[0])
+        if shape:
+            ctx.set_tuning(*shape)
+        for _ in range(2):
+            ctx.upsample(1.0 / 60.0)
+        out = [ctx.read(f)[ctx.scene_slice(0, f)] for f in (gs.GS_FIELD_HR_POS, gs.GS_FIELD_HR_VEL)]
+        ctx.close()
+        return out
+
+    ref = run([sc], (8, 0))
+    for sl, shape in (([sc], None), ([sc], (4, 7)), ([sc], (16, 0)), ([sc, scenes.cube()], None)):
+        for a, b in zip(run(sl, shape), ref):
+            np.testing.assert_array_equal(a.view(np.uint32), b.view(np.uint32))
