@@ -324,15 +324,22 @@ __global__ void __launch_bounds__(128) k_upsample_bwd_lr(const SceneDev* __restr
     }
 }
 
-// out[idx[p]] = in[p] for both arrays
+// out[idx[p]] = in[p] for both arrays; with add, their x, y, z are added to
+// what out holds (whose w stays).
 __global__ void k_scatter2(const uint32_t* __restrict__ idx, const float4* __restrict__ a, const float4* __restrict__ b,
-                           float4* __restrict__ ao, float4* __restrict__ bo, int64_t n)
+                           float4* __restrict__ ao, float4* __restrict__ bo, int64_t n, int add)
 {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const uint32_t i = idx[p];
-    ao[i] = a[p];
-    bo[i] = b[p];
+    float4 u = a[p], v = b[p];
+    if (add) {
+        const float4 x = ao[i], y = bo[i];
+        u = make_float4(x.x + u.x, x.y + u.y, x.z + u.z, x.w);
+        v = make_float4(y.x + v.x, y.y + v.y, y.z + v.z, y.w);
+    }
+    ao[i] = u;
+    bo[i] = v;
 }
 
 
@@ -486,10 +493,15 @@ __device__ __forceinline__ int lane_active_count(const PbdArgs& a, const SceneDe
     return n_act;
 }
 
-// h_p = upstream_p / n_p for one pass (n_p = active pair and SDF contacts)
+// The start of the reverse: the cotangents of the step's end, v = (x~ - x) / dt
+// and x = x~ (as k_adj_init), and h_p = upstream_p / n_p for the last pass
+// (n_p = active pair and SDF contacts).
+template <bool kSingle>
 __global__ void k_adj_h(const PbdArgs a, int stab, const float4* __restrict__ Y, const float4* __restrict__ WS,
                         const uint32_t* __restrict__ nbr, const uint32_t* __restrict__ cnt,
-                        const float4* __restrict__ gx, const float4* __restrict__ gxt, float4* __restrict__ H)
+                        const uint32_t* __restrict__ idx, const float4* __restrict__ gxo,
+                        const float4* __restrict__ gvo, float4* __restrict__ gx, float4* __restrict__ gxt,
+                        float* __restrict__ gws, float4* __restrict__ H)
 {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t p = t / kAdjLanes;
@@ -497,14 +509,19 @@ __global__ void k_adj_h(const PbdArgs a, int stab, const float4* __restrict__ Y,
     const bool live = p < a.n;   // every lane stays for the shuffles
     int n_act = 0;
     if (live) {
-        const SceneDev& sc = a.scenes[a.lr_scene[p]];
+        const SceneDev& sc = kSingle ? a.scene0 : a.scenes[a.lr_scene[p]];
         n_act = lane_active_count(a, sc, Y, WS, nbr, p, (int)cnt[p], Y[p], WS[p].w, lane);
     }
     n_act = lanes_sum(n_act);
     if (!live || lane != 0) return;
-    float4 up = gxt[p];
+    const uint32_t i = idx[p];
+    const float4 u = gxo[i], v = gvo[i];
+    float4 up = make_float4(u.x + v.x / a.dt, u.y + v.y / a.dt, u.z + v.z / a.dt, 0.0f);
+    const float4 u2 = make_float4(-v.x / a.dt, -v.y / a.dt, -v.z / a.dt, 0.0f);
+    gxt[p] = up;
+    gx[p] = u2;
+    gws[p] = 0.0f;
     if (stab) {
-        const float4 u2 = gx[p];
         up.x += u2.x;
         up.y += u2.y;
         up.z += u2.z;
@@ -523,12 +540,21 @@ __global__ void k_adj_h(const PbdArgs a, int stab, const float4* __restrict__ Y,
 // (the next to reverse), whose h = upstream / n_p the particle's lanes
 // compute at the end from its updated gradients (stab_next: that pass is a
 // stabilization pass) into H_next, bitwise as k_adj_h would.
+// fin.idx (the last pass to reverse, the step's first): the gradients of the
+// step's inputs through the prediction, as k_adj_final, in original order.
+struct AdjFinal {
+    const uint32_t* idx;
+    float4* gx0;
+    float4* gv0;
+};
+
+template <bool kSingle>
 __global__ void k_adj_pass(const PbdArgs a, int stab, const float4* __restrict__ Y, const float4* __restrict__ XT,
                            const float4* __restrict__ XF, const float4* __restrict__ WS,
                            const uint32_t* __restrict__ nbr, const uint32_t* __restrict__ cnt,
                            const float4* __restrict__ H, float4* __restrict__ gx, float4* __restrict__ gxt,
                            float* __restrict__ gws, const AdjRecord rec, const float4* __restrict__ Y_next,
-                           int stab_next, float4* __restrict__ H_next)
+                           int stab_next, float4* __restrict__ H_next, const AdjFinal fin)
 {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t p = t / kAdjLanes;
@@ -537,11 +563,11 @@ __global__ void k_adj_pass(const PbdArgs a, int stab, const float4* __restrict__
     float acc[3] = {0.f, 0.f, 0.f}, accx[3] = {0.f, 0.f, 0.f}, gw = 0.0f;
     int n_next = 0;
     if (live && Y_next) {
-        const SceneDev& sc = a.scenes[a.lr_scene[p]];
+        const SceneDev& sc = kSingle ? a.scene0 : a.scenes[a.lr_scene[p]];
         n_next = lane_active_count(a, sc, Y_next, WS, nbr, p, (int)cnt[p], Y_next[p], WS[p].w, lane);
     }
     if (live) {
-        const SceneDev& sc = a.scenes[a.lr_scene[p]];
+        const SceneDev& sc = kSingle ? a.scene0 : a.scenes[a.lr_scene[p]];
         const float d0 = 2.0f * sc.r_low;
         const float4 yp = Y[p];
         const float wp = WS[p].w;
@@ -671,14 +697,21 @@ __global__ void k_adj_pass(const PbdArgs a, int stab, const float4* __restrict__
     float4 ngx = gx[p], ngxt = gxt[p];
     if (stab) {
         ngx = make_float4(ngx.x + acc[0], ngx.y + acc[1], ngx.z + acc[2], 0.0f);
-        gx[p] = ngx;
     } else {
         ngxt = make_float4(ngxt.x + acc[0], ngxt.y + acc[1], ngxt.z + acc[2], 0.0f);
-        gxt[p] = ngxt;
         ngx = make_float4(ngx.x + accx[0], ngx.y + accx[1], ngx.z + accx[2], 0.0f);
-        gx[p] = ngx;
     }
-    gws[p] += gw;
+    gw += gws[p];
+    if (fin.idx) {
+        const SceneDev& sc = kSingle ? a.scene0 : a.scenes[a.lr_scene[p]];
+        const uint32_t i = fin.idx[p];
+        fin.gx0[i] = make_float4(ngx.x + ngxt.x, ngx.y + ngxt.y, fmaf(gw * WS[p].w, sc.mass_k, ngx.z + ngxt.z), 0.0f);
+        fin.gv0[i] = make_float4(a.dt * ngxt.x, a.dt * ngxt.y, a.dt * ngxt.z, 0.0f);
+        return;
+    }
+    gx[p] = ngx;
+    if (!stab) gxt[p] = ngxt;
+    gws[p] = gw;
     if (Y_next) {   // h of the next pass to reverse, as k_adj_h
         float4 up = ngxt;
         if (stab_next) {
@@ -733,10 +766,10 @@ cudaError_t gs_launch_upsample_bwd_lr(cudaStream_t s, const SceneDev* scenes, co
 }
 
 cudaError_t gs_launch_scatter2(cudaStream_t s, const uint32_t* idx, const float4* a, const float4* b, float4* ao,
-                               float4* bo, int64_t n, int64_t* launches)
+                               float4* bo, int64_t n, int64_t* launches, int add)
 {
     if (n <= 0) return cudaSuccess;
-    k_scatter2<<<gs_blocks(n, 256), 256, 0, s>>>(idx, a, b, ao, bo, n);
+    k_scatter2<<<gs_blocks(n, 256), 256, 0, s>>>(idx, a, b, ao, bo, n, add);
     *launches += 1;
     return cudaGetLastError();
 }
@@ -751,11 +784,15 @@ cudaError_t gs_launch_adj_init(cudaStream_t s, int64_t n, const uint32_t* idx, c
 }
 
 cudaError_t gs_launch_adj_h(cudaStream_t s, const PbdArgs& a, int stab, const float4* Y, const float4* WS,
-                            const uint32_t* nbr, const uint32_t* cnt, const float4* gx, const float4* gxt, float4* H,
-                            int64_t* launches)
+                            const uint32_t* nbr, const uint32_t* cnt, const uint32_t* idx, const float4* gxo,
+                            const float4* gvo, float4* gx, float4* gxt, float* gws, float4* H, int64_t* launches)
 {
     if (a.n <= 0) return cudaSuccess;
-    k_adj_h<<<gs_blocks(a.n * kAdjLanes, 128), 128, 0, s>>>(a, stab, Y, WS, nbr, cnt, gx, gxt, H);
+    const unsigned nb = gs_blocks(a.n * kAdjLanes, 128);
+    if (a.n_scenes == 1)
+        k_adj_h<true><<<nb, 128, 0, s>>>(a, stab, Y, WS, nbr, cnt, idx, gxo, gvo, gx, gxt, gws, H);
+    else
+        k_adj_h<false><<<nb, 128, 0, s>>>(a, stab, Y, WS, nbr, cnt, idx, gxo, gvo, gx, gxt, gws, H);
     *launches += 1;
     return cudaGetLastError();
 }
@@ -763,11 +800,18 @@ cudaError_t gs_launch_adj_h(cudaStream_t s, const PbdArgs& a, int stab, const fl
 cudaError_t gs_launch_adj_pass(cudaStream_t s, const PbdArgs& a, int stab, const float4* Y, const float4* XT,
                                const float4* XF, const float4* WS, const uint32_t* nbr, const uint32_t* cnt,
                                const float4* H, float4* gx, float4* gxt, float* gws, int64_t* launches,
-                               const AdjRecord& rec, const float4* Y_next, int stab_next, float4* H_next)
+                               const AdjRecord& rec, const float4* Y_next, int stab_next, float4* H_next,
+                               const uint32_t* fin_idx, float4* gx0, float4* gv0)
 {
     if (a.n <= 0) return cudaSuccess;
-    k_adj_pass<<<gs_blocks(a.n * kAdjLanes, 128), 128, 0, s>>>(a, stab, Y, XT, XF, WS, nbr, cnt, H, gx, gxt, gws, rec,
-                                                                Y_next, stab_next, H_next);
+    const AdjFinal fin{fin_idx, gx0, gv0};
+    const unsigned nb = gs_blocks(a.n * kAdjLanes, 128);
+    if (a.n_scenes == 1)
+        k_adj_pass<true><<<nb, 128, 0, s>>>(a, stab, Y, XT, XF, WS, nbr, cnt, H, gx, gxt, gws, rec, Y_next, stab_next,
+                                            H_next, fin);
+    else
+        k_adj_pass<false><<<nb, 128, 0, s>>>(a, stab, Y, XT, XF, WS, nbr, cnt, H, gx, gxt, gws, rec, Y_next, stab_next,
+                                             H_next, fin);
     *launches += 1;
     return cudaGetLastError();
 }

@@ -11,6 +11,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <initializer_list>
 #include <new>
 
 #include "gs_internal.cuh"
@@ -180,6 +181,30 @@ __global__ void k_flag_solid(const float4* __restrict__ pos, int64_t n, int* err
 {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n && pos[i].w == 0.0f) atomicOr(err, bit);
+}
+
+// Several arrays in one launch (the functional entry points' copies of the
+// caller's buffers; blockIdx.y picks the array).
+constexpr int kMaxCopies = 6;
+struct CopyList {
+    const float4* src[kMaxCopies];
+    float4* dst[kMaxCopies];
+    int64_t n[kMaxCopies];
+};
+__global__ void __launch_bounds__(256) k_copy_list(const CopyList l)
+{
+    const float4* src = l.src[0];
+    float4* dst = l.dst[0];
+    int64_t n = l.n[0];
+#pragma unroll
+    for (int k = 1; k < kMaxCopies; ++k)   // no indexed parameter: it would go to local memory
+        if ((int)blockIdx.y == k) {
+            src = l.src[k];
+            dst = l.dst[k];
+            n = l.n[k];
+        }
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        dst[i] = src[i];
 }
 
 // Asynchronous writes of both fields of a kind, checked on the way: a copy
@@ -529,23 +554,73 @@ int create_impl(int S, const gs_scene* scenes, const float* r_low, const float* 
     return GS_OK;
 }
 
+struct Copy {
+    const void* src;
+    void* dst;
+    int64_t n;   // float4 records
+};
+
+// One launch for all copies instead of a driver call each (a call costs the
+// host 2 to 3 us, of which an LR step and its reverse made ten); a buffer that
+// is not 16-byte aligned goes by itself.
+int copy_all(gs_ctx* c, std::initializer_list<Copy> list)
+{
+    CopyList l = {};
+    int k = 0;
+    int64_t most = 0;
+    for (const Copy& x : list) {
+        if (x.n <= 0) continue;
+        if ((((uintptr_t)x.src | (uintptr_t)x.dst) & 15u) || k == kMaxCopies) {
+            CK(cudaMemcpyAsync(x.dst, x.src, (size_t)x.n * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream),
+               "copy");
+            continue;
+        }
+        l.src[k] = (const float4*)x.src;
+        l.dst[k] = (float4*)x.dst;
+        l.n[k++] = x.n;
+        most = std::max(most, x.n);
+    }
+    if (k == 0) return GS_OK;
+    const unsigned nb = std::min(gs_blocks(most, 256), (unsigned)(8 * std::max(c->sm_count, 1)));
+    k_copy_list<<<dim3(nb, (unsigned)k), 256, 0, c->stream>>>(l);
+    c->launches += 1;
+    CK(cudaGetLastError(), "copy");
+    return GS_OK;
+}
+
 // The key buffer that holds the sorted HR keys after a reorder.
 uint32_t* hr_sorted_after_resort(const gs_ctx* c)
 {
     return c->hr_counting ? c->hr_keys[1] : c->hr_keys[((c->hr_key_bits + 7) / 8) & 1];   // where the radix passes end
 }
 
-int resort_high_impl(gs_ctx* c)
+// The reverse modes differentiate grains only: LR positions (device memory,
+// n of them) holding particles of infinite mass raise a device error bit,
+// reported as GS_ERR_STATE by the next blocking call (no wait here).
+int flag_solid(gs_ctx* c, const float4* pos, int64_t n)
+{
+    if (n <= 0) return GS_OK;
+    k_flag_solid<<<gs_blocks(n, 256), 256, 0, c->stream>>>(pos, n, c->d_err,
+                                                            GS_DEVERR_SOLID_REVERSE);
+    c->launches += 1;
+    CK(cudaGetLastError(), "flag");
+    return GS_OK;
+}
+
+// src_pos / src_vel (one-scene contexts): the HR state to sort, in original
+// order, instead of the context's own.
+int resort_high_impl(gs_ctx* c, const float4* src_pos = nullptr, const float4* src_vel = nullptr)
 {
     const int64_t MS = c->hr_slots;
     if (MS == 0) return GS_OK;
     Timed t(c, GS_TIMER_RESORT);
     const int cur = c->hr_cur;
+    const float4* pos = src_pos ? src_pos : c->hr_pos[cur];   // padding slots' positions are not read
     int which = 0;
     if (c->hr_counting) {
         CK(gs_cs_clear(c->stream, c->hr_bin_start, c->hr_bins, 1), "clear counts");
-        CK(gs_launch_scene_keys(c->stream, c->hr_pos[cur], MS, c->d_scenes, c->hr_scene, 1, c->hr_keys[0],
-                                c->hr_vals[0], &c->launches, c->hr_bin_start),
+        CK(gs_launch_scene_keys(c->stream, pos, MS, c->d_scenes, c->hr_scene, 1, c->hr_keys[0], c->hr_vals[0],
+                                &c->launches, c->hr_bin_start),
            "keys");
         CsExtras ex;
         ex.big_list = c->hr_big;
@@ -558,15 +633,20 @@ int resort_high_impl(gs_ctx* c)
            "counting sort");
         which = 1;
     } else {
-        CK(gs_launch_scene_keys(c->stream, c->hr_pos[cur], MS, c->d_scenes, c->hr_scene, 1, c->hr_keys[0],
-                                c->hr_vals[0], &c->launches),
+        CK(gs_launch_scene_keys(c->stream, pos, MS, c->d_scenes, c->hr_scene, 1, c->hr_keys[0], c->hr_vals[0],
+                                &c->launches),
            "keys");
         CK(gs_radix_sort(c->stream, c->hr_keys, c->hr_vals, &which, c->sort_hist, MS, c->hr_key_bits, &c->launches),
            "radix sort");
     }
-    CK(gs_launch_gather2(c->stream, c->hr_vals[which], c->hr_pos[cur], c->hr_vel[cur], c->hr_pos[cur ^ 1],
-                         c->hr_vel[cur ^ 1], MS, &c->launches),
-       "permute");
+    if (src_pos)
+        CK(gs_launch_gather2_ids(c->stream, c->hr_vals[which], src_pos, src_vel, c->hr_pos[cur ^ 1],
+                                 c->hr_vel[cur ^ 1], MS, c->n_high, &c->launches),
+           "permute");
+    else
+        CK(gs_launch_gather2(c->stream, c->hr_vals[which], c->hr_pos[cur], c->hr_vel[cur], c->hr_pos[cur ^ 1],
+                             c->hr_vel[cur ^ 1], MS, &c->launches),
+           "permute");
     c->hr_sorted_keys = c->hr_keys[which];
     c->hr_keys_valid = true;
     c->hr_cur = cur ^ 1;
@@ -574,9 +654,14 @@ int resort_high_impl(gs_ctx* c)
     return GS_OK;
 }
 
-int bin_low_impl(gs_ctx* c)
+// The LR state lx / lv (default: the context's) into the upsampling view.
+// reverse: for a reverse mode, which refuses particles of infinite mass
+// (GS_DEVERR_SOLID_REVERSE) and starts from cleared gradients.
+int bin_low_impl(gs_ctx* c, const float4* lx = nullptr, const float4* lv = nullptr, bool reverse = false)
 {
     Timed t(c, GS_TIMER_BIN_LOW);
+    const float4* pos = lx ? lx : c->lr_pos;
+    const float4* vel = lv ? lv : c->lr_vel;
     // counting sort by cell; its last stage copies pos and vel into cell order
     // the word after the cell starts flags LR particles of infinite mass or
     // of rigid bodies for the gather (the binning reads every position
@@ -586,21 +671,30 @@ int bin_low_impl(gs_ctx* c)
     ex.ga_solid = body;
     unsigned* flag = c->lr_cell_start + c->n_cell_total + 1;
     if (c->bins.count) {
-        CK(gs_bins_keys(c->stream, c->bins, c->lr_pos, c->n_low, c->d_scenes, c->lr_scene, c->lr_keys[0], &c->launches,
-                        1, body),
+        if (reverse) {
+            ex.zero_a = c->gXs;
+            ex.zero_b = c->gVs;
+        }
+        CK(gs_bins_keys(c->stream, c->bins, pos, c->n_low, c->d_scenes, c->lr_scene, c->lr_keys[0], &c->launches, 1,
+                        body, reverse ? c->d_err : nullptr),
            "cell keys");
         CK(gs_bins_finish(c->stream, c->bins, c->n_low, c->n_cell_total, c->lr_keys[0], c->lr_keys[1], c->lr_vals[1],
-                          c->lr_cell_start, c->lr_pos, c->lr_vel, c->lr_spos, c->lr_svel, &c->launches, ex, flag,
-                          c->d_work),
+                          c->lr_cell_start, pos, vel, c->lr_spos, c->lr_svel, &c->launches, ex, flag, c->d_work),
            "bin by cell");
     } else {
+        if (reverse && c->n_low > 0) {
+            int st = flag_solid(c, pos, c->n_low);
+            if (st) return st;
+            CK(cudaMemsetAsync(c->gXs, 0, c->n_low * sizeof(float4), c->stream), "clear");
+            CK(cudaMemsetAsync(c->gVs, 0, c->n_low * sizeof(float4), c->stream), "clear");
+        }
         CK(gs_cs_clear(c->stream, c->lr_cell_start, c->n_cell_total, 1), "clear counts");
-        CK(gs_cs_keys(c->stream, c->lr_pos, c->n_low, c->d_scenes, c->lr_scene, c->lr_keys[0], c->lr_vals[0],
+        CK(gs_cs_keys(c->stream, pos, c->n_low, c->d_scenes, c->lr_scene, c->lr_keys[0], c->lr_vals[0],
                       c->lr_cell_start, &c->launches, flag, body),
            "cell keys");
         CK(gs_cs_finish(c->stream, c->n_low, c->n_cell_total, c->lr_keys[0], c->lr_vals[0], c->lr_keys[1],
-                        c->lr_vals[1], c->lr_cell_start, c->scan_aux, c->lr_pos, c->lr_vel, c->lr_spos, c->lr_svel,
-                        &c->launches, ex),
+                        c->lr_vals[1], c->lr_cell_start, c->scan_aux, pos, vel, c->lr_spos, c->lr_svel, &c->launches,
+                        ex),
            "bin by cell");
     }
     c->lr_sorted_keys = c->lr_keys[1];
@@ -617,6 +711,7 @@ UpsampleArgs upsample_args(const gs_ctx* c, float dt, const float4* in_pos, cons
     u.hr_vel = in_vel;
     u.out_pos = out_pos;
     u.out_vel = out_vel;
+    u.id_pos = u.id_vel = nullptr;
     u.lr_spos = c->lr_spos;
     u.lr_svel = c->lr_svel;
     u.cell_start = c->lr_cell_start;
@@ -677,25 +772,40 @@ int upsample_impl(gs_ctx* c, float dt)
     return GS_OK;
 }
 
+// An LR step's input and output state (original order; may be the same
+// buffers).
+struct StepIo {
+    const float4 *x, *v;
+    float4 *xo, *vo;
+};
+
 // The beginning of an LR step: prediction fused with the counting stage of
 // the binning of x~, the binning (whose last stage copies x and x~ into cell
-// order, X and XT; cell starts in `start`), and the candidate lists.
-int step_begin(gs_ctx* c, const PbdArgs& a, float4* X, float4* XT, uint32_t* start, uint32_t* nbr, uint32_t* cnt)
+// order, X and XT; cell starts in `start`, the particle of each slot in
+// `idx`), and the candidate lists.  reverse: particles of infinite mass raise
+// GS_DEVERR_SOLID_REVERSE.
+int step_begin(gs_ctx* c, const PbdArgs& a, const StepIo& io, float4* X, float4* XT, uint32_t* start, uint32_t* nbr,
+               uint32_t* cnt, uint32_t* idx, bool reverse)
 {
     const int64_t N = c->n_low;
     if (c->bins.count) {
-        CK(gs_launch_predict_bins(c->stream, a, c->bins, c->lr_pos, c->lr_vel, c->lr_xt, c->lr_keys[0], &c->launches),
+        CK(gs_launch_predict_bins(c->stream, a, c->bins, io.x, io.v, c->lr_xt, c->lr_keys[0],
+                                  reverse ? c->d_err : nullptr, &c->launches),
            "predict");
-        CK(gs_bins_finish(c->stream, c->bins, N, c->n_cell_total, c->lr_keys[0], c->lr_keys[1], c->lr_vals[1], start,
-                          c->lr_xt, c->lr_pos, XT, X, &c->launches, step_extras(c, a)),
+        CK(gs_bins_finish(c->stream, c->bins, N, c->n_cell_total, c->lr_keys[0], c->lr_keys[1], idx, start, c->lr_xt,
+                          io.x, XT, X, &c->launches, step_extras(c, a)),
            "bin by cell");
     } else {
+        if (reverse) {
+            int st = flag_solid(c, io.x, N);
+            if (st) return st;
+        }
         CK(gs_cs_clear(c->stream, start, c->n_cell_total), "clear counts");
-        CK(gs_launch_predict_keys(c->stream, a, c->lr_pos, c->lr_vel, c->lr_xt, c->lr_keys[0], c->lr_vals[0], start,
+        CK(gs_launch_predict_keys(c->stream, a, io.x, io.v, c->lr_xt, c->lr_keys[0], c->lr_vals[0], start,
                                   &c->launches),
            "predict");
-        CK(gs_cs_finish(c->stream, N, c->n_cell_total, c->lr_keys[0], c->lr_vals[0], c->lr_keys[1], c->lr_vals[1],
-                        start, c->scan_aux, c->lr_xt, c->lr_pos, XT, X, &c->launches, step_extras(c, a)),
+        CK(gs_cs_finish(c->stream, N, c->n_cell_total, c->lr_keys[0], c->lr_vals[0], c->lr_keys[1], idx, start,
+                        c->scan_aux, c->lr_xt, io.x, XT, X, &c->launches, step_extras(c, a)),
            "bin by cell");
     }
     c->lr_sorted_keys = c->lr_keys[1];
@@ -705,16 +815,18 @@ int step_begin(gs_ctx* c, const PbdArgs& a, float4* X, float4* XT, uint32_t* sta
     return GS_OK;
 }
 
+// One LR step from io.x, io.v into io.xo, io.vo.
 // dt_dev (adaptive frames): the step length is read from device memory
 // instead of dt; rate: the finalize's atomic max of |v| / (2 r_LR).
-int step_low_impl(gs_ctx* c, float dt, int iters, const float* dt_dev = nullptr, unsigned* rate = nullptr)
+int step_low_io(gs_ctx* c, const StepIo& io, float dt, int iters, const float* dt_dev = nullptr,
+                unsigned* rate = nullptr)
 {
     const int64_t N = c->n_low;
     if (N == 0) return GS_OK;
     Timed t(c, GS_TIMER_STEP_LOW);
     PbdArgs a = pbd_args(c, dt);
     a.dt_dev = dt_dev;
-    int st = step_begin(c, a, c->s_x[0], c->s_xt[0], c->step_cell_start, c->nbr, c->nbr_cnt);
+    int st = step_begin(c, a, io, c->s_x[0], c->s_xt[0], c->step_cell_start, c->nbr, c->nbr_cnt, c->lr_vals[1], false);
     if (st) return st;
     int bx = 0, bt = 0;   // buffers holding the current x and xt
     if (c->use_solver && c->solve_blocks > 0 && c->n_bodies == 0) {
@@ -736,8 +848,8 @@ int step_low_impl(gs_ctx* c, float dt, int iters, const float* dt_dev = nullptr,
                                         c->s_xt[bt], c->lr_xo, c->body_xf, &c->launches),
                    "body transforms");
             CK(gs_launch_pass(c->stream, a, stab, c->s_x[bx], c->s_xt[bt], c->s_x[bx ^ 1], c->s_xt[bt ^ 1], c->nbr,
-                              c->nbr_cnt, &c->launches, last ? c->lr_sorted_idx : nullptr,
-                              last ? c->lr_pos : nullptr, last ? c->lr_vel : nullptr, last ? rate : nullptr),
+                              c->nbr_cnt, &c->launches, last ? c->lr_vals[1] : nullptr, last ? io.xo : nullptr,
+                              last ? io.vo : nullptr, io.x, last ? rate : nullptr),
                "pass");
             bt ^= 1;
             if (stab) bx ^= 1;
@@ -747,11 +859,17 @@ int step_low_impl(gs_ctx* c, float dt, int iters, const float* dt_dev = nullptr,
             return GS_OK;
         }
     }
-    CK(gs_launch_finalize(c->stream, a, c->lr_sorted_idx, c->s_x[bx], c->s_xt[bt], c->lr_pos, c->lr_vel,
-                          &c->launches, rate),
+    CK(gs_launch_finalize(c->stream, a, c->lr_vals[1], c->s_x[bx], c->s_xt[bt], io.xo, io.vo, io.x, &c->launches,
+                          rate),
        "finalize");
     c->lr_binned = false;   // the binning above is of the predicted positions
     return GS_OK;
+}
+
+// One LR step of the context's own state.
+int step_low_impl(gs_ctx* c, float dt, int iters, const float* dt_dev = nullptr, unsigned* rate = nullptr)
+{
+    return step_low_io(c, StepIo{c->lr_pos, c->lr_vel, c->lr_pos, c->lr_vel}, dt, iters, dt_dev, rate);
 }
 
 // HR frames of a context restricted to a slab: a reorder reads the whole
@@ -2089,28 +2207,29 @@ static int ensure_fscratch(gs_ctx* c)
     return GS_OK;
 }
 
-// The HR frame on copies: HR state in from fscratch[0..2), out to
-// fscratch[2..4) (original order); the internal order is reset and sorted.
-static int upsample_fwd_seq(gs_ctx* c, float dt)
+// The HR frame of a one-scene context from the LR state lx, lv and the HR
+// state hx, hv into hxo, hvo (all in original order; in place allowed): the
+// HR state is sorted from the caller's order and the gather leaves the
+// results in it.
+static int upsample_fwd_seq(gs_ctx* c, const float4* lx, const float4* lv, const float4* hx, const float4* hv,
+                            float4* hxo, float4* hvo, float dt)
 {
-    const int64_t M = c->n_high;
-    float4* F = c->fscratch;
-    int cur = c->hr_cur;
-    CK(launch_hr_load(c, F, c->hr_pos[cur], 1), "load");
-    CK(launch_hr_load(c, F + M, c->hr_vel[cur], 0), "load");
-    c->hr_identity = true;
-    int st = resort_high_impl(c);
+    int st = resort_high_impl(c, hx, hv);
     if (st) return st;
-    st = bin_low_impl(c);
+    st = bin_low_impl(c, lx, lv);
     if (st) return st;
-    cur = c->hr_cur;
+    const int cur = c->hr_cur;
     UpsampleArgs u = upsample_args(c, dt, c->hr_pos[cur], c->hr_vel[cur], c->hr_pos[cur], c->hr_vel[cur]);
+    u.id_pos = hxo;
+    u.id_vel = hvo;
     CK(gs_launch_upsample(c->stream, u, c->tune_warps, c->tune_blocks_per_sm, c->sm_count, &c->launches), "upsample");
-    CK(gs_launch_unpermute2(c->stream, c->hr_pos[cur], c->hr_vel[cur], c->hr_scene, F + 2 * M, F + 3 * M,
-                            c->hr_slots, M, c->d_err, &c->launches),
-       "unpermute");
     return GS_OK;
 }
+
+// From so many HR particles on the functional frame's kernels take longer
+// than their launches, so it runs on the caller's buffers directly instead of
+// as a graph between copies of them (500,000 HR: 80 us a call against 88).
+constexpr int64_t kDirectFrame = 262144;
 
 int gs_upsample_forward(gs_ctx* c, const float* lr_pos, const float* lr_vel, const float* hr_pos_in,
                         const float* hr_vel_in, float* hr_pos_out, float* hr_vel_out, float dt)
@@ -2124,52 +2243,37 @@ int gs_upsample_forward(gs_ctx* c, const float* lr_pos, const float* lr_vel, con
     const int64_t N = c->n_low, M = c->n_high;
     if ((N > 0 && (!lr_pos || !lr_vel)) || (M > 0 && (!hr_pos_in || !hr_vel_in || !hr_pos_out || !hr_vel_out)))
         return fail(c, GS_ERR_ARG, "null buffer");
-    if (N) {
-        CK(cudaMemcpyAsync(c->lr_pos, lr_pos, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-        CK(cudaMemcpyAsync(c->lr_vel, lr_vel, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    }
     c->lr_binned = false;
-    if (M == 0) return GS_OK;
+    if (M == 0) return copy_all(c, {{lr_pos, c->lr_pos, N}, {lr_vel, c->lr_vel, N}});
+    const bool aligned =
+        (((uintptr_t)hr_pos_in | (uintptr_t)hr_vel_in | (uintptr_t)hr_pos_out | (uintptr_t)hr_vel_out) & 15u) == 0;
+    if (M >= kDirectFrame && aligned) {
+        st = copy_all(c, {{lr_pos, c->lr_pos, N}, {lr_vel, c->lr_vel, N}});
+        if (st) return st;
+        return upsample_fwd_seq(c, c->lr_pos, c->lr_vel, (const float4*)hr_pos_in, (const float4*)hr_vel_in,
+                                (float4*)hr_pos_out, (float4*)hr_vel_out, dt);
+    }
     st = ensure_fscratch(c);
     if (st) return st;
     float4* F = c->fscratch;
-    CK(cudaMemcpyAsync(F, hr_pos_in, M * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    CK(cudaMemcpyAsync(F + M, hr_vel_in, M * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    st = replay_or_run(c, step_key(c, 'u', dt, 0), [&] { return upsample_fwd_seq(c, dt); });
+    st = copy_all(c, {{lr_pos, c->lr_pos, N}, {lr_vel, c->lr_vel, N}, {hr_pos_in, F, M}, {hr_vel_in, F + M, M}});
     if (st) return st;
-    CK(cudaMemcpyAsync(hr_pos_out, F + 2 * M, M * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    CK(cudaMemcpyAsync(hr_vel_out, F + 3 * M, M * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    return GS_OK;
+    st = replay_or_run(c, step_key(c, 'u', dt, 0), [&] {
+        return upsample_fwd_seq(c, c->lr_pos, c->lr_vel, F, F + M, F + 2 * M, F + 3 * M, dt);
+    });
+    if (st) return st;
+    return copy_all(c, {{F + 2 * M, hr_pos_out, M}, {F + 3 * M, hr_vel_out, M}});
 }
 
-// The reverse modes differentiate grains only: LR positions (device memory,
-// n of them) holding particles of infinite mass raise a device error bit,
-// reported as GS_ERR_STATE by the next blocking call (no wait here).
-static int flag_solid(gs_ctx* c, const float* pos, int64_t n)
-{
-    if (n <= 0) return GS_OK;
-    k_flag_solid<<<gs_blocks(n, 256), 256, 0, c->stream>>>((const float4*)pos, n, c->d_err,
-                                                            GS_DEVERR_SOLID_REVERSE);
-    c->launches += 1;
-    CK(cudaGetLastError(), "flag");
-    return GS_OK;
-}
-
-// The reverse HR frame on copies: HR state and dL/d outputs in from
-// fscratch[0..4), dL/d HR inputs out to fscratch[4..6), dL/d LR inputs out
-// to the two n_low blocks after them (original order).
-static int upsample_bwd_seq(gs_ctx* c, float dt)
+// The reverse HR frame of a one-scene context (all buffers in original
+// order): dL/d HR inputs into ghx, ghv, dL/d LR inputs into glx, glv (add: on
+// top of what they hold).
+static int upsample_bwd_seq(gs_ctx* c, const float4* lx, const float4* lv, const float4* hx, const float4* hv,
+                            const float4* gxo, const float4* gvo, float4* glx, float4* glv, float4* ghx, float4* ghv,
+                            float dt, int add)
 {
     const int64_t N = c->n_low, M = c->n_high;
-    float4* F = c->fscratch;
-    float4* G = F + 6 * M;
-    int st = flag_solid(c, (const float*)c->lr_pos, N);
-    if (st) return st;
-    if (N && !c->det_bwd) {
-        CK(cudaMemsetAsync(c->gXs, 0, N * sizeof(float4), c->stream), "clear");
-        CK(cudaMemsetAsync(c->gVs, 0, N * sizeof(float4), c->stream), "clear");
-    }
-    st = bin_low_impl(c);
+    int st = bin_low_impl(c, lx, lv, true);
     if (st) return st;
     if (c->det_bwd) {   // HR binned by the LR cells, for the LR side's gather
         // (its cells hold dozens of HR particles: ordered over the whole grid
@@ -2177,7 +2281,7 @@ static int upsample_bwd_seq(gs_ctx* c, float dt)
         uint32_t* big_count = c->det_big + M / 33 + 1;
         CK(gs_cs_clear(c->stream, c->step_cell_start, c->n_cell_total), "clear counts");
         CK(cudaMemsetAsync(big_count, 0, sizeof(uint32_t), c->stream), "clear list");
-        CK(gs_cs_keys(c->stream, F, M, c->d_scenes, c->hr_scene, c->hr_keys[0], c->hr_vals[0], c->step_cell_start,
+        CK(gs_cs_keys(c->stream, hx, M, c->d_scenes, c->hr_scene, c->hr_keys[0], c->hr_vals[0], c->step_cell_start,
                       &c->launches),
            "HR cell keys");
         CsExtras ex;
@@ -2190,8 +2294,8 @@ static int upsample_bwd_seq(gs_ctx* c, float dt)
                         c->step_cell_start, c->scan_aux, nullptr, nullptr, nullptr, nullptr, &c->launches, ex),
            "bin HR by LR cell");
     }
-    CK(gs_launch_upsample_bwd(c->stream, c->d_scenes, c->d_sdf, c->lr_spos, c->lr_svel, c->lr_cell_start, F, F + M,
-                              F + 2 * M, F + 3 * M, F + 4 * M, F + 5 * M, c->gXs, c->gVs, M, dt, &c->launches,
+    CK(gs_launch_upsample_bwd(c->stream, c->d_scenes, c->d_sdf, c->lr_spos, c->lr_svel, c->lr_cell_start, hx, hv,
+                              gxo, gvo, ghx, ghv, c->gXs, c->gVs, M, dt, &c->launches,
                               c->rec_hr, c->lr_sorted_idx, c->det_bwd ? c->det_coef : nullptr,
                               c->det_bwd ? c->hr_vals[1] : nullptr, c->det_bwd ? c->det_coef + 2 * M : nullptr),
        "upsample backward");
@@ -2200,7 +2304,7 @@ static int upsample_bwd_seq(gs_ctx* c, float dt)
                                      c->det_coef + 2 * M, c->step_cell_start, c->det_coef, c->gXs, c->gVs, N,
                                      &c->launches),
            "upsample backward, LR side");
-    CK(gs_launch_scatter2(c->stream, c->lr_sorted_idx, c->gXs, c->gVs, G, G + N, N, &c->launches), "scatter");
+    CK(gs_launch_scatter2(c->stream, c->lr_sorted_idx, c->gXs, c->gVs, glx, glv, N, &c->launches, add), "scatter");
     return GS_OK;
 }
 
@@ -2223,26 +2327,22 @@ int gs_upsample_backward(gs_ctx* c, const float* lr_pos, const float* lr_vel, co
     if (st) return st;
     float4* F = c->fscratch;
     float4* G = F + 6 * M;
-    if (N) {
-        CK(cudaMemcpyAsync(c->lr_pos, lr_pos, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-        CK(cudaMemcpyAsync(c->lr_vel, lr_vel, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    }
-    if (M) {
-        const void* in[4] = {hr_pos_in, hr_vel_in, g_hr_pos_out, g_hr_vel_out};
-        for (int k = 0; k < 4; ++k)
-            CK(cudaMemcpyAsync(F + k * M, in[k], M * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    }
-    st = replay_or_run(c, step_key(c, 'v', dt, 0), [&] { return upsample_bwd_seq(c, dt); });
+    st = copy_all(c, {{lr_pos, c->lr_pos, N},
+                      {lr_vel, c->lr_vel, N},
+                      {hr_pos_in, F, M},
+                      {hr_vel_in, F + M, M},
+                      {g_hr_pos_out, F + 2 * M, M},
+                      {g_hr_vel_out, F + 3 * M, M}});
     if (st) return st;
-    if (M) {
-        CK(cudaMemcpyAsync(g_hr_pos_in, F + 4 * M, M * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-        CK(cudaMemcpyAsync(g_hr_vel_in, F + 5 * M, M * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    }
-    if (N) {
-        CK(cudaMemcpyAsync(g_lr_pos, G, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-        CK(cudaMemcpyAsync(g_lr_vel, G + N, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    }
-    return GS_OK;
+    st = replay_or_run(c, step_key(c, 'v', dt, 0), [&] {
+        return upsample_bwd_seq(c, c->lr_pos, c->lr_vel, F, F + M, F + 2 * M, F + 3 * M, G, G + N, F + 4 * M,
+                                F + 5 * M, dt, 0);
+    });
+    if (st) return st;
+    return copy_all(c, {{F + 4 * M, g_hr_pos_in, M},
+                        {F + 5 * M, g_hr_vel_in, M},
+                        {G, g_lr_pos, N},
+                        {G + N, g_lr_vel, N}});
 }
 
 int gs_step_low_forward(gs_ctx* c, const float* x_in, const float* v_in, float* x_out, float* v_out, float dt,
@@ -2257,16 +2357,14 @@ int gs_step_low_forward(gs_ctx* c, const float* x_in, const float* v_in, float* 
     const int64_t N = c->n_low;
     if (N == 0) return GS_OK;
     if (!x_in || !v_in || !x_out || !v_out) return fail(c, GS_ERR_ARG, "null buffer");
-    CK(cudaMemcpyAsync(c->lr_pos, x_in, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    CK(cudaMemcpyAsync(c->lr_vel, v_in, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
+    st = copy_all(c, {{x_in, c->lr_pos, N}, {v_in, c->lr_vel, N}});
+    if (st) return st;
     st = replay_or_run(c, step_key(c, 'f', dt, iters), [&] { return step_low_impl(c, dt, iters); });
     if (st) return st;
     c->lr_sorted_keys = c->lr_keys[1];   // the host state the step leaves, replayed or not
     c->lr_sorted_idx = c->lr_vals[1];
     c->lr_binned = false;
-    CK(cudaMemcpyAsync(x_out, c->lr_pos, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    CK(cudaMemcpyAsync(v_out, c->lr_vel, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    return GS_OK;
+    return copy_all(c, {{c->lr_pos, x_out, N}, {c->lr_vel, v_out, N}});
 }
 
 void gs_set_alloc_failure(long long after)
@@ -2327,9 +2425,11 @@ static int ensure_snapshots(gs_ctx* c, int total)
 
 static int step_low_reverse(gs_ctx* c, float dt, int iters);
 static int step_low_record(gs_ctx* c, float dt, int iters);
-static int step_low_record_into(gs_ctx* c, float dt, int iters, float4* X, float4* XT, uint32_t* nbr, uint32_t* cnt);
+static int step_low_record_into(gs_ctx* c, const StepIo& io, float dt, int iters, float4* X, float4* XT,
+                                uint32_t* nbr, uint32_t* cnt, uint32_t* idx, bool final_state);
 static int step_low_reverse_from(gs_ctx* c, float dt, int iters, const float4* X, const float4* XT,
-                                 const uint32_t* nbr, const uint32_t* cnt, const uint32_t* idx);
+                                 const uint32_t* nbr, const uint32_t* cnt, const uint32_t* idx, const float4* gxo,
+                                 const float4* gvo, float4* gx0, float4* gv0);
 
 int gs_step_low_trace(gs_ctx* c, const float* x_in, const float* v_in, float dt, int iters, float* x_trace,
                       float* xt_trace, int n_records)
@@ -2349,8 +2449,8 @@ int gs_step_low_trace(gs_ctx* c, const float* x_in, const float* v_in, float dt,
     if (!x_in || !v_in || !x_trace || !xt_trace) return fail(c, GS_ERR_ARG, "null buffer");
     st = ensure_snapshots(c, total);
     if (st) return st;
-    CK(cudaMemcpyAsync(c->lr_pos, x_in, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    CK(cudaMemcpyAsync(c->lr_vel, v_in, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
+    st = copy_all(c, {{x_in, c->lr_pos, N}, {v_in, c->lr_vel, N}});
+    if (st) return st;
     st = step_low_record(c, dt, iters);
     if (st) return st;
     float4* xo = reinterpret_cast<float4*>(x_trace);
@@ -2434,20 +2534,11 @@ static uint64_t tape_key(const gs_ctx* c, char kind, float dt, int iters, int sl
     return (step_key(c, kind, dt, iters) ^ (0x9e3779b97f4a7c15ull * (uint64_t)(slot + 1))) * 0x100000001b3ull;
 }
 
-// The recorded forward into tape slot t, then the step's finalize from the
-// last snapshots (v = (x~ - x) / dt, x = x~, original order).
-static int step_low_tape_forward(gs_ctx* c, gs_ctx::StepTape& t, float dt, int iters)
+// The recorded forward of io into tape slot t.
+static int step_low_tape_forward(gs_ctx* c, const StepIo& io, gs_ctx::StepTape& t, float dt, int iters)
 {
-    const int64_t N = c->n_low;
-    const int total = c->n_stab + iters;
-    int st = step_low_record_into(c, dt, iters, t.X, t.XT, t.nbr, t.cnt);
+    int st = step_low_record_into(c, io, dt, iters, t.X, t.XT, t.nbr, t.cnt, t.idx, true);
     if (st) return st;
-    CK(cudaMemcpyAsync(t.idx, c->lr_sorted_idx, N * sizeof(uint32_t), cudaMemcpyDeviceToDevice, c->stream),
-       "keep the cell order");
-    const PbdArgs a = pbd_args(c, dt);
-    CK(gs_launch_finalize(c->stream, a, t.idx, t.X + (size_t)std::min(total, c->n_stab) * N, t.XT + (size_t)total * N,
-                          c->lr_pos, c->lr_vel, &c->launches, nullptr),
-       "finalize");
     c->lr_binned = false;
     return GS_OK;
 }
@@ -2473,12 +2564,14 @@ int gs_step_low_forward_taped(gs_ctx* c, const float* x_in, const float* v_in, f
     const int slot = c->tape_next;
     gs_ctx::StepTape& t = c->tapes[(size_t)slot];
     t.tag = -1;   // until the step below is enqueued
-    CK(cudaMemcpyAsync(c->lr_pos, x_in, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    CK(cudaMemcpyAsync(c->lr_vel, v_in, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    st = replay_or_run(c, tape_key(c, 'F', dt, iters, slot), [&] { return step_low_tape_forward(c, t, dt, iters); });
+    st = copy_all(c, {{x_in, c->lr_pos, N}, {v_in, c->lr_vel, N}});
     if (st) return st;
-    CK(cudaMemcpyAsync(x_out, c->lr_pos, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    CK(cudaMemcpyAsync(v_out, c->lr_vel, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
+    st = replay_or_run(c, tape_key(c, 'F', dt, iters, slot), [&] {
+        return step_low_tape_forward(c, StepIo{c->lr_pos, c->lr_vel, c->lr_pos, c->lr_vel}, t, dt, iters);
+    });
+    if (st) return st;
+    st = copy_all(c, {{c->lr_pos, x_out, N}, {c->lr_vel, v_out, N}});
+    if (st) return st;
     t.tag = tag;
     t.serial = c->tape_serial++;
     t.dt = dt;
@@ -2508,15 +2601,14 @@ int gs_step_low_backward_taped(gs_ctx* c, int64_t tag, const float* g_x_out, con
                     c->rec_max_passes);
     st = ensure_adjoint_buffers(c);
     if (st) return st;
-    CK(cudaMemcpyAsync(c->adj_io, g_x_out, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    CK(cudaMemcpyAsync(c->adj_io + N, g_v_out, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
+    st = copy_all(c, {{g_x_out, c->adj_io, N}, {g_v_out, c->adj_io + N, N}});
+    if (st) return st;
     st = replay_or_run(c, tape_key(c, 'B', t.dt, t.iters, slot), [&] {
-        return step_low_reverse_from(c, t.dt, t.iters, t.X, t.XT, t.nbr, t.cnt, t.idx);
+        return step_low_reverse_from(c, t.dt, t.iters, t.X, t.XT, t.nbr, t.cnt, t.idx, c->adj_io, c->adj_io + N,
+                                     c->adj_io + 2 * N, c->adj_io + 3 * N);
     });
     if (st) return st;
-    CK(cudaMemcpyAsync(g_x_in, c->adj_io + 2 * N, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    CK(cudaMemcpyAsync(g_v_in, c->adj_io + 3 * N, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    return GS_OK;
+    return copy_all(c, {{c->adj_io + 2 * N, g_x_in, N}, {c->adj_io + 3 * N, g_v_in, N}});
 }
 
 int gs_step_low_backward(gs_ctx* c, const float* x_in, const float* v_in, const float* g_x_out, const float* g_v_out,
@@ -2542,69 +2634,72 @@ int gs_step_low_backward(gs_ctx* c, const float* x_in, const float* v_in, const 
     if (st) return st;
     // the caller's buffers in; the rest runs on the context's own buffers
     // (replayed as a graph when graphs are enabled)
-    CK(cudaMemcpyAsync(c->lr_pos, x_in, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    CK(cudaMemcpyAsync(c->lr_vel, v_in, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    CK(cudaMemcpyAsync(c->adj_io, g_x_out, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    CK(cudaMemcpyAsync(c->adj_io + N, g_v_out, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
+    st = copy_all(c, {{x_in, c->lr_pos, N}, {v_in, c->lr_vel, N}, {g_x_out, c->adj_io, N}, {g_v_out, c->adj_io + N, N}});
+    if (st) return st;
     st = replay_or_run(c, step_key(c, 'b', dt, iters), [&] { return step_low_reverse(c, dt, iters); });
     if (st) return st;
-    CK(cudaMemcpyAsync(g_x_in, c->adj_io + 2 * N, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
-    CK(cudaMemcpyAsync(g_v_in, c->adj_io + 3 * N, N * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream), "copy");
+    st = copy_all(c, {{c->adj_io + 2 * N, g_x_in, N}, {c->adj_io + 3 * N, g_v_in, N}});
+    if (st) return st;
     c->lr_sorted_keys = c->lr_keys[1];   // the host state the reverse step leaves
     c->lr_sorted_idx = c->lr_vals[1];
     c->lr_binned = false;
     return GS_OK;
 }
 
-// The LR step on the context's buffers (from lr_pos, lr_vel) keeping what
-// every pass evaluates on, in cell order: x~ before pass it is
-// snap_xt[it], x before stabilization pass it is snap[it] (after the
-// stabilization passes snap[n_stab] throughout); snap_xt[total] holds the
-// step's final x~.  The passes read and write the snapshot buffers
-// themselves.
-// The recording into given buffers (the snapshots X, XT and the candidate
-// lists nbr / cnt; the cell order is left in lr_sorted_idx).
-static int step_low_record_into(gs_ctx* c, float dt, int iters, float4* X, float4* XT, uint32_t* nbr, uint32_t* cnt)
+// The LR step of io keeping what every pass evaluates on, in cell order (the
+// particle of each slot in idx): x~ before pass it is XT[it], x before
+// stabilization pass it is X[it] (after the stabilization passes X[n_stab]
+// throughout); the passes read and write the snapshot buffers themselves.
+// XT[total] holds the step's final x~, unless final_state: then the step's
+// end is written to io.xo, io.vo, by the last pass itself where it is a
+// solver pass (which no snapshot is needed of).
+static int step_low_record_into(gs_ctx* c, const StepIo& io, float dt, int iters, float4* X, float4* XT,
+                                uint32_t* nbr, uint32_t* cnt, uint32_t* idx, bool final_state)
 {
     const int64_t N = c->n_low;
     const int total = c->n_stab + iters;
-    int st = flag_solid(c, (const float*)c->lr_pos, N);
-    if (st) return st;
-    PbdArgs a = pbd_args(c, dt);
-    st = step_begin(c, a, X, XT, c->step_cell_start, nbr, cnt);
+    const PbdArgs a = pbd_args(c, dt);
+    int st = step_begin(c, a, io, X, XT, c->step_cell_start, nbr, cnt, idx, true);
     if (st) return st;
     for (int it = 0; it < total; ++it) {
         const int stab = it < c->n_stab;
+        const bool fin = final_state && iters > 0 && it + 1 == total;
         CK(gs_launch_pass(c->stream, a, stab, X + (size_t)std::min(it, c->n_stab) * N, XT + (size_t)it * N,
-                          X + (size_t)(it + 1) * N, XT + (size_t)(it + 1) * N, nbr, cnt, &c->launches),
+                          X + (size_t)(it + 1) * N, XT + (size_t)(it + 1) * N, nbr, cnt, &c->launches,
+                          fin ? idx : nullptr, fin ? io.xo : nullptr, fin ? io.vo : nullptr, io.x),
            "pass");
     }
+    if (final_state && iters == 0)
+        CK(gs_launch_finalize(c->stream, a, idx, X + (size_t)total * N, XT + (size_t)total * N, io.xo, io.vo, io.x,
+                              &c->launches, nullptr),
+           "finalize");
     return GS_OK;
 }
 
 static int step_low_record(gs_ctx* c, float dt, int iters)
 {
-    return step_low_record_into(c, dt, iters, c->snap, c->snap_xt, c->nbr, c->nbr_cnt);
+    return step_low_record_into(c, StepIo{c->lr_pos, c->lr_vel, nullptr, nullptr}, dt, iters, c->snap, c->snap_xt,
+                                c->nbr, c->nbr_cnt, c->lr_vals[1], false);
 }
-
-// The passes of a recorded LR step in reverse: dL/d outputs from
-// adj_io[0..1], dL/d inputs into adj_io[2..3]; X, XT, nbr, cnt as recorded,
-// idx the recording's cell order.
-static int step_low_reverse_from(gs_ctx* c, float dt, int iters, const float4* X, const float4* XT,
-                                 const uint32_t* nbr, const uint32_t* cnt, const uint32_t* idx);
 
 // The reverse LR step on the context's buffers: the step again from
 // (lr_pos, lr_vel) keeping what every pass evaluates on, then the passes in
-// reverse.
+// reverse, from adj_io[0..1] into adj_io[2..3].
 static int step_low_reverse(gs_ctx* c, float dt, int iters)
 {
+    const int64_t N = c->n_low;
     int st = step_low_record(c, dt, iters);
     if (st) return st;
-    return step_low_reverse_from(c, dt, iters, c->snap, c->snap_xt, c->nbr, c->nbr_cnt, c->lr_sorted_idx);
+    return step_low_reverse_from(c, dt, iters, c->snap, c->snap_xt, c->nbr, c->nbr_cnt, c->lr_vals[1], c->adj_io,
+                                 c->adj_io + N, c->adj_io + 2 * N, c->adj_io + 3 * N);
 }
 
+// The passes of a recorded LR step in reverse: dL/d outputs gxo, gvo, dL/d
+// inputs into gx0, gv0 (original order); X, XT, nbr, cnt as recorded, idx the
+// recording's cell order.
 static int step_low_reverse_from(gs_ctx* c, float dt, int iters, const float4* X, const float4* XT,
-                                 const uint32_t* nbr, const uint32_t* cnt, const uint32_t* idx)
+                                 const uint32_t* nbr, const uint32_t* cnt, const uint32_t* idx, const float4* gxo,
+                                 const float4* gvo, float4* gx0, float4* gv0)
 {
     const int64_t N = c->n_low;
     const int total = c->n_stab + iters;
@@ -2612,16 +2707,20 @@ static int step_low_reverse_from(gs_ctx* c, float dt, int iters, const float4* X
     auto x_before = [&](int it) { return X + (size_t)std::min(it, c->n_stab) * N; };
     const float4* xfix = x_before(total);     // x after stabilization
     const float4* ws = XT;                    // w of xt carries the inverse scaled mass (every pass keeps it)
-    CK(gs_launch_adj_init(c->stream, N, idx, c->adj_io, c->adj_io + N, dt, c->adj_gx, c->adj_gxt, c->adj_gws,
-                          &c->launches),
-       "reverse init");
     float4* Hb[2] = {c->adj_h, c->adj_h2};
     int hc = 0;
     auto y_of = [&](int it) { return it < c->n_stab ? x_before(it) : XT + (size_t)it * N; };
-    if (total > 0)
-        CK(gs_launch_adj_h(c->stream, a, (total - 1) < c->n_stab, y_of(total - 1), ws, nbr, cnt, c->adj_gx, c->adj_gxt,
-                           Hb[0], &c->launches),
-           "reverse h");
+    c->lr_binned = false;
+    if (total == 0) {   // no pass: the prediction alone
+        CK(gs_launch_adj_init(c->stream, N, idx, gxo, gvo, dt, c->adj_gx, c->adj_gxt, c->adj_gws, &c->launches),
+           "reverse init");
+        CK(gs_launch_adj_final(c->stream, a, idx, ws, c->adj_gx, c->adj_gxt, c->adj_gws, gx0, gv0, &c->launches),
+           "reverse predict");
+        return GS_OK;
+    }
+    CK(gs_launch_adj_h(c->stream, a, (total - 1) < c->n_stab, y_of(total - 1), ws, nbr, cnt, idx, gxo, gvo, c->adj_gx,
+                       c->adj_gxt, c->adj_gws, Hb[0], &c->launches),
+       "reverse h");
     for (int it = total - 1; it >= 0; --it) {
         const int stab = it < c->n_stab;
         AdjRecord rec;
@@ -2636,14 +2735,10 @@ static int step_low_reverse_from(gs_ctx* c, float dt, int iters, const float4* X
         }
         CK(gs_launch_adj_pass(c->stream, a, stab, y_of(it), XT + (size_t)it * N, xfix, ws, nbr, cnt, Hb[hc],
                               c->adj_gx, c->adj_gxt, c->adj_gws, &c->launches, rec, it > 0 ? y_of(it - 1) : nullptr,
-                              (it - 1) < c->n_stab, Hb[hc ^ 1]),
+                              (it - 1) < c->n_stab, Hb[hc ^ 1], it == 0 ? idx : nullptr, gx0, gv0),
            "reverse pass");
         hc ^= 1;
     }
-    CK(gs_launch_adj_final(c->stream, a, idx, ws, c->adj_gx, c->adj_gxt, c->adj_gws, c->adj_io + 2 * N,
-                           c->adj_io + 3 * N, &c->launches),
-       "reverse predict");
-    c->lr_binned = false;
     return GS_OK;
 }
 
@@ -2770,3 +2865,66 @@ int gs_timing_read(gs_ctx* c, int timer, double* total_ms, int64_t* launches)
 int64_t gs_launch_count(const gs_ctx* c) { return c ? c->launches : 0; }
 
 }  // extern "C"
+
+// ---- the functional sequences on given buffers, for the rollout -------------
+int gs_rollout_begin(gs_ctx* c)
+{
+    int st = check_state(c);
+    if (st) return st;
+    return settle(c);
+}
+
+int gs_rollout_buffers(gs_ctx* c, int iters, int n_slots)
+{
+    int st = GS_OK;
+    if ((int)c->tapes.size() < n_slots) st = gs_set_step_tapes(c, n_slots);
+    if (st == GS_OK && c->n_low > 0 && n_slots > 0) st = ensure_tapes(c, c->n_stab + iters);
+    if (st == GS_OK) st = ensure_adjoint_buffers(c);
+    if (st == GS_OK) st = ensure_fscratch(c);   // the deterministic reverse frame's
+    return st;
+}
+
+int gs_core_set_lr(gs_ctx* c, const float4* x, const float4* v)
+{
+    c->lr_binned = false;
+    return copy_all(c, {{x, c->lr_pos, c->n_low}, {v, c->lr_vel, c->n_low}});
+}
+
+int gs_core_step(gs_ctx* c, const float4* x, const float4* v, float4* xo, float4* vo, float dt, int iters)
+{
+    return step_low_io(c, StepIo{x, v, xo, vo}, dt, iters);
+}
+
+int gs_core_step_taped(gs_ctx* c, const float4* x, const float4* v, float4* xo, float4* vo, float dt, int iters,
+                       int slot)
+{
+    if (c->n_materials > 0 || c->n_bodies > 0)
+        return fail(c, GS_ERR_STATE, "taped LR steps cover grains of the scenes' coefficients only");
+    if (c->n_low == 0) return GS_OK;
+    return step_low_tape_forward(c, StepIo{x, v, xo, vo}, c->tapes[(size_t)slot], dt, iters);
+}
+
+int gs_core_step_backward(gs_ctx* c, int slot, float dt, int iters, const float4* gxo, const float4* gvo, float4* gx0,
+                          float4* gv0)
+{
+    if (c->rec_lr_pair && c->n_stab + iters > c->rec_max_passes)
+        return fail(c, GS_ERR_ARG, "%d passes exceed the decision record's %d", c->n_stab + iters, c->rec_max_passes);
+    if (c->n_low == 0) return GS_OK;
+    const gs_ctx::StepTape& t = c->tapes[(size_t)slot];
+    return step_low_reverse_from(c, dt, iters, t.X, t.XT, t.nbr, t.cnt, t.idx, gxo, gvo, gx0, gv0);
+}
+
+int gs_core_upsample(gs_ctx* c, const float4* lx, const float4* lv, const float4* hx, const float4* hv, float4* hxo,
+                     float4* hvo, float dt)
+{
+    if (c->n_high == 0) return GS_OK;
+    return upsample_fwd_seq(c, lx, lv, hx, hv, hxo, hvo, dt);
+}
+
+int gs_core_upsample_backward(gs_ctx* c, const float4* lx, const float4* lv, const float4* hx, const float4* hv,
+                              const float4* gxo, const float4* gvo, float4* glx, float4* glv, float4* ghx, float4* ghv,
+                              float dt)
+{
+    if (c->n_bodies > 0) return fail(c, GS_ERR_STATE, "the reverse modes do not support rigid bodies");
+    return upsample_bwd_seq(c, lx, lv, hx, hv, gxo, gvo, glx, glv, ghx, ghv, dt, 1);
+}

@@ -343,6 +343,7 @@ struct CsExtras {
     const uint32_t* gb_w = nullptr;       // the w of gb's copies is gb_w[particle] (as bits)
     const uint32_t* ga_solid = nullptr;   // nonzero: the w of ga's copy is 0
     uint32_t* slot_of = nullptr;          // slot_of[particle] = its slot
+    float4 *zero_a = nullptr, *zero_b = nullptr;   // cleared (the binning by buckets only)
     // Cells of more than 32 entries (big_list not null; only without copies):
     // listed in big_list (capacity n / 33 + 1, count in *big_count, zero on
     // entry) and ordered afterwards by big_blocks cooperating blocks, each
@@ -371,7 +372,8 @@ int gs_bins_tiles(int64_t n_cell);             // tiles, or 0 where the grid is 
 size_t gs_bins_bucket_words(int64_t n_cell);
 size_t gs_bins_count_words(int64_t n_cell);
 cudaError_t gs_bins_keys(cudaStream_t s, const LrBins& b, const float4* pos, int64_t n, const SceneDev* scenes,
-                         const uint32_t* tag, uint32_t* keys, int64_t* launches, int flag_solid, const uint32_t* body);
+                         const uint32_t* tag, uint32_t* keys, int64_t* launches, int flag_solid, const uint32_t* body,
+                         int* solid_err = nullptr);   // not null: GS_DEVERR_SOLID_REVERSE there where some w = 0
 cudaError_t gs_bins_finish(cudaStream_t s, const LrBins& b, int64_t n, int64_t n_cell, const uint32_t* keys,
                            uint32_t* out_keys, uint32_t* out_idx, uint32_t* start, const float4* ga, const float4* gb,
                            float4* ga_out, float4* gb_out, int64_t* launches, const CsExtras& ex,
@@ -385,6 +387,8 @@ cudaError_t gs_launch_cell_start(cudaStream_t s, const uint32_t* sorted_keys, in
                                  uint32_t* start, int64_t* launches);
 cudaError_t gs_launch_gather2(cudaStream_t s, const uint32_t* idx, const float4* a, const float4* b, float4* a_out,
                               float4* b_out, int64_t n, int64_t* launches);
+cudaError_t gs_launch_gather2_ids(cudaStream_t s, const uint32_t* idx, const float4* a, const float4* b, float4* a_out,
+                                  float4* b_out, int64_t n, int64_t m, int64_t* launches);
 cudaError_t gs_launch_unpermute(cudaStream_t s, const float4* pos_internal, const float4* field_internal,
                                 const uint32_t* hr_tag, float4* out, int64_t n_slots, int64_t n_real, int* err,
                                 int64_t* launches);
@@ -405,6 +409,8 @@ struct UpsampleArgs {
     const float4* hr_vel;
     float4* out_pos;
     float4* out_vel;
+    float4* id_pos;            // not null: the results in original order too
+    float4* id_vel;
     const float4* lr_spos;
     const float4* lr_svel;
     const uint32_t* cell_start;
@@ -458,18 +464,19 @@ cudaError_t gs_launch_neighbors(cudaStream_t s, const PbdArgs& a, const float4* 
 // One Jacobi pass.  With fin_idx not null the pass is the step's last: it
 // writes the finalized position and velocity to original order (fin_pos,
 // fin_vel through fin_idx) instead of x_out / xt_out.
+// fin_w: the step-start positions (their w is the inverse mass).
 // fin_rate (not null, last pass only): atomic max of |v| / (2 r_LR) of the
 // finalized velocities, as float bits.
 cudaError_t gs_launch_pass(cudaStream_t s, const PbdArgs& a, int stab, const float4* x_in, const float4* xt_in,
                            float4* x_out, float4* xt_out, const uint32_t* nbr, const uint32_t* cnt,
                            int64_t* launches, const uint32_t* fin_idx = nullptr, float4* fin_pos = nullptr,
-                           float4* fin_vel = nullptr, unsigned* fin_rate = nullptr);
+                           float4* fin_vel = nullptr, const float4* fin_w = nullptr, unsigned* fin_rate = nullptr);
 // Prediction + cell keys + arrival ranks (the counting stage of the binning).
 cudaError_t gs_launch_predict_keys(cudaStream_t s, const PbdArgs& a, const float4* pos, const float4* vel,
                                    float4* xt, uint32_t* keys, uint32_t* rank, uint32_t* cnt, int64_t* launches);
 // The same with the arrivals of the LR binning by buckets.
 cudaError_t gs_launch_predict_bins(cudaStream_t s, const PbdArgs& a, const LrBins& b, const float4* pos,
-                                   const float4* vel, float4* xt, uint32_t* keys, int64_t* launches);
+                                   const float4* vel, float4* xt, uint32_t* keys, int* solid_err, int64_t* launches);
 // All n_stab + iters passes of one step in one cooperative launch of at most
 // max_blocks blocks (gs_solve_blocks: the blocks that fit on the GPU at
 // once), with grid barriers between passes.  bar: two words of scratch.
@@ -479,7 +486,7 @@ cudaError_t gs_launch_solve(cudaStream_t s, const PbdArgs& a, int n_stab, int it
                             const uint32_t* nbr, const uint32_t* cnt, unsigned* bar, int* err, int max_blocks,
                             int64_t* launches, unsigned extra_arrivals = 0);
 cudaError_t gs_launch_finalize(cudaStream_t s, const PbdArgs& a, const uint32_t* idx, const float4* s_x,
-                               const float4* s_xt, float4* pos, float4* vel, int64_t* launches,
+                               const float4* s_xt, float4* pos, float4* vel, const float4* w_src, int64_t* launches,
                                unsigned* rate = nullptr);
 // CFL-limited substeps (gs_frame_adaptive): reset the control block for a
 // frame of t seconds; the largest |v| / (2 r_LR) of vel into st->rate; pick
@@ -529,13 +536,14 @@ struct AdjRecord {
     int n_comp = 0;
 };
 cudaError_t gs_launch_scatter2(cudaStream_t s, const uint32_t* idx, const float4* a, const float4* b, float4* ao,
-                               float4* bo, int64_t n, int64_t* launches);
+                               float4* bo, int64_t n, int64_t* launches, int add = 0);
 cudaError_t gs_launch_adj_init(cudaStream_t s, int64_t n, const uint32_t* idx, const float4* gxo, const float4* gvo,
                                float dt, float4* gx, float4* gxt, float* gws, int64_t* launches);
-// h = upstream / n per particle for one pass (the first pass to reverse).
+// The start of the reverse: gs_launch_adj_init's values, and h = upstream / n
+// per particle for the first pass to reverse.
 cudaError_t gs_launch_adj_h(cudaStream_t s, const PbdArgs& a, int stab, const float4* Y, const float4* WS,
-                            const uint32_t* nbr, const uint32_t* cnt, const float4* gx, const float4* gxt, float4* H,
-                            int64_t* launches);
+                            const uint32_t* nbr, const uint32_t* cnt, const uint32_t* idx, const float4* gxo,
+                            const float4* gvo, float4* gx, float4* gxt, float* gws, float4* H, int64_t* launches);
 // The reverse of one pass from its h (H); with Y_next the h of the pass
 // before it (evaluated on Y_next, a stabilization pass when stab_next) into
 // H_next, from the gradients this pass leaves.
@@ -543,10 +551,31 @@ cudaError_t gs_launch_adj_pass(cudaStream_t s, const PbdArgs& a, int stab, const
                                const float4* XF, const float4* WS, const uint32_t* nbr, const uint32_t* cnt,
                                const float4* H, float4* gx, float4* gxt, float* gws, int64_t* launches,
                                const AdjRecord& rec = AdjRecord{}, const float4* Y_next = nullptr,
-                               int stab_next = 0, float4* H_next = nullptr);
+                               int stab_next = 0, float4* H_next = nullptr, const uint32_t* fin_idx = nullptr,
+                               float4* gx0 = nullptr, float4* gv0 = nullptr);
 cudaError_t gs_launch_adj_final(cudaStream_t s, const PbdArgs& a, const uint32_t* idx, const float4* WS,
                                 const float4* gx, const float4* gxt, const float* gws, float4* gx0, float4* gv0,
                                 int64_t* launches);
+
+// The sequences of the functional entry points on given device buffers
+// (16-byte aligned, original order), for the rollout.  gs_rollout_buffers
+// allocates what they need for steps of `iters` solver passes with n_slots
+// tapes (nothing is allocated afterwards, so they can be captured).
+int gs_rollout_begin(gs_ctx* c);
+int gs_rollout_buffers(gs_ctx* c, int iters, int n_slots);
+int gs_core_step(gs_ctx* c, const float4* x, const float4* v, float4* xo, float4* vo, float dt, int iters);
+int gs_core_step_taped(gs_ctx* c, const float4* x, const float4* v, float4* xo, float4* vo, float dt, int iters,
+                       int slot);
+int gs_core_step_backward(gs_ctx* c, int slot, float dt, int iters, const float4* gxo, const float4* gvo, float4* gx0,
+                          float4* gv0);
+int gs_core_upsample(gs_ctx* c, const float4* lx, const float4* lv, const float4* hx, const float4* hv, float4* hxo,
+                     float4* hvo, float dt);
+// adds the LR gradients to glx / glv
+int gs_core_upsample_backward(gs_ctx* c, const float4* lx, const float4* lv, const float4* hx, const float4* hv,
+                              const float4* gxo, const float4* gvo, float4* glx, float4* glv, float4* ghx, float4* ghv,
+                              float dt);
+// Sets the context's LR state to x, v (workspace semantics of the rollout).
+int gs_core_set_lr(gs_ctx* c, const float4* x, const float4* v);
 
 // Records an error on the context (gs_last_error) and returns code.
 int gs_ctx_fail(gs_ctx* c, int code, const char* msg);

@@ -68,7 +68,7 @@ __global__ void k_predict_keys(const PbdArgs a, const float4* __restrict__ pos, 
 __global__ void __launch_bounds__(256) k_predict_bins(const PbdArgs a, const LrBins b,
                                                       const float4* __restrict__ pos,
                                                       const float4* __restrict__ vel, float4* __restrict__ xt,
-                                                      uint32_t* __restrict__ keys)
+                                                      uint32_t* __restrict__ keys, int* solid_err)
 {
     __shared__ uint32_t s_tile[kMaxBinTiles];
     bins_begin(b, s_tile);
@@ -77,6 +77,7 @@ __global__ void __launch_bounds__(256) k_predict_bins(const PbdArgs a, const LrB
         const SceneDev& sc = a.scenes[a.lr_scene[i]];
         const float dt = step_dt(a);
         float4 x = pos[i], v = vel[i];
+        if (solid_err && x.w == 0.0f) atomicOr(solid_err, GS_DEVERR_SOLID_REVERSE);
         const float gdt = x.w > 0.0f ? dt : 0.0f;   // no gravity for 1/m = 0
         float vx = v.x + gdt * sc.gx, vy = v.y + gdt * sc.gy, vz = v.z + gdt * sc.gz;
         float ws = x.w * expf(sc.mass_k * (x.z - sc.ground_z));
@@ -301,6 +302,7 @@ struct FinalOut {
     const uint32_t* idx;   // null: write the pass's outputs instead
     float4* pos;
     float4* vel;
+    const float4* w_src;   // the step-start positions (materials: their w is the inverse mass)
     unsigned* rate;        // not null: atomic max of the CFL rate of the new velocities
 };
 
@@ -318,7 +320,7 @@ __device__ __forceinline__ void pass_warp(const PbdArgs& a, int stab, int64_t p0
                                           const float4* __restrict__ x_in, const float4* __restrict__ xt_in,
                                           float4* __restrict__ x_out, float4* __restrict__ xt_out,
                                           const uint32_t* __restrict__ nbr, const uint32_t* __restrict__ cnt,
-                                          const FinalOut fin = FinalOut{nullptr, nullptr, nullptr, nullptr})
+                                          const FinalOut fin = FinalOut{nullptr, nullptr, nullptr, nullptr, nullptr})
 {
     constexpr unsigned kAll = 0xffffffffu;
     const int lane = (int)(threadIdx.x & 31u);
@@ -563,8 +565,9 @@ __device__ __forceinline__ void pass_warp(const PbdArgs& a, int stab, int64_t p0
             const float4 nv = make_float4((nt.x - nx.x) / dt, (nt.y - nx.y) / dt, (nt.z - nx.z) / dt, 0.0f);
             fin.vel[i] = nv;
             // with materials x.w holds the material id: the inverse mass comes
-            // from the step-start position, which only this thread touches
-            const float w = kMat ? fin.pos[i].w : nx.w;
+            // from the step-start position, which (also where the step works
+            // in place) only this thread touches
+            const float w = kMat ? fin.w_src[i].w : nx.w;
             fin.pos[i] = make_float4(nt.x, nt.y, nt.z, w);
             if (reduce) q = cfl_rate_bits(nv.x, nv.y, nv.z, sc.r_low);
         }
@@ -679,8 +682,8 @@ __global__ void __launch_bounds__(128, 6) k_solve(const SolveArgs s)
 }
 
 __global__ void k_finalize(const PbdArgs a, const uint32_t* __restrict__ idx, const float4* __restrict__ s_x,
-                           const float4* __restrict__ s_xt, float4* __restrict__ pos, float4* __restrict__ vel,
-                           unsigned* rate)
+                           const float4* __restrict__ s_xt, float4* pos, float4* __restrict__ vel,
+                           const float4* w_src, unsigned* rate)
 {
     int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     unsigned q = 0u;
@@ -690,7 +693,7 @@ __global__ void k_finalize(const PbdArgs a, const uint32_t* __restrict__ idx, co
         const float4 x = s_x[p], xt = s_xt[p];
         const float4 nv = make_float4((xt.x - x.x) / dt, (xt.y - x.y) / dt, (xt.z - x.z) / dt, 0.0f);
         vel[i] = nv;
-        const float w = a.mu_cross ? pos[i].w : x.w;   // x.w is the material id with materials
+        const float w = a.mu_cross ? w_src[i].w : x.w;   // x.w is the material id with materials
         pos[i] = make_float4(xt.x, xt.y, xt.z, w);
         if (rate) q = cfl_rate_bits(nv.x, nv.y, nv.z, a.scenes[a.lr_scene[i]].r_low);
     }
@@ -885,10 +888,10 @@ cudaError_t gs_launch_predict_keys(cudaStream_t s, const PbdArgs& a, const float
 }
 
 cudaError_t gs_launch_predict_bins(cudaStream_t s, const PbdArgs& a, const LrBins& b, const float4* pos,
-                                   const float4* vel, float4* xt, uint32_t* keys, int64_t* launches)
+                                   const float4* vel, float4* xt, uint32_t* keys, int* solid_err, int64_t* launches)
 {
     if (a.n <= 0) return cudaSuccess;
-    k_predict_bins<<<gs_blocks(a.n, 256), 256, 0, s>>>(a, b, pos, vel, xt, keys);
+    k_predict_bins<<<gs_blocks(a.n, 256), 256, 0, s>>>(a, b, pos, vel, xt, keys, solid_err);
     *launches += 1;
     return cudaGetLastError();
 }
@@ -948,10 +951,10 @@ static void launch_pass(cudaStream_t s, const PbdArgs& a, int stab, const float4
 cudaError_t gs_launch_pass(cudaStream_t s, const PbdArgs& a, int stab, const float4* x_in, const float4* xt_in,
                            float4* x_out, float4* xt_out, const uint32_t* nbr, const uint32_t* cnt,
                            int64_t* launches, const uint32_t* fin_idx, float4* fin_pos, float4* fin_vel,
-                           unsigned* fin_rate)
+                           const float4* fin_w, unsigned* fin_rate)
 {
     if (a.n <= 0) return cudaSuccess;
-    const FinalOut fin{fin_idx, fin_pos, fin_vel, fin_idx ? fin_rate : nullptr};
+    const FinalOut fin{fin_idx, fin_pos, fin_vel, fin_w, fin_idx ? fin_rate : nullptr};
     if (a.n <= kWideMax) launch_pass<8>(s, a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt, fin);
     else launch_pass<2>(s, a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt, fin);
     *launches += 1;
@@ -1000,10 +1003,11 @@ cudaError_t gs_launch_solve(cudaStream_t s, const PbdArgs& a, int n_stab, int it
 }
 
 cudaError_t gs_launch_finalize(cudaStream_t s, const PbdArgs& a, const uint32_t* idx, const float4* s_x,
-                               const float4* s_xt, float4* pos, float4* vel, int64_t* launches, unsigned* rate)
+                               const float4* s_xt, float4* pos, float4* vel, const float4* w_src, int64_t* launches,
+                               unsigned* rate)
 {
     if (a.n <= 0) return cudaSuccess;
-    k_finalize<<<gs_blocks(a.n, 256), 256, 0, s>>>(a, idx, s_x, s_xt, pos, vel, rate);
+    k_finalize<<<gs_blocks(a.n, 256), 256, 0, s>>>(a, idx, s_x, s_xt, pos, vel, w_src, rate);
     *launches += 1;
     return cudaGetLastError();
 }

@@ -19,15 +19,6 @@
 
 namespace {
 
-// a += b over n float4 records (the w components are left as they are)
-__global__ void k_add4(float4* __restrict__ a, const float4* __restrict__ b, int64_t n)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float4 x = a[i], y = b[i];
-    a[i] = make_float4(x.x + y.x, x.y + y.y, x.z + y.z, x.w);
-}
-
 int grow(gs_ctx* c, float4** buf, int64_t* cap, int64_t need, const char* what)
 {
     if (need <= *cap && *buf) return GS_OK;
@@ -78,15 +69,15 @@ int rollout_forward_body(gs_ctx* c, void* arg)
 {
     const RolloutCfg& g = *(const RolloutCfg*)arg;
     const int64_t N = c->n_low, M = c->n_high, rec = 2 * N + 2 * M;
-    float *lx = (float*)io(c, 4), *lv = (float*)io(c, 5), *hx = (float*)io(c, 6), *hv = (float*)io(c, 7);
-    RO(copy(c, io(c, 4), io(c, 0), rec));   // the four fields are contiguous
+    float4 *lx = io(c, 4), *lv = io(c, 5), *hx = io(c, 6), *hv = io(c, 7);
+    RO(copy(c, lx, io(c, 0), rec));   // the four fields are contiguous
     const float dts = g.dt / (float)g.n_sub;
     for (int f = 0; f < g.frames; ++f) {
-        if (f % g.every == 0) RO(copy(c, c->ro_ckpt + (int64_t)(f / g.every) * rec, io(c, 4), rec));
-        for (int s = 0; s < g.n_sub; ++s) RO(gs_step_low_forward(c, lx, lv, lx, lv, dts, g.iters));
-        RO(gs_upsample_forward(c, lx, lv, hx, hv, hx, hv, g.dt));
+        if (f % g.every == 0) RO(copy(c, c->ro_ckpt + (int64_t)(f / g.every) * rec, lx, rec));
+        for (int s = 0; s < g.n_sub; ++s) RO(gs_core_step(c, lx, lv, lx, lv, dts, g.iters));
+        RO(gs_core_upsample(c, lx, lv, hx, hv, hx, hv, g.dt));
     }
-    return GS_OK;
+    return g.frames > 0 ? gs_core_set_lr(c, lx, lv) : GS_OK;
 }
 
 int rollout_backward_body(gs_ctx* c, void* arg)
@@ -103,54 +94,35 @@ int rollout_backward_body(gs_ctx* c, void* arg)
     auto Hx = [&](int j) { return W + H0 + (int64_t)j * 2 * M; };
     float4* gl = W + G0;            // cotangent of the LR state (x | v)
     float4* gl2 = gl + 2 * N;       // the LR step's input cotangent
-    float4* gu = gl2 + 2 * N;       // the upsampling's LR gradient
-    float4* gh = gu + 2 * N;        // cotangent of the HR state (x | v)
+    float4* gh = gl2 + 2 * N;       // cotangent of the HR state (x | v)
     float4* gh2 = gh + 2 * M;       // the upsampling's HR-input gradient
     RO(copy(c, gl, io(c, 0), 2 * N));
     RO(copy(c, gh, io(c, 2), 2 * M));
-    // tags of the taped steps: the step's index in the rollout, above the
-    // range a caller's own tags use
-    const int64_t base = (int64_t)1 << 56;
     const int n_seg = (frames + every - 1) / every;
     for (int seg = n_seg - 1; seg >= 0; --seg) {
         const int f0 = seg * every, k = std::min(every, frames - f0);
         const float4* ck = c->ro_ckpt + (int64_t)seg * rec;
-        RO(copy(c, Lx(0), ck, 2 * N));
-        RO(copy(c, Hx(0), ck + 2 * N, 2 * M));
-        // recompute the segment, LR steps taped
+        // the segment's first state stays in its checkpoint
+        auto lr = [&](int i) { return i == 0 ? ck : (const float4*)Lx(i); };
+        auto hr = [&](int j) { return j == 0 ? ck + 2 * N : (const float4*)Hx(j); };
+        // recompute the segment, LR steps taped (step i of the segment in slot i)
         for (int j = 0; j < k; ++j) {
             for (int s = 0; s < n_sub; ++s) {
-                float4* in = Lx(j * n_sub + s);
-                float4* out = Lx(j * n_sub + s + 1);
-                RO(gs_step_low_forward_taped(c, (const float*)in, (const float*)(in + N), (float*)out,
-                                             (float*)(out + N), dts, iters, base + (int64_t)(f0 + j) * n_sub + s));
+                const int i = j * n_sub + s;
+                RO(gs_core_step_taped(c, lr(i), lr(i) + N, Lx(i + 1), Lx(i + 1) + N, dts, iters, i));
             }
             if (j + 1 < k) {
-                const float4* lr = Lx((j + 1) * n_sub);
-                RO(gs_upsample_forward(c, (const float*)lr, (const float*)(lr + N), (const float*)Hx(j),
-                                       (const float*)(Hx(j) + M), (float*)Hx(j + 1), (float*)(Hx(j + 1) + M), dt));
+                const float4* l = lr((j + 1) * n_sub);
+                RO(gs_core_upsample(c, l, l + N, hr(j), hr(j) + M, Hx(j + 1), Hx(j + 1) + M, dt));
             }
         }
         // the frames in reverse
         for (int j = k - 1; j >= 0; --j) {
-            const float4* lr = Lx((j + 1) * n_sub);
-            RO(gs_upsample_backward(c, (const float*)lr, (const float*)(lr + N), (const float*)Hx(j),
-                                    (const float*)(Hx(j) + M), (const float*)gh, (const float*)(gh + M), (float*)gu,
-                                    (float*)(gu + N), (float*)gh2, (float*)(gh2 + M), dt));
-            k_add4<<<gs_blocks(2 * N, 256), 256, 0, c->stream>>>(gl, gu, 2 * N);
-            if (cudaGetLastError() != cudaSuccess) return gs_ctx_fail(c, GS_ERR_CUDA, "rollout add failed");
-            c->launches += 1;
+            const float4* l = lr((j + 1) * n_sub);
+            RO(gs_core_upsample_backward(c, l, l + N, hr(j), hr(j) + M, gh, gh + M, gl, gl + N, gh2, gh2 + M, dt));
             std::swap(gh, gh2);
             for (int s = n_sub - 1; s >= 0; --s) {
-                const int64_t tag = base + (int64_t)(f0 + j) * n_sub + s;
-                int st = gs_step_low_backward_taped(c, tag, (const float*)gl, (const float*)(gl + N), (float*)gl2,
-                                                    (float*)(gl2 + N));
-                if (st == GS_ERR_STATE) {   // the record is gone: record the step again
-                    const float4* in = Lx(j * n_sub + s);
-                    st = gs_step_low_backward(c, (const float*)in, (const float*)(in + N), (const float*)gl,
-                                              (const float*)(gl + N), (float*)gl2, (float*)(gl2 + N), dts, iters);
-                }
-                if (st != GS_OK) return st;
+                RO(gs_core_step_backward(c, j * n_sub + s, dts, iters, gl, gl + N, gl2, gl2 + N));
                 std::swap(gl, gl2);
             }
         }
@@ -192,6 +164,7 @@ extern "C" int gs_rollout_forward(gs_ctx* c, const float* lr_x0, const float* lr
     const int64_t N = c->n_low, M = c->n_high;
     if (!lr_x0 || !lr_v0 || !hr_x0 || !hr_v0 || !lr_x || !lr_v || !hr_x || !hr_v)
         return gs_ctx_fail(c, GS_ERR_ARG, "null buffer");
+    RO(gs_rollout_begin(c));
     c->ro_valid = false;
     const int64_t rec = 2 * N + 2 * M;                                    // one state
     const int n_ckpt = (frames + checkpoint_every - 1) / checkpoint_every;  // segment starts
@@ -227,16 +200,14 @@ extern "C" int gs_rollout_backward(gs_ctx* c, const float* g_lr_x, const float* 
     if (!c->ro_valid) return gs_ctx_fail(c, GS_ERR_STATE, "no rollout forward to differentiate");
     if (!g_lr_x || !g_lr_v || !g_hr_x || !g_hr_v || !g_lr_x0 || !g_lr_v0 || !g_hr_x0 || !g_hr_v0)
         return gs_ctx_fail(c, GS_ERR_ARG, "null buffer");
+    RO(gs_rollout_begin(c));
     const int64_t N = c->n_low, M = c->n_high;
     RolloutCfg g{c->ro_dt, c->ro_frames, c->ro_n_sub, c->ro_iters, c->ro_every};
     const int k_max = std::min(g.every, std::max(g.frames, 1));
-    const int64_t need = (int64_t)(k_max * g.n_sub + 1) * 2 * N + (int64_t)k_max * 2 * M + 3 * 2 * N + 2 * 2 * M;
+    const int64_t need = (int64_t)(k_max * g.n_sub + 1) * 2 * N + (int64_t)k_max * 2 * M + 2 * 2 * N + 2 * 2 * M;
     if (c->ro_work_cap < need) c->ro_seen.clear();   // buffers move: capture anew
     RO(grow(c, &c->ro_work, &c->ro_work_cap, need, "no memory for the rollout's backward"));
-    if ((int)c->tapes.size() < k_max * g.n_sub) {
-        c->ro_seen.clear();
-        RO(gs_set_step_tapes(c, k_max * g.n_sub));
-    }
+    RO(gs_rollout_buffers(c, g.iters, g.frames > 0 ? k_max * g.n_sub : 0));
     RO(copy(c, io(c, 0), (const float4*)g_lr_x, N));
     RO(copy(c, io(c, 1), (const float4*)g_lr_v, N));
     RO(copy(c, io(c, 2), (const float4*)g_hr_x, M));

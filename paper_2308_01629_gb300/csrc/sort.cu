@@ -662,7 +662,7 @@ __global__ void __launch_bounds__(kThreads) k_cs_order_big(const uint32_t* __res
 __global__ void __launch_bounds__(256) k_bins_keys(const LrBins b, const float4* __restrict__ pos, int64_t n,
                                                    const SceneDev* __restrict__ scenes,
                                                    const uint32_t* __restrict__ tag, uint32_t* __restrict__ keys,
-                                                   int flag_solid, const uint32_t* __restrict__ body)
+                                                   int flag_solid, const uint32_t* __restrict__ body, int* solid_err)
 {
     __shared__ uint32_t s_tile[kMaxBinTiles];
     bins_begin(b, s_tile);
@@ -671,6 +671,7 @@ __global__ void __launch_bounds__(256) k_bins_keys(const LrBins b, const float4*
         const SceneDev& sc = scenes[tag[i] & ~kPadBit];
         const float4 p = pos[i];
         if (flag_solid && (p.w == 0.0f || (body && body[i] != 0u))) atomicOr(b.words + kBinSolidAcc, 1u);
+        if (solid_err && p.w == 0.0f) atomicOr(solid_err, GS_DEVERR_SOLID_REVERSE);
         const uint32_t cell = grid_cell_of(sc, p.x, p.y, p.z);
         keys[i] = cell;
         bins_arrive(b, s_tile, cell, (uint32_t)i);
@@ -746,6 +747,8 @@ __global__ void __launch_bounds__(128) k_bins_place(const LrBins b, int64_t n, c
     ga_out[slot] = u;
     gb_out[slot] = v;
     if (ex.slot_of) ex.slot_of[i] = slot;
+    if (ex.zero_a) ex.zero_a[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (ex.zero_b) ex.zero_b[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 __global__ void k_cell_start(const uint32_t* __restrict__ sk, int64_t n, int64_t n_cell, uint32_t* __restrict__ start)
@@ -769,6 +772,26 @@ __global__ void k_gather2(const uint32_t* __restrict__ idx, const float4* __rest
     uint32_t i = idx[p];
     ao[p] = a[i];
     if (b) bo[p] = b[i];
+}
+
+// A caller's HR state (one scene, m particles in original order) into sorted
+// slots: slot p takes particle idx[p] with its id in the w of the position;
+// idx >= m are the padding slots.
+__global__ void k_gather2_ids(const uint32_t* __restrict__ idx, const float4* __restrict__ a,
+                              const float4* __restrict__ b, float4* __restrict__ ao, float4* __restrict__ bo, int64_t n,
+                              int64_t m)
+{
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= n) return;
+    const uint32_t i = idx[p];
+    float4 u = make_float4(0.f, 0.f, 0.f, __uint_as_float(0xffffffffu)), v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if ((int64_t)i < m) {
+        u = a[i];
+        v = b[i];
+        u.w = __uint_as_float(i);
+    }
+    ao[p] = u;
+    bo[p] = v;
 }
 
 // HR exchange in original-id order: slot p (a real particle, not padding)
@@ -915,10 +938,11 @@ size_t gs_bins_bucket_words(int64_t n_cell) { return (size_t)n_cell * kBucket; }
 size_t gs_bins_count_words(int64_t n_cell) { return (size_t)gs_bins_tiles(n_cell) * kBinTile; }
 
 cudaError_t gs_bins_keys(cudaStream_t s, const LrBins& b, const float4* pos, int64_t n, const SceneDev* scenes,
-                         const uint32_t* tag, uint32_t* keys, int64_t* launches, int flag_solid, const uint32_t* body)
+                         const uint32_t* tag, uint32_t* keys, int64_t* launches, int flag_solid, const uint32_t* body,
+                         int* solid_err)
 {
     if (n <= 0) return cudaSuccess;
-    k_bins_keys<<<gs_blocks(n, 256), 256, 0, s>>>(b, pos, n, scenes, tag, keys, flag_solid, body);
+    k_bins_keys<<<gs_blocks(n, 256), 256, 0, s>>>(b, pos, n, scenes, tag, keys, flag_solid, body, solid_err);
     *launches += 1;
     return cudaGetLastError();
 }
@@ -960,6 +984,15 @@ cudaError_t gs_launch_gather2(cudaStream_t s, const uint32_t* idx, const float4*
 {
     if (n <= 0) return cudaSuccess;
     k_gather2<<<gs_blocks(n, 256), 256, 0, s>>>(idx, a, b, a_out, b_out, n);
+    *launches += 1;
+    return cudaGetLastError();
+}
+
+cudaError_t gs_launch_gather2_ids(cudaStream_t s, const uint32_t* idx, const float4* a, const float4* b, float4* a_out,
+                                  float4* b_out, int64_t n, int64_t m, int64_t* launches)
+{
+    if (n <= 0) return cudaSuccess;
+    k_gather2_ids<<<gs_blocks(n, 256), 256, 0, s>>>(idx, a, b, a_out, b_out, n, m);
     *launches += 1;
     return cudaGetLastError();
 }

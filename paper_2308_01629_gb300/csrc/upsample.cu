@@ -389,6 +389,11 @@ __device__ __forceinline__ void upsample_item(const UpsampleArgs& a, int64_t ite
     hr_boundary(nx, ny, nz, nvx, nvy, nvz, a.sdf + sc.sdf_begin, sc.n_sdf, sc.r_high);
     __stcs(a.out_pos + i, make_float4(nx, ny, nz, p.w));
     __stcs(a.out_vel + i, make_float4(nvx, nvy, nvz, 0.0f));
+    if (a.id_pos) {   // the caller's buffers, in original order
+        const uint32_t id = __float_as_uint(p.w);
+        a.id_pos[id] = make_float4(nx, ny, nz, p.w);
+        a.id_vel[id] = make_float4(nvx, nvy, nvz, 0.0f);
+    }
 }
 
 template <int WARPS, bool kSolid, bool kSingle>
