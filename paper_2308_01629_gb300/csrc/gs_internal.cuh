@@ -458,6 +458,16 @@ struct PbdArgs {
     const float4* body_xf;
     const uint32_t* sorted_idx;
 };
+// What the last pass of a step does beyond its own: nothing, the next step's
+// prediction and arrivals (of the same length), or the arrivals of the final
+// positions for the upsampling's binning (binning by buckets only).
+enum { kNextNone = 0, kNextStep = 1, kNextUpsample = 2 };
+struct NextBins {
+    int mode = kNextNone;
+    LrBins b;
+    float4* xt = nullptr;      // kNextStep: the predicted positions
+    uint32_t* keys = nullptr;
+};
 cudaError_t gs_launch_neighbors(cudaStream_t s, const PbdArgs& a, const float4* s_xt, const uint32_t* skeys,
                                 const uint32_t* cell_start, uint32_t* nbr, uint32_t* cnt, int cap, int* err,
                                 int64_t* launches);
@@ -470,7 +480,8 @@ cudaError_t gs_launch_neighbors(cudaStream_t s, const PbdArgs& a, const float4* 
 cudaError_t gs_launch_pass(cudaStream_t s, const PbdArgs& a, int stab, const float4* x_in, const float4* xt_in,
                            float4* x_out, float4* xt_out, const uint32_t* nbr, const uint32_t* cnt,
                            int64_t* launches, const uint32_t* fin_idx = nullptr, float4* fin_pos = nullptr,
-                           float4* fin_vel = nullptr, const float4* fin_w = nullptr, unsigned* fin_rate = nullptr);
+                           float4* fin_vel = nullptr, const float4* fin_w = nullptr, unsigned* fin_rate = nullptr,
+                           const NextBins& next = NextBins{});
 // Prediction + cell keys + arrival ranks (the counting stage of the binning).
 cudaError_t gs_launch_predict_keys(cudaStream_t s, const PbdArgs& a, const float4* pos, const float4* vel,
                                    float4* xt, uint32_t* keys, uint32_t* rank, uint32_t* cnt, int64_t* launches);
@@ -563,7 +574,7 @@ cudaError_t gs_launch_adj_final(cudaStream_t s, const PbdArgs& a, const uint32_t
 // tapes (nothing is allocated afterwards, so they can be captured).
 int gs_rollout_begin(gs_ctx* c);
 int gs_rollout_buffers(gs_ctx* c, int iters, int n_slots);
-int gs_core_step(gs_ctx* c, const float4* x, const float4* v, float4* xo, float4* vo, float dt, int iters);
+int gs_core_frame(gs_ctx* c, float4* lx, float4* lv, float4* hx, float4* hv, float dt, int n_sub, int iters);
 int gs_core_step_taped(gs_ctx* c, const float4* x, const float4* v, float4* xo, float4* vo, float dt, int iters,
                        int slot);
 int gs_core_step_backward(gs_ctx* c, int slot, float dt, int iters, const float4* gxo, const float4* gvo, float4* gx0,

@@ -22,6 +22,7 @@
 
 #include <cuda_runtime.h>
 
+#include "grid.cuh"
 #include "gs_internal.cuh"
 
 constexpr int kBucket = 16;
@@ -42,6 +43,17 @@ __device__ __forceinline__ void bins_arrive(const LrBins& b, uint32_t* s_tile, u
     if (rank < (uint32_t)kBucket) b.bucket[(size_t)cell * kBucket + rank] = i;
     else b.spill[atomicAdd(b.words + kBinSpillAcc, 1u)] = i;
     atomicAdd(s_tile + cell / kBinTile, 1u);
+}
+
+// The same by the lanes `mask` of a warp without the block's help (the last
+// pass of a step): lanes of the same tile add to it once.
+__device__ __forceinline__ void bins_arrive_warp(const LrBins& b, unsigned mask, uint32_t cell, uint32_t i)
+{
+    const uint32_t rank = atomicAdd(b.count + cell, 1u);
+    if (rank < (uint32_t)kBucket) b.bucket[(size_t)cell * kBucket + rank] = i;
+    else b.spill[atomicAdd(b.words + kBinSpillAcc, 1u)] = i;
+    const unsigned peers = __match_any_sync(mask, cell / kBinTile);
+    if ((int)(threadIdx.x & 31u) == __ffs(peers) - 1) atomicAdd(b.tile + cell / kBinTile, (uint32_t)__popc(peers));
 }
 
 // Adds the block's tile counts to the tiles' (after every thread's arrival).

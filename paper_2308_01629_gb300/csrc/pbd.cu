@@ -44,6 +44,19 @@ __device__ __forceinline__ unsigned cfl_rate_bits(float vx, float vy, float vz, 
     return __float_as_uint(__fdiv_rn(__fsqrt_rn(s), __fmul_rn(2.0f, r_low)));
 }
 
+// x~ and the inverse height-scaled mass from a step-start state.  Particles of
+// infinite mass (1/m = 0: sampled boundaries, rigid bodies) keep their
+// prescribed velocity; 1/m* = (1/m) e^{h(x)}, h = k (z - ground).  The
+// multiply-adds are written out: the last pass of a step predicts the next
+// one's with the same bits.
+__device__ __forceinline__ float4 predicted(const SceneDev& sc, float4 x, float4 v, float dt)
+{
+    const float gdt = x.w > 0.0f ? dt : 0.0f;
+    const float vx = fmaf(gdt, sc.gx, v.x), vy = fmaf(gdt, sc.gy, v.y), vz = fmaf(gdt, sc.gz, v.z);
+    const float ws = x.w * expf(sc.mass_k * (x.z - sc.ground_z));
+    return make_float4(fmaf(dt, vx, x.x), fmaf(dt, vy, x.y), fmaf(dt, vz, x.z), ws);
+}
+
 // Prediction fused with the first stage of the binning: x~ as above, then
 // the cell of x~ under the grid contract and its arrival rank in the cell.
 __global__ void k_predict_keys(const PbdArgs a, const float4* __restrict__ pos, const float4* __restrict__ vel,
@@ -75,13 +88,9 @@ __global__ void __launch_bounds__(256) k_predict_bins(const PbdArgs a, const LrB
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < a.n) {
         const SceneDev& sc = a.scenes[a.lr_scene[i]];
-        const float dt = step_dt(a);
-        float4 x = pos[i], v = vel[i];
+        const float4 x = pos[i], v = vel[i];
         if (solid_err && x.w == 0.0f) atomicOr(solid_err, GS_DEVERR_SOLID_REVERSE);
-        const float gdt = x.w > 0.0f ? dt : 0.0f;   // no gravity for 1/m = 0
-        float vx = v.x + gdt * sc.gx, vy = v.y + gdt * sc.gy, vz = v.z + gdt * sc.gz;
-        float ws = x.w * expf(sc.mass_k * (x.z - sc.ground_z));
-        const float4 p = make_float4(x.x + dt * vx, x.y + dt * vy, x.z + dt * vz, ws);
+        const float4 p = predicted(sc, x, v, step_dt(a));
         xt[i] = p;
         const uint32_t cell = grid_cell_of(sc, p.x, p.y, p.z);
         keys[i] = cell;
@@ -304,6 +313,7 @@ struct FinalOut {
     float4* vel;
     const float4* w_src;   // the step-start positions (materials: their w is the inverse mass)
     unsigned* rate;        // not null: atomic max of the CFL rate of the new velocities
+    NextBins next;
 };
 
 // The pass of the warp's particles [p0, p0 + 32 / kLanes); every lane of the
@@ -315,12 +325,14 @@ struct FinalOut {
 // shape-matching delta (R xo + c) - x~ (Sec. 3), counted once in n_i.
 // kSingle: a context of one scene, whose parameters ride in the arguments
 // (constant memory) instead of two dependent loads per particle.
-template <int kLanes, bool kL2, bool kMat, bool kBody, bool kSingle>
+// kFin: the step's last pass, which finalizes it (fin) instead of writing
+// x_out / xt_out; its code apart keeps the other passes' registers.
+template <int kLanes, bool kL2, bool kMat, bool kBody, bool kSingle, bool kFin>
 __device__ __forceinline__ void pass_warp(const PbdArgs& a, int stab, int64_t p0, PassShared& sh,
                                           const float4* __restrict__ x_in, const float4* __restrict__ xt_in,
                                           float4* __restrict__ x_out, float4* __restrict__ xt_out,
                                           const uint32_t* __restrict__ nbr, const uint32_t* __restrict__ cnt,
-                                          const FinalOut fin = FinalOut{nullptr, nullptr, nullptr, nullptr, nullptr})
+                                          const FinalOut fin = FinalOut{nullptr, nullptr, nullptr, nullptr, nullptr, NextBins{}})
 {
     constexpr unsigned kAll = 0xffffffffu;
     const int lane = (int)(threadIdx.x & 31u);
@@ -541,7 +553,8 @@ __device__ __forceinline__ void pass_warp(const PbdArgs& a, int stab, int64_t p0
     acc.Dz += __shfl_xor_sync(kAll, acc.Dz, 1);
     acc.n += __shfl_xor_sync(kAll, acc.n, 1);
     const bool writer = valid && sub == 0;
-    const bool reduce = fin.idx && fin.rate;   // the whole warp meets in the rate reduction below
+    const unsigned writers = kFin ? __ballot_sync(kAll, writer) : 0u;
+    const bool reduce = kFin && fin.rate;   // the whole warp meets in the rate reduction below
     if (!writer && !reduce) return;
     float4 nt = xtp;
     float4 nx = xp;
@@ -557,7 +570,7 @@ __device__ __forceinline__ void pass_warp(const PbdArgs& a, int stab, int64_t p0
             nx.z += uz;
         }
     }
-    if (fin.idx) {
+    if constexpr (kFin) {
         unsigned q = 0u;
         if (writer) {
             const float dt = step_dt(a);
@@ -568,7 +581,20 @@ __device__ __forceinline__ void pass_warp(const PbdArgs& a, int stab, int64_t p0
             // from the step-start position, which (also where the step works
             // in place) only this thread touches
             const float w = kMat ? fin.w_src[i].w : nx.w;
-            fin.pos[i] = make_float4(nt.x, nt.y, nt.z, w);
+            const float4 np = make_float4(nt.x, nt.y, nt.z, w);
+            fin.pos[i] = np;
+            if (fin.next.mode != kNextNone) {
+                float4 at = np;
+                if (fin.next.mode == kNextStep) {
+                    at = predicted(sc, np, nv, dt);
+                    fin.next.xt[i] = at;
+                } else if (w == 0.0f || (kBody && a.body[i] != 0u)) {
+                    atomicOr(fin.next.b.words + kBinSolidAcc, 1u);
+                }
+                const uint32_t cell = grid_cell_of(sc, at.x, at.y, at.z);
+                fin.next.keys[i] = cell;
+                bins_arrive_warp(fin.next.b, writers, cell, i);
+            }
             if (reduce) q = cfl_rate_bits(nv.x, nv.y, nv.z, sc.r_low);
         }
         if (reduce) {
@@ -581,7 +607,7 @@ __device__ __forceinline__ void pass_warp(const PbdArgs& a, int stab, int64_t p0
     if (stab) st_pos<kL2>(x_out + p, nx);
 }
 
-template <int kLanes, bool kMat, bool kBody, bool kSingle>
+template <int kLanes, bool kMat, bool kBody, bool kSingle, bool kFin>
 __global__ void __launch_bounds__(kPassThreads, kPassBlocks) k_pass(
     const PbdArgs a, int stab, const float4* __restrict__ x_in, const float4* __restrict__ xt_in,
     float4* __restrict__ x_out, float4* __restrict__ xt_out, const uint32_t* __restrict__ nbr,
@@ -591,7 +617,7 @@ __global__ void __launch_bounds__(kPassThreads, kPassBlocks) k_pass(
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t p0 = w * (32 / kLanes);
     if (p0 >= a.n) return;   // whole warps
-    pass_warp<kLanes, false, kMat, kBody, kSingle>(a, stab, p0, sh[kLanes == 2 ? 0 : threadIdx.x >> 5], x_in, xt_in,
+    pass_warp<kLanes, false, kMat, kBody, kSingle, kFin>(a, stab, p0, sh[kLanes == 2 ? 0 : threadIdx.x >> 5], x_in, xt_in,
                                                    x_out, xt_out, nbr, cnt, fin);
 }
 
@@ -674,7 +700,7 @@ __global__ void __launch_bounds__(128, 6) k_solve(const SolveArgs s)
         float4* ti = bt ? s.xt1 : s.xt0;
         float4* to = bt ? s.xt0 : s.xt1;
         for (int64_t p0 = warp * kPer; p0 < s.a.n; p0 += warps * kPer)
-            pass_warp<kSolveLanes, true, kMat, false, false>(s.a, stab, p0, sh[0], xi, ti, xo, to, s.nbr, s.cnt);
+            pass_warp<kSolveLanes, true, kMat, false, false, false>(s.a, stab, p0, sh[0], xi, ti, xo, to, s.nbr, s.cnt);
         bt ^= 1;
         if (stab) bx ^= 1;
         if (it + 1 < total && !grid_barrier(s.bar, gridDim.x + s.extra_arrivals, (unsigned)it + 1u, s.err)) return;
@@ -918,43 +944,41 @@ cudaError_t gs_launch_neighbors(cudaStream_t s, const PbdArgs& a, const float4* 
     return cudaGetLastError();
 }
 
-template <int kLanes, bool kSingle>
-static void launch_pass_scenes(cudaStream_t s, const PbdArgs& a, int stab, const float4* x_in, const float4* xt_in,
-                               float4* x_out, float4* xt_out, const uint32_t* nbr, const uint32_t* cnt,
-                               const FinalOut& fin)
+template <int kLanes, bool kSingle, bool kFin>
+static void launch_pass_kind(cudaStream_t s, const PbdArgs& a, int stab, const float4* x_in, const float4* xt_in,
+                             float4* x_out, float4* xt_out, const uint32_t* nbr, const uint32_t* cnt,
+                             const FinalOut& fin)
 {
     const unsigned nb = gs_blocks(a.n * kLanes, kPassThreads);
-    if (a.body) {
-        if (a.mu_cross)
-            k_pass<kLanes, true, true, kSingle><<<nb, kPassThreads, 0, s>>>(a, stab, x_in, xt_in, x_out, xt_out, nbr,
-                                                                            cnt, fin);
-        else
-            k_pass<kLanes, false, true, kSingle><<<nb, kPassThreads, 0, s>>>(a, stab, x_in, xt_in, x_out, xt_out, nbr,
-                                                                             cnt, fin);
-    } else if (a.mu_cross) {
-        k_pass<kLanes, true, false, kSingle><<<nb, kPassThreads, 0, s>>>(a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt,
-                                                                         fin);
-    } else {
-        k_pass<kLanes, false, false, kSingle><<<nb, kPassThreads, 0, s>>>(a, stab, x_in, xt_in, x_out, xt_out, nbr,
-                                                                          cnt, fin);
-    }
+    auto go = [&](auto kernel) {
+        kernel<<<nb, kPassThreads, 0, s>>>(a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt, fin);
+    };
+    if (a.body && a.mu_cross) go(k_pass<kLanes, true, true, kSingle, kFin>);
+    else if (a.body) go(k_pass<kLanes, false, true, kSingle, kFin>);
+    else if (a.mu_cross) go(k_pass<kLanes, true, false, kSingle, kFin>);
+    else go(k_pass<kLanes, false, false, kSingle, kFin>);
 }
 
 template <int kLanes>
 static void launch_pass(cudaStream_t s, const PbdArgs& a, int stab, const float4* x_in, const float4* xt_in,
                         float4* x_out, float4* xt_out, const uint32_t* nbr, const uint32_t* cnt, const FinalOut& fin)
 {
-    if (a.n_scenes == 1) launch_pass_scenes<kLanes, true>(s, a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt, fin);
-    else launch_pass_scenes<kLanes, false>(s, a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt, fin);
+    if (a.n_scenes == 1) {
+        if (fin.idx) launch_pass_kind<kLanes, true, true>(s, a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt, fin);
+        else launch_pass_kind<kLanes, true, false>(s, a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt, fin);
+    } else {
+        if (fin.idx) launch_pass_kind<kLanes, false, true>(s, a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt, fin);
+        else launch_pass_kind<kLanes, false, false>(s, a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt, fin);
+    }
 }
 
 cudaError_t gs_launch_pass(cudaStream_t s, const PbdArgs& a, int stab, const float4* x_in, const float4* xt_in,
                            float4* x_out, float4* xt_out, const uint32_t* nbr, const uint32_t* cnt,
                            int64_t* launches, const uint32_t* fin_idx, float4* fin_pos, float4* fin_vel,
-                           const float4* fin_w, unsigned* fin_rate)
+                           const float4* fin_w, unsigned* fin_rate, const NextBins& next)
 {
     if (a.n <= 0) return cudaSuccess;
-    const FinalOut fin{fin_idx, fin_pos, fin_vel, fin_w, fin_idx ? fin_rate : nullptr};
+    const FinalOut fin{fin_idx, fin_pos, fin_vel, fin_w, fin_idx ? fin_rate : nullptr, next};
     if (a.n <= kWideMax) launch_pass<8>(s, a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt, fin);
     else launch_pass<2>(s, a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt, fin);
     *launches += 1;

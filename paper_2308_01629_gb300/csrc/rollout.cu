@@ -71,11 +71,9 @@ int rollout_forward_body(gs_ctx* c, void* arg)
     const int64_t N = c->n_low, M = c->n_high, rec = 2 * N + 2 * M;
     float4 *lx = io(c, 4), *lv = io(c, 5), *hx = io(c, 6), *hv = io(c, 7);
     RO(copy(c, lx, io(c, 0), rec));   // the four fields are contiguous
-    const float dts = g.dt / (float)g.n_sub;
     for (int f = 0; f < g.frames; ++f) {
         if (f % g.every == 0) RO(copy(c, c->ro_ckpt + (int64_t)(f / g.every) * rec, lx, rec));
-        for (int s = 0; s < g.n_sub; ++s) RO(gs_core_step(c, lx, lv, lx, lv, dts, g.iters));
-        RO(gs_core_upsample(c, lx, lv, hx, hv, hx, hv, g.dt));
+        RO(gs_core_frame(c, lx, lv, hx, hv, g.dt, g.n_sub, g.iters));
     }
     return g.frames > 0 ? gs_core_set_lr(c, lx, lv) : GS_OK;
 }

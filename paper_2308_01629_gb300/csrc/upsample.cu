@@ -133,7 +133,9 @@ __device__ __forceinline__ int sub_floor(float x, float o, float inv_h)
 // max w per lane), zero on entry and on return.  kSingle: a context of one
 // scene, whose parameters ride in the arguments instead of two dependent
 // loads per item.
-template <bool kSolid, bool kSingle>
+// kIds: the results go to the caller's buffers in original order too (its
+// registers would cost the plain gather 4 %).
+template <bool kSolid, bool kSingle, bool kIds>
 __device__ __forceinline__ void upsample_item(const UpsampleArgs& a, int64_t item, float* st, uint32_t* rows,
                                               float* sol, int lane)
 {
@@ -389,14 +391,14 @@ __device__ __forceinline__ void upsample_item(const UpsampleArgs& a, int64_t ite
     hr_boundary(nx, ny, nz, nvx, nvy, nvz, a.sdf + sc.sdf_begin, sc.n_sdf, sc.r_high);
     __stcs(a.out_pos + i, make_float4(nx, ny, nz, p.w));
     __stcs(a.out_vel + i, make_float4(nvx, nvy, nvz, 0.0f));
-    if (a.id_pos) {   // the caller's buffers, in original order
+    if constexpr (kIds) {
         const uint32_t id = __float_as_uint(p.w);
         a.id_pos[id] = make_float4(nx, ny, nz, p.w);
         a.id_vel[id] = make_float4(nvx, nvy, nvz, 0.0f);
     }
 }
 
-template <int WARPS, bool kSolid, bool kSingle>
+template <int WARPS, bool kSolid, bool kSingle, bool kIds>
 __global__ void __launch_bounds__(WARPS * 32, WARPS == 4 && !kSolid ? kAutoBlocks : 24 / WARPS)
     k_upsample(const UpsampleArgs a, int persistent)
 {
@@ -435,13 +437,13 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == 4 && !kSolid ? kAutoBlock
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(a.hr_vel + line));
             }
         }
-        upsample_item<kSolid, kSingle>(a, a.item_begin + item, s_st[warp], s_rows[warp], s_sol[kSolid ? warp : 0], lane);
+        upsample_item<kSolid, kSingle, kIds>(a, a.item_begin + item, s_st[warp], s_rows[warp], s_sol[kSolid ? warp : 0], lane);
     }
 }
 
 }  // namespace
 
-template <int WARPS, bool kSingle>
+template <int WARPS, bool kSingle, bool kIds>
 static cudaError_t launch_w(cudaStream_t s, const UpsampleArgs& a, int blocks_per_sm, int sm_count)
 {
     // both instantiations; the one the device flag does not select returns
@@ -451,18 +453,22 @@ static cudaError_t launch_w(cudaStream_t s, const UpsampleArgs& a, int blocks_pe
     const unsigned need = gs_blocks(a.n_warps, WARPS);
     const int64_t resident = (int64_t)std::max(blocks_per_sm, 1) * sm_count;
     const unsigned nb = (unsigned)std::min<int64_t>(resident, need);
-    if (blocks_per_sm <= 0) k_upsample<WARPS, false, kSingle><<<need, WARPS * 32, 0, s>>>(a, 0);
-    else k_upsample<WARPS, false, kSingle><<<nb, WARPS * 32, 0, s>>>(a, 1);
+    if (blocks_per_sm <= 0) k_upsample<WARPS, false, kSingle, kIds><<<need, WARPS * 32, 0, s>>>(a, 0);
+    else k_upsample<WARPS, false, kSingle, kIds><<<nb, WARPS * 32, 0, s>>>(a, 1);
     const unsigned nb_solid = (unsigned)std::min<int64_t>((int64_t)(24 / WARPS) * sm_count, need);
-    k_upsample<WARPS, true, kSingle><<<nb_solid, WARPS * 32, 0, s>>>(a, 1);
+    k_upsample<WARPS, true, kSingle, kIds><<<nb_solid, WARPS * 32, 0, s>>>(a, 1);
     return cudaGetLastError();
 }
 
 template <int WARPS>
 static cudaError_t launch_scenes(cudaStream_t s, const UpsampleArgs& a, int blocks_per_sm, int sm_count)
 {
-    return a.n_scenes == 1 ? launch_w<WARPS, true>(s, a, blocks_per_sm, sm_count)
-                           : launch_w<WARPS, false>(s, a, blocks_per_sm, sm_count);
+    if (a.id_pos) {   // the functional frame: one scene
+        if (a.n_scenes != 1) return cudaErrorInvalidValue;
+        return launch_w<WARPS, true, true>(s, a, blocks_per_sm, sm_count);
+    }
+    return a.n_scenes == 1 ? launch_w<WARPS, true, false>(s, a, blocks_per_sm, sm_count)
+                           : launch_w<WARPS, false, false>(s, a, blocks_per_sm, sm_count);
 }
 
 cudaError_t gs_launch_upsample(cudaStream_t s, const UpsampleArgs& a, int warps_per_block, int blocks_per_sm,

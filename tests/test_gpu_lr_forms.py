@@ -118,3 +118,26 @@ def test_gather_shapes_and_scene_forms_give_the_same_bits(ratio, solid):
     for sl, shape in (([sc], None), ([sc], (4, 7)), ([sc], (16, 0)), ([sc, scenes.cube()], None)):
         for a, b in zip(run(sl, shape), ref):
             np.testing.assert_array_equal(a.view(np.uint32), b.view(np.uint32))
+
+
+@pytest.mark.parametrize("kind", ["cube", "bed", "solids", "body", "materials", "batch"])
+def test_steps_that_begin_the_next_binning_give_the_same_bits(kind):
+    # within a frame a step's last pass begins the next binning; with the
+    # timers on every phase keeps its own launches
+    import paper_2308_01629_gb300 as gs
+    sc = {"cube": scenes.cube, "bed": lambda: scenes.digging(ratio=2, size=0.7), "solids": scenes.cube_on_particle_floor,
+          "body": scenes.cube_with_block, "materials": scenes.cube,
+          "batch": lambda: scenes.batch(n_scenes=3, lo_count=300, hi_count=900)}[kind]()
+    out = []
+    for timing in (False, True):
+        ctx = gs.Context(sc)
+        if kind == "materials":
+            ctx.set_materials(*scenes.materials(sc, 3))
+        ctx.set_timing(timing)
+        for _ in range(3):
+            ctx.frame(1.0 / 60.0, 3, 4)
+        out.append([ctx.read(f).view(np.uint32) for f in (gs.GS_FIELD_LR_POS, gs.GS_FIELD_LR_VEL, gs.GS_FIELD_HR_POS,
+                                                           gs.GS_FIELD_HR_VEL)])
+        ctx.close()
+    for a, b in zip(*out):
+        np.testing.assert_array_equal(a, b)
