@@ -503,6 +503,11 @@ int create_impl(int S, const gs_scene* scenes, const float* r_low, const float* 
         A(dalloc(&c->hr_bin_start, c->hr_bins + 2));
         A(dalloc(&c->hr_big, MS / 33 + 1));
         A(dalloc(&c->hr_scan_aux, gs_scan_aux_words(c->hr_bins + 1)));
+        c->hr_count.n_tiles = gs_bins_tiles(c->hr_bins);
+        if (c->hr_count.n_tiles > 0) {
+            A(dalloc(&c->hr_count.count, gs_bins_count_words(c->hr_bins)));
+            A(dalloc(&c->hr_count.tile, c->hr_count.n_tiles));
+        }
     }
     A(dalloc(&c->d_work, 1));
     A(dalloc(&c->d_err, 2));   // [0] device error bits, [1] scratch word of the host checks
@@ -542,6 +547,10 @@ int create_impl(int S, const gs_scene* scenes, const float* r_low, const float* 
         Z(cudaMemsetAsync(c->bins.count, 0, gs_bins_count_words(cells) * sizeof(uint32_t), c->stream));
         Z(cudaMemsetAsync(c->bins.tile, 0, c->bins.n_tiles * sizeof(uint32_t), c->stream));
         Z(cudaMemsetAsync(c->bins.words, 0, kBinWords * sizeof(uint32_t), c->stream));
+    }
+    if (c->hr_count.count) {
+        Z(cudaMemsetAsync(c->hr_count.count, 0, gs_bins_count_words(c->hr_bins) * sizeof(uint32_t), c->stream));
+        Z(cudaMemsetAsync(c->hr_count.tile, 0, c->hr_count.n_tiles * sizeof(uint32_t), c->stream));
     }
     if (z) Z(launch_hr_load(c, c->tmp4, c->hr_pos[0], 1));
     if (z) Z(launch_hr_load(c, c->tmp4, c->hr_vel[0], 0));
@@ -618,11 +627,16 @@ int resort_high_impl(gs_ctx* c, const float4* src_pos = nullptr, const float4* s
     const float4* pos = src_pos ? src_pos : c->hr_pos[cur];   // padding slots' positions are not read
     int which = 0;
     if (c->hr_counting) {
-        CK(gs_cs_clear(c->stream, c->hr_bin_start, c->hr_bins, 1), "clear counts");
-        CK(gs_launch_scene_keys(c->stream, pos, MS, c->d_scenes, c->hr_scene, 1, c->hr_keys[0], c->hr_vals[0],
-                                &c->launches, c->hr_bin_start),
-           "keys");
         CsExtras ex;
+        if (c->hr_count.count) {
+            ex.scan_bins = &c->hr_count;
+        } else {
+            CK(gs_cs_clear(c->stream, c->hr_bin_start, c->hr_bins, 1), "clear counts");
+        }
+        CK(gs_launch_scene_keys(c->stream, pos, MS, c->d_scenes, c->hr_scene, 1, c->hr_keys[0], c->hr_vals[0],
+                                &c->launches, ex.scan_bins ? c->hr_count.count : c->hr_bin_start, c->hr_count.tile,
+                                c->hr_count.n_tiles),
+           "keys");
         ex.big_list = c->hr_big;
         ex.big_count = c->hr_bin_start + c->hr_bins + 1;
         ex.big_scratch = c->hr_vals[0];   // the ranks are dead once scattered
@@ -1361,7 +1375,8 @@ void gs_destroy(gs_ctx* c)
                     c->body_start, c->body_xf, c->lr_slot, c->hr_bin_start, c->hr_big, c->hr_scan_aux,
                     c->async_in[0], c->async_in[1], c->async_in[2], c->async_in[3],
                     c->async_out[0], c->async_out[1], c->async_out[2], c->async_out[3], c->slab_stage,
-                    c->bins.count, c->bins.bucket, c->bins.tile, c->bins.spill, c->bins.words};
+                    c->bins.count, c->bins.bucket, c->bins.tile, c->bins.spill, c->bins.words,
+                    c->hr_count.count, c->hr_count.tile};
     for (void* b : bufs)
         if (b) cudaFree(b);
     free_tapes(c);

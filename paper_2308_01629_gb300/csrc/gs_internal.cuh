@@ -197,6 +197,7 @@ struct gs_ctx {
     bool hr_counting = false;
     int64_t hr_bins = 0;
     uint32_t* hr_bin_start = nullptr;
+    LrBins hr_count;                    // its counts and tile sums, zero between reorders; count null: counted in the starts
     uint32_t* hr_big = nullptr;
     uint32_t* hr_scan_aux = nullptr;
     float4* tmp4 = nullptr;                       // staging for reads / writes
@@ -344,6 +345,12 @@ struct CsExtras {
     const uint32_t* ga_solid = nullptr;   // nonzero: the w of ga's copy is 0
     uint32_t* slot_of = nullptr;          // slot_of[particle] = its slot
     float4 *zero_a = nullptr, *zero_b = nullptr;   // cleared (the binning by buckets only)
+    // counts and tile sums that the keys were counted in (gs_launch_scene_keys
+    // with tiles), apart from the starts: one scan launch makes the starts and
+    // clears *big_count, the order kernel clears the counts for the next sort
+    const LrBins* scan_bins = nullptr;
+    uint32_t *clear_count = nullptr, *clear_tile = nullptr;   // (gs_cs_finish sets these)
+    int n_clear_tiles = 0;
     // Cells of more than 32 entries (big_list not null; only without copies):
     // listed in big_list (capacity n / 33 + 1, count in *big_count, zero on
     // entry) and ordered afterwards by big_blocks cooperating blocks, each
@@ -379,10 +386,11 @@ cudaError_t gs_bins_finish(cudaStream_t s, const LrBins& b, int64_t n, int64_t n
                            float4* ga_out, float4* gb_out, int64_t* launches, const CsExtras& ex,
                            unsigned* solid_flag = nullptr, unsigned* clear = nullptr);   // *clear = 0 on the way
 // vals[i] = i, or with count not null the arrival rank of slot i in its
-// key's counter (count[key] += 1), for a counting sort by key.
+// key's counter (count[key] += 1), for a counting sort by key; tile: the
+// particles per tile of keys too.
 cudaError_t gs_launch_scene_keys(cudaStream_t s, const float4* pos, int64_t n, const SceneDev* scenes,
                                  const uint32_t* tag, int fine, uint32_t* keys, uint32_t* vals, int64_t* launches,
-                                 uint32_t* count = nullptr);
+                                 uint32_t* count = nullptr, uint32_t* tile = nullptr, int n_tiles = 0);
 cudaError_t gs_launch_cell_start(cudaStream_t s, const uint32_t* sorted_keys, int64_t n, int64_t n_cell,
                                  uint32_t* start, int64_t* launches);
 cudaError_t gs_launch_gather2(cudaStream_t s, const uint32_t* idx, const float4* a, const float4* b, float4* a_out,

@@ -197,12 +197,22 @@ __device__ __forceinline__ uint32_t scene_key(const float4* __restrict__ pos, in
 // Global key of a slot that belongs to scene tag & ~kPadBit: the scene's
 // cell offset plus its cell id (times 8 plus the octant when fine); padding
 // slots take the scene's padding cell so they sort to the end of its range.
-__global__ void k_scene_keys(const float4* __restrict__ pos, int64_t n, const SceneDev* __restrict__ scenes,
-                             const uint32_t* __restrict__ tag, int fine, uint32_t* __restrict__ keys,
-                             uint32_t* __restrict__ vals, uint32_t* __restrict__ count)
+// tile (with count): particles per tile of kBinTile keys, summed per block
+// first, so that one scan launch makes the starts (k_bins_scan).
+__global__ void __launch_bounds__(256) k_scene_keys(const float4* __restrict__ pos, int64_t n,
+                                                    const SceneDev* __restrict__ scenes,
+                                                    const uint32_t* __restrict__ tag, int fine,
+                                                    uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
+                                                    uint32_t* __restrict__ count, uint32_t* __restrict__ tile,
+                                                    int n_tiles)
 {
+    __shared__ uint32_t s_tile[kMaxBinTiles];
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (count) {
+        if (tile) {
+            for (int t = threadIdx.x; t < n_tiles; t += blockDim.x) s_tile[t] = 0u;
+            __syncthreads();
+        }
         // counting sort: the lanes of a warp that share a key take
         // consecutive ranks from one atomic (a reordered set arrives sorted)
         const bool ok = i < n;
@@ -210,11 +220,19 @@ __global__ void k_scene_keys(const float4* __restrict__ pos, int64_t n, const Sc
         const unsigned peers = __match_any_sync(0xffffffffu, key);
         const int lane = threadIdx.x & 31, leader = __ffs(peers) - 1;
         uint32_t base = 0;
-        if (ok && lane == leader) base = atomicAdd(count + key, (uint32_t)__popc(peers));
+        if (ok && lane == leader) {
+            base = atomicAdd(count + key, (uint32_t)__popc(peers));
+            if (tile) atomicAdd(s_tile + key / kBinTile, (uint32_t)__popc(peers));
+        }
         base = __shfl_sync(0xffffffffu, base, leader);
         if (ok) {
             keys[i] = key;
             vals[i] = base + __popc(peers & ((1u << lane) - 1u));
+        }
+        if (tile) {
+            __syncthreads();
+            for (int t = threadIdx.x; t < n_tiles; t += blockDim.x)
+                if (s_tile[t]) atomicAdd(tile + t, s_tile[t]);
         }
         return;
     }
@@ -534,6 +552,8 @@ __global__ void __launch_bounds__(256, 4) k_cs_order(const uint32_t* __restrict_
 {
     const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = (int)(threadIdx.x & 31u);
+    if (ex.clear_count && c < n_cell) ex.clear_count[c] = 0u;
+    if (c < ex.n_clear_tiles) ex.clear_tile[c] = 0u;
     uint32_t b = 0, e = 0;
     bool big = false;   // every lane reaches the ballot below: no early return
     if (c < n_cell) {
@@ -700,10 +720,12 @@ __global__ void __launch_bounds__(kScanBlock) k_bins_scan(const LrBins b, uint32
         run += c[k];
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {   // this binning's words, and zero for the next one's arrivals
-        b.words[kBinSpill] = b.words[kBinSpillAcc];
-        b.words[kBinSpillAcc] = 0u;
-        if (solid_flag) *solid_flag = b.words[kBinSolidAcc];
-        b.words[kBinSolidAcc] = 0u;
+        if (b.words) {
+            b.words[kBinSpill] = b.words[kBinSpillAcc];
+            b.words[kBinSpillAcc] = 0u;
+            if (solid_flag) *solid_flag = b.words[kBinSolidAcc];
+            b.words[kBinSolidAcc] = 0u;
+        }
         if (clear) *clear = 0u;
     }
 }
@@ -901,22 +923,36 @@ cudaError_t gs_cs_keys(cudaStream_t s, const float4* pos, int64_t n, const Scene
 
 cudaError_t gs_cs_finish(cudaStream_t s, int64_t n, int64_t n_cell, const uint32_t* keys, uint32_t* rank,
                          uint32_t* out_keys, uint32_t* out_idx, uint32_t* cell_start, uint32_t* aux, const float4* ga,
-                         const float4* gb, float4* ga_out, float4* gb_out, int64_t* launches, const CsExtras& ex)
+                         const float4* gb, float4* ga_out, float4* gb_out, int64_t* launches, const CsExtras& ex_in)
 {
     const int64_t total = n_cell + 1;
-    const int64_t nt = (total + kScanTile - 1) / kScanTile;
-    // up to kScanBlock tiles the apply blocks add up the tile totals before
-    // them themselves (at most one word per thread), saving the tile-sum scan
-    const int raw = nt <= kScanBlock;
-    k_scan_tiles<<<(unsigned)nt, kScanBlock, 0, s>>>(cell_start, total, aux);
-    if (!raw) k_scan_sums<<<1, kScanBlock, 0, s>>>(aux, nt);
-    k_scan_apply<<<(unsigned)nt, kScanBlock, 0, s>>>(cell_start, total, aux, raw);
-    *launches += raw ? 2 : 3;
+    if (ex_in.scan_bins) {
+        // counts and tile sums apart from the starts: one launch, and the
+        // order kernel clears them for the next sort
+        k_bins_scan<<<(unsigned)ex_in.scan_bins->n_tiles, kScanBlock, 0, s>>>(*ex_in.scan_bins, cell_start, total, nullptr,
+                                                                          ex_in.big_count);
+        *launches += 1;
+    } else {
+        const int64_t nt = (total + kScanTile - 1) / kScanTile;
+        // up to kScanBlock tiles the apply blocks add up the tile totals before
+        // them themselves (at most one word per thread), saving the tile-sum scan
+        const int raw = nt <= kScanBlock;
+        k_scan_tiles<<<(unsigned)nt, kScanBlock, 0, s>>>(cell_start, total, aux);
+        if (!raw) k_scan_sums<<<1, kScanBlock, 0, s>>>(aux, nt);
+        k_scan_apply<<<(unsigned)nt, kScanBlock, 0, s>>>(cell_start, total, aux, raw);
+        *launches += raw ? 2 : 3;
+    }
     if (n > 0) {
-        if (ex.big_list && (ga || ex.slot_of || ex.big_blocks <= 0 || !ex.big_count || !ex.big_scratch))
+        if (ex_in.big_list && (ga || ex_in.slot_of || ex_in.big_blocks <= 0 || !ex_in.big_count || !ex_in.big_scratch))
             return cudaErrorInvalidValue;   // listed cells are ordered without copies
         k_cs_scatter<<<gs_blocks(n, 256), 256, 0, s>>>(keys, rank, n, cell_start, out_keys, out_idx);
         // the ranks are dead once scattered: scratch for large cells
+        CsExtras ex = ex_in;
+        if (ex.scan_bins) {
+            ex.clear_count = ex.scan_bins->count;
+            ex.clear_tile = ex.scan_bins->tile;
+            ex.n_clear_tiles = ex.scan_bins->n_tiles;
+        }
         k_cs_order<<<gs_blocks(n_cell, 256), 256, 0, s>>>(cell_start, n_cell, out_idx, ga, gb, ga_out, gb_out, rank,
                                                           gs_key_bits(n), ex);
         *launches += 2;
@@ -1032,10 +1068,10 @@ cudaError_t gs_launch_permute_in(cudaStream_t s, const float4* pos_internal, con
 
 cudaError_t gs_launch_scene_keys(cudaStream_t s, const float4* pos, int64_t n, const SceneDev* scenes,
                                  const uint32_t* tag, int fine, uint32_t* keys, uint32_t* vals, int64_t* launches,
-                                 uint32_t* count)
+                                 uint32_t* count, uint32_t* tile, int n_tiles)
 {
     if (n <= 0) return cudaSuccess;
-    k_scene_keys<<<gs_blocks(n, 256), 256, 0, s>>>(pos, n, scenes, tag, fine, keys, vals, count);
+    k_scene_keys<<<gs_blocks(n, 256), 256, 0, s>>>(pos, n, scenes, tag, fine, keys, vals, count, tile, n_tiles);
     *launches += 1;
     return cudaGetLastError();
 }
