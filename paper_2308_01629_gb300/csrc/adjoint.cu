@@ -37,12 +37,20 @@ __device__ __forceinline__ int cell_of(float x, float o, float inv_h, int dim)
 
 constexpr int kMaxSteps = 32;
 constexpr int kBwdLanes = 4;
+constexpr int kBwdThreads = 128;
+// LR particles in reach that a lane remembers from the forward sums (about 14
+// of the 60 to 130 candidates of an HR particle are, 3 or 4 per lane); a lane
+// with more walks its candidates again.
+constexpr int kBwdHits = 16;
 
 // rec (optional): the decisions this reverse mode differentiates, four words
 // per HR particle: the LR particle of largest weight (original index through
 // lr_idx, or all ones), the blend case (1: alpha = 1 - max w), bit c = SDF
 // component c in contact, bit c = normal velocity removed at component c.
-__global__ void k_upsample_bwd(const SceneDev* __restrict__ scenes, const gs_sdf* __restrict__ sdf,
+// Instruction issue bounds it (12,600 warp instructions per 32 HR particles
+// when the second half walked every candidate again, 6,600 now; 64,000 HR: 46
+// us, now 34).
+__global__ void __launch_bounds__(kBwdThreads, 6) k_upsample_bwd(const SceneDev* __restrict__ scenes, const gs_sdf* __restrict__ sdf,
                                const float4* __restrict__ lr_spos, const float4* __restrict__ lr_svel,
                                const uint32_t* __restrict__ cell_start, const float4* __restrict__ hx,
                                const float4* __restrict__ hv, const float4* __restrict__ gxo,
@@ -59,6 +67,8 @@ __global__ void k_upsample_bwd(const SceneDev* __restrict__ scenes, const gs_sdf
     // particles are taken in the order `order` (slot -> particle), and the
     // coefficients and the position go to the slot (coef[2 slot ..],
     // pos_sorted[slot]) instead of any atomic.
+    __shared__ uint32_t s_hit[kBwdHits][kBwdThreads];
+    int n_hit = 0;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t slot = t / kBwdLanes;
     const int sub = (int)(t % kBwdLanes);
@@ -89,6 +99,8 @@ __global__ void k_upsample_bwd(const SceneDev* __restrict__ scenes, const gs_sdf
                 const float t = 1.0f - d2 * inv9r2;
                 const float w = t * t * t;
                 const float4 qv = lr_svel[j];
+                if (n_hit < kBwdHits) s_hit[n_hit][threadIdx.x] = j;
+                ++n_hit;
                 S += w;
                 Vx += w * qv.x;
                 Vy += w * qv.y;
@@ -188,29 +200,35 @@ __global__ void k_upsample_bwd(const SceneDev* __restrict__ scenes, const gs_sdf
     if (live && S > 0.0f) {
         const float gVx = gvtx / S, gVy = gvty / S, gVz = gvtz / S;
         const float gS = -(gvtx * vtx + gvty * vty + gvtz * vtz) / S;
-        for (int cz = cz0; cz <= cz1; ++cz)
-            for (int cy = cy0; cy <= cy1; ++cy) {
-                const int64_t row = (int64_t)sc.cell_off + ((int64_t)cz * g.dy + cy) * g.dx;
-                const uint32_t b = cell_start[row + cx0], e = cell_start[row + cx1 + 1];
-                for (uint32_t j = b + sub; j < e; j += kBwdLanes) {
-                    const float4 q = lr_spos[j];
-                    const float dx = p.x - q.x, dy = p.y - q.y, dz = p.z - q.z;
-                    const float d2 = dx * dx + dy * dy + dz * dz;
-                    if (!(d2 < R2)) continue;
-                    const float t = 1.0f - d2 * inv9r2;
-                    const float w = t * t * t;
-                    const float4 qv = lr_svel[j];
-                    const float gwj = gS + gVx * qv.x + gVy * qv.y + gVz * qv.z + (j == jstar ? gwmax : 0.0f);
-                    const float k6 = gwj * 6.0f * t * t * inv9r2;
-                    if (!coef) {   // one vector reduction per gradient (global float4 atomics, sm_90 and later)
-                        atomicAdd(gXs + j, make_float4(k6 * dx, k6 * dy, k6 * dz, 0.0f));
-                        atomicAdd(gVs + j, make_float4(w * gVx, w * gVy, w * gVz, 0.0f));
-                    }
-                    gpx -= k6 * dx;
-                    gpy -= k6 * dy;
-                    gpz -= k6 * dz;
-                }
+        // the gradients of LR particle j (in reach)
+        auto push = [&](uint32_t j) {
+            const float4 q = lr_spos[j];
+            const float dx = p.x - q.x, dy = p.y - q.y, dz = p.z - q.z;
+            const float d2 = dx * dx + dy * dy + dz * dz;
+            if (!(d2 < R2)) return;
+            const float t = 1.0f - d2 * inv9r2;
+            const float w = t * t * t;
+            const float4 qv = lr_svel[j];
+            const float gwj = gS + gVx * qv.x + gVy * qv.y + gVz * qv.z + (j == jstar ? gwmax : 0.0f);
+            const float k6 = gwj * 6.0f * t * t * inv9r2;
+            if (!coef) {   // one vector reduction per gradient (global float4 atomics, sm_90 and later)
+                atomicAdd(gXs + j, make_float4(k6 * dx, k6 * dy, k6 * dz, 0.0f));
+                atomicAdd(gVs + j, make_float4(w * gVx, w * gVy, w * gVz, 0.0f));
             }
+            gpx -= k6 * dx;
+            gpy -= k6 * dy;
+            gpz -= k6 * dz;
+        };
+        if (n_hit <= kBwdHits) {
+            for (int h = 0; h < n_hit; ++h) push(s_hit[h][threadIdx.x]);
+        } else {
+            for (int cz = cz0; cz <= cz1; ++cz)
+                for (int cy = cy0; cy <= cy1; ++cy) {
+                    const int64_t row = (int64_t)sc.cell_off + ((int64_t)cz * g.dy + cy) * g.dx;
+                    const uint32_t b = cell_start[row + cx0], e = cell_start[row + cx1 + 1];
+                    for (uint32_t j = b + sub; j < e; j += kBwdLanes) push(j);
+                }
+        }
     }
 #pragma unroll
     for (int o = 1; o < kBwdLanes; o <<= 1) {
@@ -353,82 +371,52 @@ __global__ void k_scatter2(const uint32_t* __restrict__ idx, const float4* __res
 //             F = s P rel (P = I - e e^T / e.e; s = 1 or thr_k / |P rel|)
 // A pass moves p by (sum c)/n_p; the reverse pass pushes h = g / n back
 // through every contribution that involves p (its own and its partners').
-struct M3 {
-    float a[9];
-};
+//
+// Only products of the Jacobians with one vector are needed, so none is
+// formed: with P and the perpendicular part's dependence on e applied to h
+// directly, a friction term takes about 50 multiply-adds where the 3 x 3
+// products took 200.  (K is symmetric: K^T h = (2r/L - 1) h - (2r/L) u (u.h).)
 
-__device__ __forceinline__ void m3_eye(M3& A, float s)
-{
-#pragma unroll
-    for (int k = 0; k < 9; ++k) A.a[k] = 0.0f;
-    A.a[0] = A.a[4] = A.a[8] = s;
-}
-
-__device__ __forceinline__ void m3_outer_add(M3& A, float s, const float* u, const float* v)
-{
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) A.a[3 * r + c] += s * u[r] * v[c];
-}
-
-// out += s A^T h
-__device__ __forceinline__ void m3_tmul_add(float* out, float s, const M3& A, const float* h)
-{
-#pragma unroll
-    for (int c = 0; c < 3; ++c) out[c] += s * (A.a[c] * h[0] + A.a[3 + c] * h[1] + A.a[6 + c] * h[2]);
-}
-
-__device__ __forceinline__ M3 m3_mul(const M3& A, const M3& B)
-{
-    M3 R;
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-            R.a[3 * r + c] = A.a[3 * r] * B.a[c] + A.a[3 * r + 1] * B.a[3 + c] + A.a[3 * r + 2] * B.a[6 + c];
-    return R;
-}
-
-// F and its Jacobians with respect to rel and e (e_is_normal: SDF, e = n).
-__device__ void fric_jac(const float* rel, const float* e, float ee, bool e_is_normal, float thr_s, float thr_k,
-                         bool mode1, float mu_k, const float* u, float* F, M3& Fr, M3& Fe, bool* kinetic = nullptr)
+// out = F^T-products for the upstream vector h: F and
+//   g_rel = (dF/d rel)^T h,  g_e = (dF/d e)^T h  (e_is_normal: SDF, e = n and
+// g_e = 0 except in mode 1, which the caller adds).
+__device__ __forceinline__ void fric_vjp(const float* rel, const float* e, float ee, bool e_is_normal, float thr_s,
+                                         float thr_k, bool mode1, float mu_k, const float* u, const float* h, float* F,
+                                         float* g_rel, float* g_e, bool* kinetic = nullptr)
 {
     const Tangent tg = tangent_part(rel[0], rel[1], rel[2], e[0], e[1], e[2], ee);
     const float perp[3] = {tg.tx, tg.ty, tg.tz};
-    M3 P, G;
-    m3_eye(P, 1.0f);
-    m3_outer_add(P, -1.0f / ee, e, e);
-#pragma unroll
-    for (int k = 0; k < 9; ++k) G.a[k] = 0.0f;
-    if (!e_is_normal) {
-        const float re = rel[0] * e[0] + rel[1] * e[1] + rel[2] * e[2];
-        m3_outer_add(G, -1.0f / ee, e, rel);
-        G.a[0] -= re / ee;
-        G.a[4] -= re / ee;
-        G.a[8] -= re / ee;
-        m3_outer_add(G, 2.0f * re / (ee * ee), e, e);
-    }
     const float Lp = tg.L;
     const bool clipped = !(Lp < thr_s) && Lp > 0.0f && thr_k / Lp < 1.0f;
     if (kinetic) *kinetic = clipped;
+    // F = s perp; upstream of perp: h, or Q h = (thr_k / L)(h - pu (pu.h))
+    float q[3] = {h[0], h[1], h[2]}, pu_h = 0.0f;
     if (clipped) {
+        const float s = thr_k / Lp;
         const float pu[3] = {perp[0] / Lp, perp[1] / Lp, perp[2] / Lp};
-        M3 Q;
-        m3_eye(Q, thr_k / Lp);
-        m3_outer_add(Q, -thr_k / Lp, pu, pu);
-        F[0] = thr_k * pu[0];
-        F[1] = thr_k * pu[1];
-        F[2] = thr_k * pu[2];
-        Fr = m3_mul(Q, P);
-        Fe = m3_mul(Q, G);
-        if (mode1) m3_outer_add(Fe, -mu_k, pu, u);
+        pu_h = pu[0] * h[0] + pu[1] * h[1] + pu[2] * h[2];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            q[k] = s * (h[k] - pu[k] * pu_h);
+            F[k] = thr_k * pu[k];
+        }
     } else {
-        F[0] = perp[0];
-        F[1] = perp[1];
-        F[2] = perp[2];
-        Fr = P;
-        Fe = G;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) F[k] = perp[k];
+    }
+    // perp = rel - (rel.e / ee) e:  P^T q = q - e (e.q) / ee, and
+    // (d perp / d e)^T q = -(rel (e.q) + q (rel.e)) / ee + 2 (rel.e)(e.q) e / ee^2
+    const float eq = (e[0] * q[0] + e[1] * q[1] + e[2] * q[2]) / ee;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) g_rel[k] = q[k] - eq * e[k];
+    if (!e_is_normal) {
+        const float re = (rel[0] * e[0] + rel[1] * e[1] + rel[2] * e[2]) / ee;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) g_e[k] = 2.0f * re * eq * e[k] - eq * rel[k] - re * q[k];
+        if (clipped && mode1) {   // the threshold 2r - |e| in place of 2r
+#pragma unroll
+            for (int k = 0; k < 3; ++k) g_e[k] -= mu_k * pu_h * u[k];
+        }
     }
 }
 
@@ -600,15 +588,11 @@ __global__ void k_adj_pass(const PbdArgs a, int stab, const float4* __restrict__
             const float u[3] = {g.ex / g.d, g.ey / g.d, g.ez / g.d};
             const float4 hq4 = H[q];
             const float hq[3] = {hq4.x, hq4.y, hq4.z};
-            M3 K;
-            m3_eye(K, d0 / g.d - 1.0f);
-            m3_outer_add(K, -d0 / g.d, u, u);
-            float tv[3] = {0.f, 0.f, 0.f};
-            m3_tmul_add(tv, -mp, K, hp);
-            m3_tmul_add(tv, mq, K, hq);
-            acc[0] -= tv[0];
-            acc[1] -= tv[1];
-            acc[2] -= tv[2];
+            // -K^T (m_q h_q - m_p h_p)
+            const float hF[3] = {mq * hq[0] - mp * hp[0], mq * hq[1] - mp * hp[1], mq * hq[2] - mp * hp[2]};
+            const float kd = d0 / g.d, uF = kd * (u[0] * hF[0] + u[1] * hF[1] + u[2] * hF[2]);
+#pragma unroll
+            for (int k2 = 0; k2 < 3; ++k2) acc[k2] -= (kd - 1.0f) * hF[k2] - uF * u[k2];
             const float uh = u[0] * (hp[0] + hq[0]) + u[1] * (hp[1] + hq[1]) + u[2] * (hp[2] + hq[2]);
             gw += -pen * (wq / (W * W)) * uh;
             if (!stab) {
@@ -616,17 +600,12 @@ __global__ void k_adj_pass(const PbdArgs a, int stab, const float4* __restrict__
                 const float rel[3] = {(xtp.x - xfp.x) - (xtq.x - xfq.x), (xtp.y - xfp.y) - (xtq.y - xfq.y),
                                       (xtp.z - xfp.z) - (xtq.z - xfq.z)};
                 const float base = sc.friction_mode == 1 ? pen : d0;
-                float F[3];
-                M3 Fr, Fe;
+                float F[3], grel[3], ge[3];
                 bool kin = false;
-                fric_jac(rel, e, g.d2, false, base * sc.mu_s, base * sc.mu_k, sc.friction_mode == 1, sc.mu_k, u, F, Fr,
-                         Fe, &kin);
+                fric_vjp(rel, e, g.d2, false, base * sc.mu_s, base * sc.mu_k, sc.friction_mode == 1, sc.mu_k, u, hF, F,
+                         grel, ge, &kin);
                 if (rb && kin) *rb |= 2;
-                const float hF[3] = {-mp * hp[0] + mq * hq[0], -mp * hp[1] + mq * hq[1], -mp * hp[2] + mq * hq[2]};
-                float grel[3] = {0.f, 0.f, 0.f}, ge[3] = {0.f, 0.f, 0.f};
-                m3_tmul_add(grel, 1.0f, Fr, hF);
-                m3_tmul_add(ge, 1.0f, Fe, hF);
-    #pragma unroll
+#pragma unroll
                 for (int k2 = 0; k2 < 3; ++k2) {
                     acc[k2] += grel[k2] - ge[k2];
                     accx[k2] -= grel[k2];
@@ -659,17 +638,14 @@ __global__ void k_adj_pass(const PbdArgs a, int stab, const float4* __restrict__
                         const float dv[3] = {(xtp.x - xfp.x) - b.vel[0] * a.dt, (xtp.y - xfp.y) - b.vel[1] * a.dt,
                                              (xtp.z - xfp.z) - b.vel[2] * a.dt};
                         const float base = sc.friction_mode == 1 ? pen : d0;
-                        float F[3];
-                        M3 Fr, Fe;
+                        float F[3], gd[3], ge[3];
                         bool kin = false;
-                        fric_jac(dv, n, 1.0f, true, base * bmu_s, base * bmu_k, false, bmu_k, n, F, Fr, Fe, &kin);
+                        fric_vjp(dv, n, 1.0f, true, base * bmu_s, base * bmu_k, false, bmu_k, n, hp, F, gd, ge, &kin);
                         if (sb && kin) *sb |= 2;
-                        float gd[3] = {0.f, 0.f, 0.f};
-                        m3_tmul_add(gd, -1.0f, Fr, hp);
-    #pragma unroll
+#pragma unroll
                         for (int k2 = 0; k2 < 3; ++k2) {
-                            acc[k2] += gd[k2];
-                            accx[k2] -= gd[k2];
+                            acc[k2] -= gd[k2];
+                            accx[k2] += gd[k2];
                         }
                         if (sc.friction_mode == 1) {
                             const Tangent tg = tangent_part(dv[0], dv[1], dv[2], n[0], n[1], n[2], 1.0f);
@@ -747,7 +723,7 @@ cudaError_t gs_launch_upsample_bwd(cudaStream_t s, const SceneDev* scenes, const
                                    const uint32_t* lr_idx, float4* coef, const uint32_t* order, float4* pos_sorted)
 {
     if (m <= 0) return cudaSuccess;
-    k_upsample_bwd<<<gs_blocks(m * kBwdLanes, 128), 128, 0, s>>>(scenes, sdf, lr_spos, lr_svel, cell_start, hx, hv, gxo, gvo, ghx,
+    k_upsample_bwd<<<gs_blocks(m * kBwdLanes, kBwdThreads), kBwdThreads, 0, s>>>(scenes, sdf, lr_spos, lr_svel, cell_start, hx, hv, gxo, gvo, ghx,
                                                       ghv, gXs, gVs, m, dt, rec, lr_idx, coef, order, pos_sorted);
     *launches += 1;
     return cudaGetLastError();
