@@ -3,7 +3,7 @@
 // frame with respect to the LR positions and velocities and the HR state
 // before the frame.
 //
-// One thread per HR particle recomputes the forward pass of its particle
+// Four lanes per HR particle recompute the forward pass of their particle
 // (weights, blend case, the LR particle of largest weight, SDF contacts) and
 // then applies the chain rule backwards for those branch decisions:
 //   SDF steps (last first), normal held fixed:  g <- g - n (n . g)
@@ -16,10 +16,11 @@
 //        g_w_j = g_S + g_V . V_j + [j = argmax] g_wmax
 //        g_X_j += g_w_j 6 t^2 (x - X_j) / 9r^2,  g_x -= the same,
 //        g_V_j += w_j g_V
-// LR gradients are summed in cell order with atomics and then scattered back
-// to the original LR order.
+// LR gradients are summed in cell order, over a warp's HR particles first and
+// with atomics from there, and then scattered back to the original LR order.
 #include <cuda_runtime.h>
 
+#include "grid.cuh"
 #include "gs_internal.cuh"
 #include "pbd_common.cuh"
 #include "sdf.cuh"
@@ -42,14 +43,40 @@ constexpr int kBwdThreads = 128;
 // of the 60 to 130 candidates of an HR particle are, 3 or 4 per lane); a lane
 // with more walks its candidates again.
 constexpr int kBwdHits = 16;
+// LR particles staged per warp: 32 per lane, so that a lane's hits are a bit
+// mask.  The eight HR particles of a warp, children of one LR particle, have
+// 35 to 60 in reach together.
+constexpr int kBwdStage = 128;
+constexpr uint32_t kBwdWalk = 512;   // candidates a warp looks at for that
+
+// Shared memory of a warp.
+struct BwdShared {
+    union {
+        float4 pos[kBwdStage];            // staged LR positions, w = slot
+        uint32_t hit[kBwdHits][32];       // the general path's
+    };
+    float4 vel[kBwdStage];
+    float4 hr_p[32 / kBwdLanes];          // HR position, g_S
+    float4 hr_g[32 / kBwdLanes];          // g_V, g_wmax
+    uint32_t hr_j[32 / kBwdLanes];        // slot of the largest weight
+    uint32_t rows[32];
+};
 
 // rec (optional): the decisions this reverse mode differentiates, four words
 // per HR particle: the LR particle of largest weight (original index through
 // lr_idx, or all ones), the blend case (1: alpha = 1 - max w), bit c = SDF
 // component c in contact, bit c = normal velocity removed at component c.
-// Instruction issue bounds it (12,600 warp instructions per 32 HR particles
-// when the second half walked every candidate again, 6,600 now; 64,000 HR: 46
-// us, now 34).
+// A warp whose HR particles lie together (callers keep the children of an LR
+// particle side by side) stages the LR particles around their box once, as
+// the forward gather does, evaluates from there, and sums an LR particle's
+// gradients over its eight HR particles in the lane that owns it: one pair of
+// atomics per staged LR particle.  A warp with more rows of cells than lanes,
+// or more candidates than the stage holds (scattered or heavily compressed
+// HR), walks the rows lane by lane and takes an atomic pair per HR and LR
+// particle.  The dependent chain of a warp's phases bounds it (24 warps per SM,
+// a third of the issue slots; without its atomics it is no faster).  Rollout of
+// 30 steps with its reverse, 4,000 LR / 64,000 HR: 4.06 -> 3.93 ms; a stirred
+// set of that size, where a fifth of the HR lie apart, 34 -> 35 us by itself.
 __global__ void __launch_bounds__(kBwdThreads, 6) k_upsample_bwd(const SceneDev* __restrict__ scenes, const gs_sdf* __restrict__ sdf,
                                const float4* __restrict__ lr_spos, const float4* __restrict__ lr_svel,
                                const uint32_t* __restrict__ cell_start, const float4* __restrict__ hx,
@@ -67,8 +94,10 @@ __global__ void __launch_bounds__(kBwdThreads, 6) k_upsample_bwd(const SceneDev*
     // particles are taken in the order `order` (slot -> particle), and the
     // coefficients and the position go to the slot (coef[2 slot ..],
     // pos_sorted[slot]) instead of any atomic.
-    __shared__ uint32_t s_hit[kBwdHits][kBwdThreads];
-    int n_hit = 0;
+    __shared__ BwdShared s_warp[kBwdThreads / 32];
+    BwdShared& sh = s_warp[threadIdx.x >> 5];
+    const int lane = (int)(threadIdx.x & 31u);
+    constexpr unsigned kAll = 0xffffffffu;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t slot = t / kBwdLanes;
     const int sub = (int)(t % kBwdLanes);
@@ -84,33 +113,112 @@ __global__ void __launch_bounds__(kBwdThreads, 6) k_upsample_bwd(const SceneDev*
     const int cx0 = cell_of(p.x - R, g.ox, g.inv_h, g.dx), cx1 = cell_of(p.x + R, g.ox, g.inv_h, g.dx);
     const int cy0 = cell_of(p.y - R, g.oy, g.inv_h, g.dy), cy1 = cell_of(p.y + R, g.oy, g.inv_h, g.dy);
     const int cz0 = cell_of(p.z - R, g.oz, g.inv_h, g.dz), cz1 = cell_of(p.z + R, g.oz, g.inv_h, g.dz);
+    // stage the LR particles around the warp's HR particles, in slot order
+    int staged = -1;   // how many, or -1: the general path
+    {
+        const unsigned lt = (1u << lane) - 1u, le = (lt << 1) | 1u;
+        const int x0 = __reduce_min_sync(kAll, live ? cx0 : g.dx), x1 = __reduce_max_sync(kAll, live ? cx1 : -1);
+        const int y0 = __reduce_min_sync(kAll, live ? cy0 : g.dy), y1 = __reduce_max_sync(kAll, live ? cy1 : -1);
+        const int z0 = __reduce_min_sync(kAll, live ? cz0 : g.dz), z1 = __reduce_max_sync(kAll, live ? cz1 : -1);
+        const int ny = y1 - y0 + 1, nz = z1 - z0 + 1;
+        if (x1 >= 0 && ny <= 32 && nz <= 32 && ny * nz <= 32) {   // warp-uniform
+            uint32_t rb = 0, len = 0;   // lane j: row j
+            if (lane < ny * nz) {
+                const int64_t row = (int64_t)sc.cell_off + ((int64_t)(z0 + lane / ny) * g.dy + (y0 + lane % ny)) * g.dx;
+                rb = __ldg(cell_start + row + x0);
+                len = __ldg(cell_start + row + x1 + 1) - rb;
+            }
+            uint32_t incl = len;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(kAll, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const uint32_t excl = incl - len, total = __shfl_sync(kAll, incl, 31);
+            if (total <= kBwdWalk) {
+                const float lx = ord2f(__reduce_min_sync(kAll, f2ord(live ? p.x : 3.0e38f)));
+                const float ly = ord2f(__reduce_min_sync(kAll, f2ord(live ? p.y : 3.0e38f)));
+                const float lz = ord2f(__reduce_min_sync(kAll, f2ord(live ? p.z : 3.0e38f)));
+                const float hx_ = ord2f(__reduce_max_sync(kAll, f2ord(live ? p.x : -3.0e38f)));
+                const float hy_ = ord2f(__reduce_max_sync(kAll, f2ord(live ? p.y : -3.0e38f)));
+                const float hz_ = ord2f(__reduce_max_sync(kAll, f2ord(live ? p.z : -3.0e38f)));
+                const float R2p = R2 * 1.0001f;   // padded against rounding
+                // rows that hold any, in order: flat index f of the t-th is slot f + rows[t]
+                const unsigned some = __ballot_sync(kAll, len != 0u);
+                if (len != 0u) sh.rows[__popc(some & lt)] = rb - excl;
+                __syncwarp();
+                int before = 0, cnt = 0;
+                for (uint32_t base = 0; base < total; base += 32) {
+                    const uint32_t off = excl - base, f = base + (uint32_t)lane;
+                    const unsigned starts = __reduce_or_sync(kAll, len != 0u && off < 32u ? 1u << off : 0u);
+                    const int r = before + __popc(starts & le) - 1;
+                    before += __popc(starts);
+                    bool take = false;
+                    uint32_t j = 0;
+                    float4 q = zero4;
+                    if (f < total) {
+                        j = f + sh.rows[r];
+                        q = __ldg(lr_spos + j);
+                        const float ex = fmaxf(fmaxf(lx - q.x, q.x - hx_), 0.0f);
+                        const float ey = fmaxf(fmaxf(ly - q.y, q.y - hy_), 0.0f);
+                        const float ez = fmaxf(fmaxf(lz - q.z, q.z - hz_), 0.0f);
+                        take = ex * ex + ey * ey + ez * ez < R2p;
+                    }
+                    const unsigned bal = __ballot_sync(kAll, take);
+                    const int k = cnt + __popc(bal & lt);
+                    cnt += __popc(bal);
+                    if (take && k < kBwdStage) {
+                        sh.pos[k] = make_float4(q.x, q.y, q.z, __uint_as_float(j));
+                        sh.vel[k] = __ldg(lr_svel + j);
+                    }
+                }
+                if (cnt <= kBwdStage) staged = cnt;
+                __syncwarp();   // staged; or the hits below take the stage's place
+            }
+        }
+    }
     // forward
     float S = 0.f, Vx = 0.f, Vy = 0.f, Vz = 0.f, wmax = 0.f;
     uint32_t jstar = 0xffffffffu;
-    for (int cz = cz0; live && cz <= cz1; ++cz)
-        for (int cy = cy0; cy <= cy1; ++cy) {
-            const int64_t row = (int64_t)sc.cell_off + ((int64_t)cz * g.dy + cy) * g.dx;
-            const uint32_t b = cell_start[row + cx0], e = cell_start[row + cx1 + 1];
-            for (uint32_t j = b + sub; j < e; j += kBwdLanes) {
-                const float4 q = lr_spos[j];
-                const float dx = p.x - q.x, dy = p.y - q.y, dz = p.z - q.z;
-                const float d2 = dx * dx + dy * dy + dz * dz;
-                if (!(d2 < R2)) continue;
-                const float t = 1.0f - d2 * inv9r2;
-                const float w = t * t * t;
-                const float4 qv = lr_svel[j];
-                if (n_hit < kBwdHits) s_hit[n_hit][threadIdx.x] = j;
-                ++n_hit;
-                S += w;
-                Vx += w * qv.x;
-                Vy += w * qv.y;
-                Vz += w * qv.z;
-                if (w > wmax) {
-                    wmax = w;
-                    jstar = j;
+    uint32_t hits = 0u;   // staged: bit b is the lane's b-th candidate
+    int n_hit = 0;        // general path
+    auto weigh = [&](float d2, const float4& qv, uint32_t j) {
+        const float t = 1.0f - d2 * inv9r2;
+        const float w = t * t * t;
+        S += w;
+        Vx += w * qv.x;
+        Vy += w * qv.y;
+        Vz += w * qv.z;
+        if (w > wmax) {
+            wmax = w;
+            jstar = j;
+        }
+    };
+    if (staged >= 0) {
+        for (int k = sub; live && k < staged; k += kBwdLanes) {
+            const float4 q = sh.pos[k];
+            const float dx = p.x - q.x, dy = p.y - q.y, dz = p.z - q.z;
+            const float d2 = dx * dx + dy * dy + dz * dz;
+            if (!(d2 < R2)) continue;
+            hits |= 1u << (k / kBwdLanes);
+            weigh(d2, sh.vel[k], __float_as_uint(q.w));
+        }
+    } else {
+        for (int cz = cz0; live && cz <= cz1; ++cz)
+            for (int cy = cy0; cy <= cy1; ++cy) {
+                const int64_t row = (int64_t)sc.cell_off + ((int64_t)cz * g.dy + cy) * g.dx;
+                const uint32_t b = cell_start[row + cx0], e = cell_start[row + cx1 + 1];
+                for (uint32_t j = b + sub; j < e; j += kBwdLanes) {
+                    const float4 q = lr_spos[j];
+                    const float dx = p.x - q.x, dy = p.y - q.y, dz = p.z - q.z;
+                    const float d2 = dx * dx + dy * dy + dz * dz;
+                    if (!(d2 < R2)) continue;
+                    if (n_hit < kBwdHits) sh.hit[n_hit][lane] = j;
+                    ++n_hit;
+                    weigh(d2, lr_svel[j], j);
                 }
             }
-        }
+    }
     // the lanes' sums; the largest weight with the lowest slot among equals
     // (the first one met in slot order)
 #pragma unroll
@@ -197,21 +305,76 @@ __global__ void __launch_bounds__(kBwdThreads, 6) k_upsample_bwd(const SceneDev*
     const float galpha = gvpx * (bx - vtx) + gvpy * (by - vty) + gvpz * (bz - vtz);
     const float gwmax = branch ? -galpha : 0.0f;
     if (live && sub == 0) ghv[i] = make_float4(alpha * gvpx, alpha * gvpy, alpha * gvpz, 0.0f);
-    if (live && S > 0.0f) {
-        const float gVx = gvtx / S, gVy = gvty / S, gVz = gvtz / S;
-        const float gS = -(gvtx * vtx + gvty * vty + gvtz * vtz) / S;
+    const bool spread = live && S > 0.0f;
+    const float gVx = spread ? gvtx / S : 0.f, gVy = spread ? gvty / S : 0.f, gVz = spread ? gvtz / S : 0.f;
+    const float gS = spread ? -(gvtx * vtx + gvty * vty + gvtz * vtz) / S : 0.f;
+    // dL/dw_j 6 t^2 / 9r^2 of LR particle j at squared distance d2
+    auto slope = [&](float d2, const float4& qv, uint32_t j, float gs, float gvx, float gvy, float gvz, float gwm,
+                     uint32_t js) {
+        const float t = 1.0f - d2 * inv9r2;
+        const float gwj = gs + gvx * qv.x + gvy * qv.y + gvz * qv.z + (j == js ? gwm : 0.0f);
+        return gwj * 6.0f * t * t * inv9r2;
+    };
+    if (staged >= 0) {
+        if (spread) {
+            while (hits) {
+                const int k = (__ffs(hits) - 1) * kBwdLanes + sub;
+                hits &= hits - 1u;
+                const float4 q = sh.pos[k];
+                const float dx = p.x - q.x, dy = p.y - q.y, dz = p.z - q.z;
+                const float k6 = slope(dx * dx + dy * dy + dz * dz, sh.vel[k], __float_as_uint(q.w), gS, gVx, gVy, gVz,
+                                       gwmax, jstar);
+                gpx -= k6 * dx;
+                gpy -= k6 * dy;
+                gpz -= k6 * dz;
+            }
+        }
+        if (!coef) {   // a lane per staged LR particle sums over the warp's HR particles
+            if (sub == 0) {
+                const int h = lane / kBwdLanes;
+                sh.hr_p[h] = spread ? make_float4(p.x, p.y, p.z, gS) : make_float4(1.0e18f, 1.0e18f, 1.0e18f, 0.f);
+                sh.hr_g[h] = make_float4(gVx, gVy, gVz, gwmax);
+                sh.hr_j[h] = jstar;
+            }
+            __syncwarp();
+            for (int k = lane; k < staged; k += 32) {
+                const float4 q = sh.pos[k], qv = sh.vel[k];
+                const uint32_t j = __float_as_uint(q.w);
+                float ax_ = 0.f, ay_ = 0.f, az_ = 0.f, bx_ = 0.f, by_ = 0.f, bz_ = 0.f;
+                bool any = false;
+#pragma unroll 2
+                for (int h = 0; h < 32 / kBwdLanes; ++h) {
+                    const float4 P = sh.hr_p[h];
+                    const float dx = P.x - q.x, dy = P.y - q.y, dz = P.z - q.z;
+                    const float d2 = dx * dx + dy * dy + dz * dz;
+                    if (!(d2 < R2)) continue;
+                    any = true;
+                    const float4 G = sh.hr_g[h];
+                    const float k6 = slope(d2, qv, j, P.w, G.x, G.y, G.z, G.w, sh.hr_j[h]);
+                    const float t = 1.0f - d2 * inv9r2, w = t * t * t;
+                    ax_ += k6 * dx;
+                    ay_ += k6 * dy;
+                    az_ += k6 * dz;
+                    bx_ += w * G.x;
+                    by_ += w * G.y;
+                    bz_ += w * G.z;
+                }
+                if (any) {   // one vector reduction per gradient (global float4 atomics, sm_90 and later)
+                    atomicAdd(gXs + j, make_float4(ax_, ay_, az_, 0.0f));
+                    atomicAdd(gVs + j, make_float4(bx_, by_, bz_, 0.0f));
+                }
+            }
+        }
+    } else if (spread) {
         // the gradients of LR particle j (in reach)
         auto push = [&](uint32_t j) {
             const float4 q = lr_spos[j];
             const float dx = p.x - q.x, dy = p.y - q.y, dz = p.z - q.z;
             const float d2 = dx * dx + dy * dy + dz * dz;
             if (!(d2 < R2)) return;
-            const float t = 1.0f - d2 * inv9r2;
-            const float w = t * t * t;
-            const float4 qv = lr_svel[j];
-            const float gwj = gS + gVx * qv.x + gVy * qv.y + gVz * qv.z + (j == jstar ? gwmax : 0.0f);
-            const float k6 = gwj * 6.0f * t * t * inv9r2;
-            if (!coef) {   // one vector reduction per gradient (global float4 atomics, sm_90 and later)
+            const float k6 = slope(d2, lr_svel[j], j, gS, gVx, gVy, gVz, gwmax, jstar);
+            if (!coef) {
+                const float t = 1.0f - d2 * inv9r2, w = t * t * t;
                 atomicAdd(gXs + j, make_float4(k6 * dx, k6 * dy, k6 * dz, 0.0f));
                 atomicAdd(gVs + j, make_float4(w * gVx, w * gVy, w * gVz, 0.0f));
             }
@@ -220,7 +383,7 @@ __global__ void __launch_bounds__(kBwdThreads, 6) k_upsample_bwd(const SceneDev*
             gpz -= k6 * dz;
         };
         if (n_hit <= kBwdHits) {
-            for (int h = 0; h < n_hit; ++h) push(s_hit[h][threadIdx.x]);
+            for (int h = 0; h < n_hit; ++h) push(sh.hit[h][lane]);
         } else {
             for (int cz = cz0; cz <= cz1; ++cz)
                 for (int cy = cy0; cy <= cy1; ++cy) {

@@ -29,3 +29,16 @@ __device__ __forceinline__ uint32_t grid_cell_of(const SceneDev& sc, float x, fl
     return sc.cell_off +
            ((uint32_t)(sz >> 1) * (uint32_t)g.dy + (uint32_t)(sy >> 1)) * (uint32_t)g.dx + (uint32_t)(sx >> 1);
 }
+
+// Order-preserving map of non-NaN floats onto unsigned integers (and back),
+// so that a warp's minimum or maximum of a float is one integer reduction.
+__device__ __forceinline__ unsigned f2ord(float f)
+{
+    const unsigned u = __float_as_uint(f);
+    return u ^ ((u & 0x80000000u) ? 0xffffffffu : 0x80000000u);
+}
+
+__device__ __forceinline__ float ord2f(unsigned u)
+{
+    return __uint_as_float(u ^ ((u & 0x80000000u) ? 0x80000000u : 0xffffffffu));
+}

@@ -27,6 +27,7 @@
 
 #include <algorithm>
 
+#include "grid.cuh"
 #include "gs_internal.cuh"
 #include "sdf.cuh"
 
@@ -100,19 +101,6 @@ __device__ __forceinline__ void hr_boundary(float& x, float& y, float& z, float&
             }
         }
     }
-}
-
-// Order-preserving map of non-NaN floats onto unsigned integers (and back),
-// so that a warp's minimum or maximum of a float is one integer reduction.
-__device__ __forceinline__ unsigned f2ord(float f)
-{
-    const unsigned u = __float_as_uint(f);
-    return u ^ ((u & 0x80000000u) ? 0xffffffffu : 0x80000000u);
-}
-
-__device__ __forceinline__ float ord2f(unsigned u)
-{
-    return __uint_as_float(u ^ ((u & 0x80000000u) ? 0x80000000u : 0xffffffffu));
 }
 
 // Lanes whose sub-cells (side h/2) are within one of the group leader's are
