@@ -415,7 +415,6 @@ int create_impl(int S, const gs_scene* scenes, const float* r_low, const float* 
     int coop = 0;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c->device);
     if (e == cudaSuccess && coop) c->solve_blocks = gs_solve_blocks(c->sm_count);
-    if (e == cudaSuccess) c->cluster_passes = gs_cluster_passes_available();
     if (e != cudaSuccess) {
         delete c;
         return GS_ERR_CUDA;
@@ -882,13 +881,7 @@ int step_low_io(gs_ctx* c, const StepIo& io, float dt, int iters, const float* d
     } else {
         // the last pass also finalizes (v = (x~ - x) / dt, x = x~, original order)
         const int total = c->n_stab + iters;
-        const bool one_launch = c->cluster_passes && gs_cluster_passes_fit(a);
-        if (one_launch)
-            CK(gs_launch_passes(c->stream, a, PassSeq{c->n_stab, total, c->s_x[0], c->s_x[1], c->s_xt[0], c->s_xt[1]},
-                                c->nbr, c->nbr_cnt, &c->launches, c->lr_vals[1], io.xo, io.vo, io.x,
-                                next_bins(c, next)),
-               "passes");
-        for (int it = 0; it < total && !one_launch; ++it) {
+        for (int it = 0; it < total; ++it) {
             const int stab = it < c->n_stab;
             const bool last = it + 1 == total;
             if (c->n_bodies > 0 && !stab)   // the bodies' transforms from this pass's x~
@@ -2728,14 +2721,7 @@ static int step_low_record_into(gs_ctx* c, const StepIo& io, float dt, int iters
     const PbdArgs a = pbd_args(c, dt);
     int st = step_begin(c, a, io, X, XT, c->step_cell_start, nbr, cnt, idx, true);
     if (st) return st;
-    const bool one_launch = c->cluster_passes && gs_cluster_passes_fit(a);
-    if (one_launch) {
-        const bool fin = final_state && iters > 0;
-        CK(gs_launch_passes(c->stream, a, PassSeq{c->n_stab, total, X, nullptr, XT, nullptr}, nbr, cnt, &c->launches,
-                            fin ? idx : nullptr, fin ? io.xo : nullptr, fin ? io.vo : nullptr, io.x),
-           "passes");
-    }
-    for (int it = 0; it < total && !one_launch; ++it) {
+    for (int it = 0; it < total; ++it) {
         const int stab = it < c->n_stab;
         const bool fin = final_state && iters > 0 && it + 1 == total;
         CK(gs_launch_pass(c->stream, a, stab, X + (size_t)std::min(it, c->n_stab) * N, XT + (size_t)it * N,

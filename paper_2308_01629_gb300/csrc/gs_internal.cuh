@@ -297,7 +297,6 @@ struct gs_ctx {
     int* d_err = nullptr;
     unsigned* d_bar = nullptr;   // grid-barrier words of the persistent LR solver
     int solve_blocks = 0;        // resident blocks of the solver; 0 = per-pass launches
-    bool cluster_passes = false; // small sets: all passes of a step in one cluster
     bool use_solver = false;    // per-pass launches by default: faster under graph replay
     bool solver_selftest = false;   // the barrier waits for one block that does not exist
     int* h_err = nullptr;                         // pinned
@@ -491,21 +490,6 @@ cudaError_t gs_launch_pass(cudaStream_t s, const PbdArgs& a, int stab, const flo
                            int64_t* launches, const uint32_t* fin_idx = nullptr, float4* fin_pos = nullptr,
                            float4* fin_vel = nullptr, const float4* fin_w = nullptr, unsigned* fin_rate = nullptr,
                            const NextBins& next = NextBins{});
-// All passes of a step in one launch, for small sets without bodies and with
-// the step length known on the host (gs_cluster_passes_fit) where the device
-// takes the cluster.  x before pass it is the buffer min(it, n_stab) of x,
-// x~ the buffer it of xt: alternating with the other one where x_other /
-// xt_other are given, else n particles apart.  fin_idx as in gs_launch_pass.
-struct PassSeq {
-    int n_stab, total;
-    float4 *x, *x_other, *xt, *xt_other;
-};
-bool gs_cluster_passes_available();
-bool gs_cluster_passes_fit(const PbdArgs& a);
-cudaError_t gs_launch_passes(cudaStream_t s, const PbdArgs& a, const PassSeq& q, const uint32_t* nbr,
-                             const uint32_t* cnt, int64_t* launches, const uint32_t* fin_idx = nullptr,
-                             float4* fin_pos = nullptr, float4* fin_vel = nullptr, const float4* fin_w = nullptr,
-                             const NextBins& next = NextBins{});
 // Prediction + cell keys + arrival ranks (the counting stage of the binning).
 cudaError_t gs_launch_predict_keys(cudaStream_t s, const PbdArgs& a, const float4* pos, const float4* vel,
                                    float4* xt, uint32_t* keys, uint32_t* rank, uint32_t* cnt, int64_t* launches);

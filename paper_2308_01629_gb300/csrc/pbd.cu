@@ -707,53 +707,6 @@ __global__ void __launch_bounds__(128, 6) k_solve(const SolveArgs s)
     }
 }
 
-// ---- all passes of a small set's step in one cluster -----------------------
-// A pass of a small set is a launch and a few round trips to L2.  Up to
-// kClusterMax particles fit one cluster of 16 blocks at eight lanes each, and
-// the hardware's cluster barrier separates the passes (its release and
-// acquire order the weak loads and stores of the position buffers; ld_pos
-// keeps them off the non-coherent path).  Same lanes, same order, same bits
-// as k_pass.  Frame of the cube of 1,000 LR (four steps of six passes): 69.4 ->
-// 65.5 us.  The cluster's 16 SMs bound it there (a pass is 250 warps, four per
-// scheduler), so a set that needs a second round of warps keeps its launches.
-constexpr int kClusterThreads = 512;
-constexpr int kClusterLanes = 8;
-constexpr int64_t kClusterMax = 16 * kClusterThreads / kClusterLanes;
-constexpr size_t kClusterShared = (size_t)(kClusterThreads / 32) * sizeof(PassShared);
-
-__device__ __forceinline__ float4* seq_buf(float4* first, float4* second, int64_t n, int k)
-{
-    return second ? (k & 1 ? second : first) : first + (int64_t)k * n;
-}
-
-template <bool kMat, bool kSingle>
-__global__ void __launch_bounds__(kClusterThreads, 1) k_passes(const PbdArgs a, const PassSeq q,
-                                                               const uint32_t* __restrict__ nbr,
-                                                               const uint32_t* __restrict__ cnt, const FinalOut fin)
-{
-    extern __shared__ __align__(16) unsigned char s_raw[];
-    PassShared& sh = reinterpret_cast<PassShared*>(s_raw)[threadIdx.x >> 5];
-    constexpr int kPer = 32 / kClusterLanes;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const int64_t p_first = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kPer;
-    for (int it = 0; it < q.total; ++it) {
-        const int stab = it < q.n_stab, kx = min(it, q.n_stab);
-        const float4 *xi = seq_buf(q.x, q.x_other, a.n, kx), *ti = seq_buf(q.xt, q.xt_other, a.n, it);
-        float4 *xo = seq_buf(q.x, q.x_other, a.n, kx + 1), *to = seq_buf(q.xt, q.xt_other, a.n, it + 1);
-        const bool last = fin.idx && it + 1 == q.total;
-        for (int64_t p0 = p_first; p0 < a.n; p0 += warps * kPer) {
-            if (last)
-                pass_warp<kClusterLanes, true, kMat, false, kSingle, true>(a, stab, p0, sh, xi, ti, xo, to, nbr, cnt, fin);
-            else
-                pass_warp<kClusterLanes, true, kMat, false, kSingle, false>(a, stab, p0, sh, xi, ti, xo, to, nbr, cnt);
-        }
-        if (it + 1 < q.total) {
-            __syncwarp();
-            asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-        }
-    }
-}
-
 __global__ void k_finalize(const PbdArgs a, const uint32_t* __restrict__ idx, const float4* __restrict__ s_x,
                            const float4* __restrict__ s_xt, float4* pos, float4* __restrict__ vel,
                            const float4* w_src, unsigned* rate)
@@ -1030,62 +983,6 @@ cudaError_t gs_launch_pass(cudaStream_t s, const PbdArgs& a, int stab, const flo
     else launch_pass<2>(s, a, stab, x_in, xt_in, x_out, xt_out, nbr, cnt, fin);
     *launches += 1;
     return cudaGetLastError();
-}
-
-namespace {
-
-struct ClusterLaunch {
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr = {};
-    ClusterLaunch(cudaStream_t s, unsigned blocks)
-    {
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = blocks;
-        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-        cfg.gridDim = dim3(blocks);
-        cfg.blockDim = dim3(kClusterThreads);
-        cfg.dynamicSmemBytes = kClusterShared;
-        cfg.stream = s;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-    }
-};
-
-}  // namespace
-
-// Whether the device takes k_passes' largest cluster (16 blocks need the
-// opt-in beyond the portable eight); called once per context.
-bool gs_cluster_passes_available()
-{
-    auto ready = [](auto kernel) {
-        int clusters = 0;
-        ClusterLaunch l(nullptr, 16);
-        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterShared) ==
-                   cudaSuccess &&
-               cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-               cudaOccupancyMaxActiveClusters(&clusters, kernel, &l.cfg) == cudaSuccess && clusters > 0;
-    };
-    const bool ok = ready(k_passes<false, false>) && ready(k_passes<false, true>) && ready(k_passes<true, false>) &&
-                    ready(k_passes<true, true>);
-    if (!ok) cudaGetLastError();
-    return ok;
-}
-
-bool gs_cluster_passes_fit(const PbdArgs& a) { return a.n <= kClusterMax && !a.body && !a.dt_dev; }
-
-cudaError_t gs_launch_passes(cudaStream_t s, const PbdArgs& a, const PassSeq& q, const uint32_t* nbr,
-                             const uint32_t* cnt, int64_t* launches, const uint32_t* fin_idx, float4* fin_pos,
-                             float4* fin_vel, const float4* fin_w, const NextBins& next)
-{
-    if (a.n <= 0 || q.total <= 0) return cudaSuccess;
-    const FinalOut fin{fin_idx, fin_pos, fin_vel, fin_w, nullptr, next};
-    ClusterLaunch l(s, gs_blocks(a.n * kClusterLanes, kClusterThreads));
-    *launches += 1;
-    if (a.n_scenes == 1)
-        return a.mu_cross ? cudaLaunchKernelEx(&l.cfg, k_passes<true, true>, a, q, nbr, cnt, fin)
-                          : cudaLaunchKernelEx(&l.cfg, k_passes<false, true>, a, q, nbr, cnt, fin);
-    return a.mu_cross ? cudaLaunchKernelEx(&l.cfg, k_passes<true, false>, a, q, nbr, cnt, fin)
-                      : cudaLaunchKernelEx(&l.cfg, k_passes<false, false>, a, q, nbr, cnt, fin);
 }
 
 int gs_solve_blocks(int sm_count)
