@@ -56,8 +56,8 @@ FLUSH_BYTES = 512 << 20
 # DRAM bytes of one upsampling launch on this workload, and its DRAM, SM and
 # issue utilisation, from an ncu capture of the kernel source with this hash
 # (profiles/); reported only while the source is unchanged.
-TRAFFIC_CAPTURE = {"source_sha1": "6be7d4f2f05b84c922ae0661ecf4df758ad19515", "bytes": 82662400,
-                   "dram_throughput_pct": 6.8, "sm_throughput_pct": 59.1, "issue_active_pct": 62.2}
+TRAFFIC_CAPTURE = {"source_sha1": "9024c95ff09a363a6c48ec63cde3b88ea4c2ac90", "bytes": 73041664,
+                   "dram_throughput_pct": 7.5, "sm_throughput_pct": 69.9, "issue_active_pct": 73.6}
 
 
 class L2Flush:
