@@ -43,11 +43,13 @@ constexpr int kBwdThreads = 128;
 // of the 60 to 130 candidates of an HR particle are, 3 or 4 per lane); a lane
 // with more walks its candidates again.
 constexpr int kBwdHits = 16;
-// LR particles staged per warp: 32 per lane, so that a lane's hits are a bit
-// mask.  The eight HR particles of a warp, children of one LR particle, have
-// 35 to 60 in reach together.
-constexpr int kBwdStage = 128;
-constexpr uint32_t kBwdWalk = 512;   // candidates a warp looks at for that
+// LR particles staged per warp, 16 per lane, whose hits are a bit mask.  The
+// eight HR particles of a warp, children of one LR particle, have 35 to 60
+// around them, out of 90 to 150 in the cells: groups with more lie apart and
+// gain nothing (a stage of 128 out of 512 candidates: 74.2 us where 64 out of
+// 192 take 73.0, and 6 % on 1,200 HR in random order).
+constexpr int kBwdStage = 64;
+constexpr uint32_t kBwdWalk = 192;   // candidates a warp looks at for that
 
 // Shared memory of a warp.
 struct BwdShared {
@@ -74,9 +76,9 @@ struct BwdShared {
 // or more candidates than the stage holds (scattered or heavily compressed
 // HR), walks the rows lane by lane and takes an atomic pair per HR and LR
 // particle.  The dependent chain of a warp's phases bounds it (24 warps per SM,
-// a third of the issue slots; without its atomics it is no faster).  Rollout of
-// 30 steps with its reverse, 4,000 LR / 64,000 HR: 4.06 -> 3.93 ms; a stirred
-// set of that size, where a fifth of the HR lie apart, 34 -> 35 us by itself.
+// a third of the issue slots; without its atomics it is no faster).  The whole
+// reverse call, HR by parent: 120,000 HR 80.5 -> 73.0 us, 1,200 HR 30.8 ->
+// 28.8; in random order 111.9 -> 113.7 and 30.8 -> 30.8.
 __global__ void __launch_bounds__(kBwdThreads, 6) k_upsample_bwd(const SceneDev* __restrict__ scenes, const gs_sdf* __restrict__ sdf,
                                const float4* __restrict__ lr_spos, const float4* __restrict__ lr_svel,
                                const uint32_t* __restrict__ cell_start, const float4* __restrict__ hx,
