@@ -84,7 +84,10 @@ struct SampleGrid {
 // passes the negative real axis (each angle is below a half turn, so it
 // passes upwards only from Im > 0 by det > 0 to Im < 0, downwards the other
 // way); one atan2f at the end gives the rest.  Each product rounds by less
-// than 8 u.
+// than 8 u.  A product exactly on the negative real axis (Im = 0, as round
+// angles make it at the centre of a symmetric mesh) is on neither side of the
+// cut, and the next angle would pass it uncounted: such a candidate is left
+// open.
 
 __device__ __forceinline__ float cell_units(double x, double mid, double inv_r)
 {
@@ -161,6 +164,7 @@ __global__ void __launch_bounds__(128) k_sample_classify(const float4* __restric
                 const float nr = zr * c - zi * s, ni = zr * s + zi * c;
                 if (zi > 0.0f && s > 0.0f && ni < 0.0f) ++turns;
                 if (zi < 0.0f && s < 0.0f && ni > 0.0f) --turns;
+                unsure |= ni == 0.0f && !(nr > 0.0f);
                 zr = nr;
                 zi = ni;
             }

@@ -141,3 +141,55 @@ def test_inside_decisions_near_the_surface_equal_the_oracle(orc, mesh, scale, sh
     assert rc == gs.GS_OK
     np.testing.assert_array_equal(inside, ref_inside)
     np.testing.assert_array_equal(sel, ref_sel)
+
+
+def _symmetric_meshes():
+    """Convex meshes whose centres and lattice points see their triangles under round angles, with the centre."""
+    rng = np.random.default_rng(41)
+    out = [(*scenes.box_mesh((0, 0, 0), (1, 1, 1)), np.full(3, 0.5)),
+           (*scenes.box_mesh((-1, -2, -3), (1, 2, 3)), np.zeros(3)),
+           (*scenes.box_mesh((0.125, 0.25, 0.5), (0.375, 0.75, 0.625)), np.array([0.25, 0.5, 0.5625]))]
+    tet = np.array([(1, 1, 1), (1, -1, -1), (-1, 1, -1), (-1, -1, 1)], float)
+    out.append((tet, np.array([(0, 1, 2), (0, 2, 3), (0, 3, 1), (1, 3, 2)], np.int32), np.zeros(3)))
+    for axes in (np.eye(3), np.array([(1, 2, 2), (1, -2, -2), (-1, 2, -2)], float)):   # the latter: den exactly 0
+        V = np.concatenate([axes, -axes])
+        T = np.array([(a, 1 + b, 2 + c) for a in (0, 3) for b in (0, 3) for c in (0, 3)], np.int32)
+        for t in T:
+            if np.linalg.det(V[t]) < 0.0:
+                t[1:] = t[2:0:-1]
+        out.append((V, T, np.zeros(3)))
+    # scaled and shifted cubes, whose coordinates round
+    out += [(V0 * s + c, T0, c + 0.5 * s) for V0, T0, _ in out[:1]
+            for s, c in [(rng.uniform(0.1, 10.0), rng.uniform(-1.0, 1.0, 3)) for _ in range(4)]]
+    return out
+
+
+@pytest.mark.parametrize("mesh", range(10))
+def test_inside_decisions_at_symmetric_points_equal_the_oracle(orc, mesh):
+    # the product of the triangles' unit numbers meets the cut of its angle
+    # exactly at such points, in an order of the triangles that depends on the
+    # mesh: many orders, centre and lattice points off the surface.  The
+    # double evaluation is off by about 1e-15 there, so equality
+    import paper_2308_01629_gb300 as gs
+    V, T, c = _symmetric_meshes()[mesh]
+    rng = np.random.default_rng(42 + mesh)
+    half = 0.5 * (V.max(0) - V.min(0))
+    k = np.arange(-5, 6) / 4.0
+    off = np.array([(x, y, z) for x in k for y in k for z in k])
+    if mesh == 3:       # |x| + |y| + |z| style faces: keep clear of them
+        keep = np.min([np.abs(off @ n - 1.0) for n in ((1, 1, -1), (1, -1, 1), (-1, 1, 1), (-1, -1, -1))], 0) > 1e-3
+    elif mesh in (4, 5):
+        P = np.linalg.solve(V[:3].T, (off * half).T).T
+        keep = np.abs(np.abs(P).sum(1) - 1.0) > 1e-3
+    else:
+        keep = np.abs(np.abs(off).max(1) - 1.0) > 1e-3
+    cand = c + off[keep] * half
+    r = 0.02 * float(half.max())
+    for _ in range(60):
+        P = T[rng.permutation(len(T))]
+        P = np.array([np.roll(t, rng.integers(3)) for t in P], np.int32)
+        rc, sel, inside = gs.gs_sample_volume(V, P, cand, r)
+        ref_sel, ref_inside = orc.sample_volume(V, P, cand, r)
+        assert rc == gs.GS_OK and ref_inside[np.flatnonzero(keep).searchsorted(len(off) // 2)]
+        np.testing.assert_array_equal(inside, ref_inside)
+        np.testing.assert_array_equal(sel, ref_sel)
