@@ -78,7 +78,8 @@ struct SampleGrid {
 // den)|, as long as D < h / 4 and the pair cannot lie on the other side of
 // the cut (den < 0 and |det| <= D): otherwise the candidate is left open.
 // NaN and infinity (a corner at p, coordinates out of range) leave it open
-// too, since every comparison is written to fail with them.
+// too: every comparison is written to fail with them, and 1 / h = 0 says that
+// the sum of squares left the range (from about 2e6 box sizes away).
 // The angles are summed without an arctangent per triangle: the unit numbers
 // (den + i det) / h are multiplied up and the turns counted where the product
 // passes the negative real axis (each angle is below a half turn, so it
@@ -158,7 +159,7 @@ __global__ void __launch_bounds__(128) k_sample_classify(const float4* __restric
                 const float D = d10 * (lab + lc * (la + lb)) + 256.0f * u * L;
                 const float rh = rsqrtf(det * det + den * den);
                 const float rel = D * rh;
-                unsure |= !(rel < 0.25f && (den > 0.0f || fabsf(det) > D));
+                unsure |= !(rel < 0.25f && rh > 0.0f && (den > 0.0f || fabsf(det) > D));
                 E += rel;
                 const float c = den * rh, s = det * rh;
                 const float nr = zr * c - zi * s, ni = zr * s + zi * c;

@@ -193,3 +193,23 @@ def test_inside_decisions_at_symmetric_points_equal_the_oracle(orc, mesh):
         assert rc == gs.GS_OK and ref_inside[np.flatnonzero(keep).searchsorted(len(off) // 2)]
         np.testing.assert_array_equal(inside, ref_inside)
         np.testing.assert_array_equal(sel, ref_sel)
+
+
+@pytest.mark.parametrize("mesh", ["box", "sphere"])
+def test_far_candidates_equal_the_oracle(orc, mesh):
+    # from about 2e6 box sizes on the single-precision products leave their
+    # range, from 1e13 on the lengths do: up to there and beyond it
+    import paper_2308_01629_gb300 as gs
+    V, T = scenes.box_mesh((0, 0, 0), (1e-3, 2e-3, 1e-3)) if mesh == "box" else scenes.icosphere((0, 0, 0), 1e-3, 2)
+    rng = np.random.default_rng(43)
+    d = rng.normal(size=(4000, 3))
+    d[::4, 1:] = 0.0                                  # along an axis: in the planes of a box's faces or not at all
+    d /= np.linalg.norm(d, axis=1, keepdims=True)
+    size = float((V.max(0) - V.min(0)).max())
+    far = V.mean(0) + d * size * 10.0 ** rng.uniform(3.0, 17.0, (len(d), 1))
+    cand = np.concatenate([scenes.volume_candidates(V, 1e-4, seed=44), far])
+    rc, sel, inside = gs.gs_sample_volume(V, T, cand, 1e-4)
+    ref_sel, ref_inside = orc.sample_volume(V, T, cand, 1e-4)
+    assert rc == gs.GS_OK and not inside[-len(far):].any()
+    np.testing.assert_array_equal(inside, ref_inside)
+    np.testing.assert_array_equal(sel, ref_sel)
