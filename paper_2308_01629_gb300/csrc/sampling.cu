@@ -90,6 +90,12 @@ struct SampleGrid {
 // cut, and the next angle would pass it uncounted: such a candidate is left
 // open.
 
+// A position relative to its cell's centre in units of r, or NaN where single
+// precision would not do: more than 64 r away, or a mesh farther from the
+// origin than kMaxUnits r (the host then passes a NaN as 1 / r), whose cell
+// centres round by more than 2^-52 kMaxUnits = 7e-6 r.
+constexpr double kMaxUnits = 3.0e10;
+
 __device__ __forceinline__ float cell_units(double x, double mid, double inv_r)
 {
     const float f = (float)(__dsub_rn(x, mid) * inv_r);
@@ -231,8 +237,9 @@ __global__ void __launch_bounds__(128) k_sample_winding(const double* __restrict
 // positions relative to the cell, in units of r, and in double precision only
 // when a squared distance comes within 1e-3 of the threshold 4, since FP64
 // issues at 1/64 of the FP32 rate.  (Coordinates of at most 64 units round by
-// 4e-6 each, so a squared distance near 4 is off by less than 1e-4; farther
-// candidates, beyond the mesh's box, become NaN and are tested in double.)
+// 4e-6 each, and kMaxUnits bounds the rounding of a cell's centre, so a
+// squared distance near 4 is off by less than 3e-4; farther candidates, beyond
+// the mesh's box, become NaN and are tested in double.)
 // With one thread per cell and every test in double a phase was a serial
 // chain of up to 125 lookups per candidate: 168 us per phase for a million
 // candidates in 265,000 cells (52 us with this layout but all tests in
@@ -427,6 +434,9 @@ static int sample_impl(const double* vertices, int64_t n_vertices, const int32_t
     if (nc) {
         const double extent = std::fmax(hi[0] - g.lo[0], std::fmax(hi[1] - g.lo[1], hi[2] - g.lo[2]));
         const double inv_extent = extent > 0.0 ? 1.0 / extent : 1.0;
+        double reach = 0.0;
+        for (int k = 0; k < 3; ++k) reach = std::fmax(reach, std::fmax(std::fabs(g.lo[k]), std::fabs(hi[k])));
+        const double inv_r = reach <= kMaxUnits * r ? 1.0 / r : std::nan("");
         uint32_t* n_open = dopen + (surface ? 0 : nc);
         SK(cudaMemsetAsync(n_open, 0, sizeof(uint32_t), s));
         if (n_triangles) {
@@ -434,7 +444,7 @@ static int sample_impl(const double* vertices, int64_t n_vertices, const int32_t
             SK(cudaGetLastError());
         }
         k_sample_classify<<<gs_blocks(nc, 128), 128, 0, s>>>((const float4*)dtri, n_triangles, dC, nc, g, inv_extent,
-                                                             din, keys, rank, start, dopen, n_open, drel, 1.0 / r,
+                                                             din, keys, rank, start, dopen, n_open, drel, inv_r,
                                                              surface);
         SK(cudaGetLastError());
         if (!surface) {

@@ -213,3 +213,28 @@ def test_far_candidates_equal_the_oracle(orc, mesh):
     assert rc == gs.GS_OK and not inside[-len(far):].any()
     np.testing.assert_array_equal(inside, ref_inside)
     np.testing.assert_array_equal(sel, ref_sel)
+
+
+@pytest.mark.parametrize("shift", [1e9, 1e11, 1e13, 3e14])
+@pytest.mark.parametrize("surface", [False, True])
+def test_picks_far_from_the_origin_equal_the_oracle(orc, surface, shift):
+    # in units of r: the distance test's positions are relative to cell
+    # centres, which round by 2^-53 of the coordinate; beyond some 1e10 the
+    # rounding is no longer small against the test's margin.  The candidates
+    # themselves are exact, so equality
+    import paper_2308_01629_gb300 as gs
+    V, T = scenes.box_mesh((0, 0, 0), (24, 18, 21))
+    V = V + np.array([shift, -shift, 0.5 * shift])
+    rng = np.random.default_rng(45)
+    if surface:
+        cand = np.rint(scenes.surface_candidates(V, T, 1.0, per_cell=30.0, seed=46))
+        cand = np.clip(cand + rng.integers(-64, 65, cand.shape) / 64.0, V.min(0), V.max(0))
+        rc, sel = gs.gs_sample_surface(V, cand, 1.0)
+        ref = orc.sample_surface(V, cand, 1.0)
+    else:
+        cand = scenes.volume_candidates(V, 1.0, per_cell=30.0, seed=46)
+        rc, sel, inside = gs.gs_sample_volume(V, T, cand, 1.0)
+        ref, ref_inside = orc.sample_volume(V, T, cand, 1.0)
+        np.testing.assert_array_equal(inside, ref_inside)
+    assert rc == gs.GS_OK
+    np.testing.assert_array_equal(sel, ref)
