@@ -468,6 +468,7 @@ int create_impl(int S, const gs_scene* scenes, const float* r_low, const float* 
         A(dalloc(&c->bins.bucket, gs_bins_bucket_words(cells)));
         A(dalloc(&c->bins.tile, c->bins.n_tiles));
         A(dalloc(&c->bins.spill, N));
+        c->bins.list = c->lr_vals[0];   // the general sort's arrival ranks
         A(dalloc(&c->bins.words, kBinWords));
     }
     A(dalloc(&c->lr_spos, N));

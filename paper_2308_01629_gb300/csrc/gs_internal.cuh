@@ -86,13 +86,14 @@ struct CflState {
 };
 
 // Scratch of the LR binning (lr_bins.cuh); all counts zero between binnings.
-enum { kBinSpillAcc = 0, kBinSpill = 1, kBinSolidAcc = 2, kBinWords = 4 };
+enum { kBinSpill = 0, kBinSolid = 1, kBinWords = 2 };
 struct LrBins {
     uint32_t* count = nullptr;    // per cell, padded to whole tiles; null: the general counting sort
     uint32_t* bucket = nullptr;   // [n_cell][kBucket] particles of a cell in order of arrival
     uint32_t* tile = nullptr;     // [n_tiles] particles per tile of cells
-    uint32_t* spill = nullptr;    // [n] particles beyond their cell's bucket
-    uint32_t* words = nullptr;    // spilled so far, spilled (of this binning), flag of solid particles so far
+    uint4* spill = nullptr;       // [n] particles beyond their cell's bucket: index, cell, arrival rank
+    uint32_t* list = nullptr;     // [n] those particles again, each cell's at its slots beyond kBucket
+    uint32_t* words = nullptr;    // spilled, flag of solid particles
     int n_tiles = 0;
 };
 

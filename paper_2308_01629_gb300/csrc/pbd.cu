@@ -589,7 +589,7 @@ __device__ __forceinline__ void pass_warp(const PbdArgs& a, int stab, int64_t p0
                     at = predicted(sc, np, nv, dt);
                     fin.next.xt[i] = at;
                 } else if (w == 0.0f || (kBody && a.body[i] != 0u)) {
-                    atomicOr(fin.next.b.words + kBinSolidAcc, 1u);
+                    atomicOr(fin.next.b.words + kBinSolid, 1u);
                 }
                 const uint32_t cell = grid_cell_of(sc, at.x, at.y, at.z);
                 fin.next.keys[i] = cell;

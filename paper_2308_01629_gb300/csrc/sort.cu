@@ -690,7 +690,7 @@ __global__ void __launch_bounds__(256) k_bins_keys(const LrBins b, const float4*
     if (i < n) {
         const SceneDev& sc = scenes[tag[i] & ~kPadBit];
         const float4 p = pos[i];
-        if (flag_solid && (p.w == 0.0f || (body && body[i] != 0u))) atomicOr(b.words + kBinSolidAcc, 1u);
+        if (flag_solid && (p.w == 0.0f || (body && body[i] != 0u))) atomicOr(b.words + kBinSolid, 1u);
         if (solid_err && p.w == 0.0f) atomicOr(solid_err, GS_DEVERR_SOLID_REVERSE);
         const uint32_t cell = grid_cell_of(sc, p.x, p.y, p.z);
         keys[i] = cell;
@@ -700,7 +700,9 @@ __global__ void __launch_bounds__(256) k_bins_keys(const LrBins b, const float4*
 }
 
 // One block per tile of cells.  The tile sums before it (at most one per
-// thread) give its base, so no launch sums tiles and no block waits.
+// thread) give its base, so no launch sums tiles and no block waits.  Where
+// particles spilled, the block also puts its tile's into the list (every block
+// reads all of them: 17,000 of a bed of 24 per cell are 17 per thread).
 __global__ void __launch_bounds__(kScanBlock) k_bins_scan(const LrBins b, uint32_t* __restrict__ start, int64_t total,
                                                           unsigned* solid_flag, unsigned* clear)
 {
@@ -709,6 +711,7 @@ __global__ void __launch_bounds__(kScanBlock) k_bins_scan(const LrBins b, uint32
     const int64_t i0 = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanPer;
     const uint4 v = *reinterpret_cast<const uint4*>(b.count + i0);   // padded to whole tiles
     const uint32_t before = threadIdx.x < blockIdx.x ? b.tile[threadIdx.x] : 0u;
+    const uint32_t spilled = b.words ? b.words[kBinSpill] : 0u;      // cleared by place
     uint32_t base, tot;
     block_scan(before, ws, &base);
     const uint32_t sum = v.x + v.y + v.z + v.w;
@@ -719,17 +722,32 @@ __global__ void __launch_bounds__(kScanBlock) k_bins_scan(const LrBins b, uint32
         if (i0 + k < total) start[i0 + k] = run;
         run += c[k];
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {   // this binning's words, and zero for the next one's arrivals
+    if (blockIdx.x == 0 && threadIdx.x == 0) {   // this binning's flag, and zero for the next one's arrivals
         if (b.words) {
-            b.words[kBinSpill] = b.words[kBinSpillAcc];
-            b.words[kBinSpillAcc] = 0u;
-            if (solid_flag) *solid_flag = b.words[kBinSolidAcc];
-            b.words[kBinSolidAcc] = 0u;
+            if (solid_flag) *solid_flag = b.words[kBinSolid];
+            b.words[kBinSolid] = 0u;
         }
         if (clear) *clear = 0u;
     }
+    if (spilled != 0u) {   // the same on every thread
+        __syncthreads();   // the tile's starts
+#pragma unroll 4
+        for (uint32_t k = threadIdx.x; k < spilled; k += kScanBlock) {
+            const uint4 e = __ldg(b.spill + k);   // read ahead of the stores
+            if (e.y / kBinTile == blockIdx.x) b.list[start[e.y] + e.z] = e.x;
+        }
+    }
 }
 
+// A rank in a cell of up to kCrowd particles takes one thread, which looks at
+// the cell's own entries.  In a larger cell the lanes of a warp count for all of
+// its particles in the warp together (the entries before the warp's first
+// particle, then the ones within it), so that a cell of c costs c^2 / 1,024
+// steps of a warp.  gs_bin_low, before (every particle of a crowded cell walked
+// the spilled ones of all cells) -> now, and the general counting sort, whose
+// warps order a crowded cell each: 50,527 LR at 24 per cell 781 -> 25 us (39),
+// at 1,024 2,417 -> 84 (205), in one cell 2,488 -> 524 (5,462); 202,112 LR at
+// 24 per cell 4,813 -> 50 us (51), in one cell 16.7 -> 2.1 ms (30.4).
 __global__ void __launch_bounds__(128) k_bins_place(const LrBins b, int64_t n, const uint32_t* __restrict__ keys,
                                                     const uint32_t* __restrict__ start,
                                                     uint32_t* __restrict__ out_keys, uint32_t* __restrict__ out_idx,
@@ -739,7 +757,10 @@ __global__ void __launch_bounds__(128) k_bins_place(const LrBins b, int64_t n, c
 {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     for (int64_t k = t; k < b.n_tiles; k += (int64_t)gridDim.x * blockDim.x) b.tile[k] = 0u;
-    if (t >= n) return;
+    if (t == 0) b.words[kBinSpill] = 0u;
+    const bool live = t < n;
+    const unsigned lanes = __ballot_sync(0xffffffffu, live);
+    if (!live) return;
     const uint32_t i = (uint32_t)t;
     const uint32_t key = keys[i];
     float4 u = ga[i], v = gb[i];
@@ -753,12 +774,23 @@ __global__ void __launch_bounds__(128) k_bins_place(const LrBins b, int64_t n, c
         rank += (e.x < i ? 1u : 0u) + (k + 1 < c && e.y < i ? 1u : 0u) + (k + 2 < c && e.z < i ? 1u : 0u) +
                 (k + 3 < c && e.w < i ? 1u : 0u);
     }
-    if (c > (uint32_t)kBucket) {
-        const uint32_t m = b.words[kBinSpill];
-        for (uint32_t k = 0; k < m; ++k) {
-            const uint32_t j = b.spill[k];
-            if (j < i && keys[j] == key) ++rank;
+    if (c > (uint32_t)kBucket && c <= kCrowd)
+        for (uint32_t k = s + kBucket; k < s + c; ++k) rank += b.list[k] < i ? 1u : 0u;
+    unsigned todo = __ballot_sync(lanes, c > kCrowd);
+    while (todo) {   // warp-uniform
+        const int leader = __ffs(todo) - 1, lane = (int)(threadIdx.x & 31u);
+        const uint32_t lk = __shfl_sync(lanes, key, leader), ls = __shfl_sync(lanes, s, leader),
+                       lc = __shfl_sync(lanes, c, leader);
+        const unsigned peers = __ballot_sync(lanes, key == lk);
+        const uint32_t first = i - (uint32_t)lane;   // the warp's first particle
+        uint32_t less = 0;
+        for (uint32_t k = (uint32_t)lane; k < lc; k += (uint32_t)__popc(lanes)) {   // the last warp's lanes end early
+            const uint32_t j = k < (uint32_t)kBucket ? b.bucket[(size_t)lk * kBucket + k] : b.list[ls + k];
+            less += j < first ? 1u : 0u;
         }
+        less = __reduce_add_sync(lanes, less);
+        if (key == lk) rank = less + (uint32_t)__popc(peers & ((1u << lane) - 1u));
+        todo &= ~peers;
     }
     b.count[key] = 0u;   // every particle of the cell writes the same
     const uint32_t slot = s + rank;

@@ -141,3 +141,68 @@ def test_steps_that_begin_the_next_binning_give_the_same_bits(kind):
         ctx.close()
     for a, b in zip(*out):
         np.testing.assert_array_equal(a, b)
+
+
+def _crowds(sc, kind, rng):
+    """LR positions whose cells hold far more particles than a bucket."""
+    p = sc["lr_pos"].copy()
+    n, hi = len(p), np.asarray(sc["box_hi"])
+    h = float(np.float32(3.0 * sc["r_low"] * (1.0 + 1.0 / 1024.0)))
+    if kind == "bed":            # 24 in most cells
+        side = h * (n / 24.0) ** (1.0 / 3.0)
+        p[:, :3] = 0.1 + rng.uniform(0.0, side, (n, 3))
+    elif kind == "pile":         # all in one cell
+        p[:, :3] = 10.5 * h + rng.uniform(0.0, 1e-3, (n, 3))
+    elif kind == "piles":        # over a thousand in each of some cells, the particles of a cell far apart in the set
+        c = rng.uniform(0.1, 0.9, (40, 3)) * hi
+        p[:, :3] = c[rng.integers(0, len(c), n)] + rng.uniform(0.0, 1e-4, (n, 3))
+    elif kind == "line":         # on each side of the line between the two ways of counting
+        p[:, :3] = rng.uniform(0.0, 1.0, (n, 3)) * hi
+        at = rng.permutation(n)
+        p[at[:2048], :3] = h * np.array([20.5, 5.5, 5.5])
+        p[at[2048:4097], :3] = h * np.array([25.5, 5.5, 5.5])
+        p[at[4097:], 0] = np.where(np.abs(p[at[4097:], 0] - 23.0 * h) < 4.0 * h, 0.1, p[at[4097:], 0])
+    else:                        # outside the grid: clamped into its edge cells
+        p[:, :3] = hi * rng.uniform(0.0, 1.0, (n, 3)) + (0.0, 0.0, 10.0)
+        p[: n // 3, :3] += 10.0
+    return p
+
+
+@pytest.mark.parametrize("kind", ["bed", "pile", "piles", "line", "outside"])
+def test_crowded_cells_are_ordered_and_cost_no_more_than_the_general_sort(orc, kind):
+    # the same particles in a grid of a few cells and in one of over four
+    # million, which takes the general counting sort (linear in the crowd);
+    # the bound on the time is twice that
+    import torch
+
+    import paper_2308_01629_gb300 as gs
+    base = scenes.digging(ratio=1)
+    p = _crowds(base, kind, np.random.default_rng(17))
+    ms = []
+    for box_hi in (base["box_hi"], tuple(np.asarray(base["box_hi"]) * 5.1)):
+        sc = dict(base, box_hi=box_hi)
+        q = p.copy()
+        if kind == "outside":    # beyond this grid too
+            q[:, 2] += box_hi[2]
+        with torch.cuda.stream(torch.cuda.Stream()):
+            ctx = gs.Context(dict(sc, lr_pos=q), stream="torch")
+            ctx.set_graphs(False)
+            best = 1e9
+            for _ in range(4):
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                a.record()
+                ctx.bin_low()
+                b.record()
+                b.synchronize()
+                best = min(best, a.elapsed_time(b))
+            ms.append(best)
+            o, _, ih, dims = orc.grid(float(np.float32(sc["r_low"])), np.float32(sc["box_lo"]).astype(float),
+                                      np.float32(box_hi).astype(float))
+            nc = int(np.prod(dims))
+            ref_idx, ref_start = orc.counting_sort(orc.cell_keys(q, o, ih, dims), nc)
+            np.testing.assert_array_equal(ctx.read(gs.GS_FIELD_LR_SORTED_INDEX), ref_idx)
+            np.testing.assert_array_equal(ctx.read(gs.GS_FIELD_LR_CELL_START)[:nc + 1], ref_start)
+            ctx.close()
+    print(f"{kind}: buckets {ms[0]:.3f} ms, general sort {ms[1]:.3f} ms, {len(p)} LR, largest cell "
+          f"{np.diff(ref_start).max()}")
+    assert ms[0] < 2.0 * ms[1]
