@@ -432,31 +432,29 @@ __global__ void __launch_bounds__(WARPS * 32, WARPS == 4 && !kSolid ? kAutoBlock
 }  // namespace
 
 template <int WARPS, bool kSingle, bool kIds>
-static cudaError_t launch_w(cudaStream_t s, const UpsampleArgs& a, int blocks_per_sm, int sm_count)
+static cudaError_t launch_w(cudaStream_t s, const UpsampleArgs& a, int blocks_per_sm, int solid_per_sm, int sm_count)
 {
     // both instantiations; the one the device flag does not select returns
-    // (the one for solid particles always as a persistent grid, so that a
-    // frame without them pays for few blocks: the full grid's empty blocks
-    // took 18 us on the 2 x 2 m bed)
     const unsigned need = gs_blocks(a.n_warps, WARPS);
-    const int64_t resident = (int64_t)std::max(blocks_per_sm, 1) * sm_count;
-    const unsigned nb = (unsigned)std::min<int64_t>(resident, need);
-    if (blocks_per_sm <= 0) k_upsample<WARPS, false, kSingle, kIds><<<need, WARPS * 32, 0, s>>>(a, 0);
-    else k_upsample<WARPS, false, kSingle, kIds><<<nb, WARPS * 32, 0, s>>>(a, 1);
-    const unsigned nb_solid = (unsigned)std::min<int64_t>((int64_t)(24 / WARPS) * sm_count, need);
-    k_upsample<WARPS, true, kSingle, kIds><<<nb_solid, WARPS * 32, 0, s>>>(a, 1);
+    auto go = [&](auto kernel, int per_sm) {
+        if (per_sm <= 0) kernel<<<need, WARPS * 32, 0, s>>>(a, 0);
+        else kernel<<<(unsigned)std::min<int64_t>((int64_t)per_sm * sm_count, need), WARPS * 32, 0, s>>>(a, 1);
+    };
+    go(k_upsample<WARPS, false, kSingle, kIds>, blocks_per_sm);
+    go(k_upsample<WARPS, true, kSingle, kIds>, solid_per_sm);
     return cudaGetLastError();
 }
 
 template <int WARPS>
-static cudaError_t launch_scenes(cudaStream_t s, const UpsampleArgs& a, int blocks_per_sm, int sm_count)
+static cudaError_t launch_scenes(cudaStream_t s, const UpsampleArgs& a, int blocks_per_sm, int solid_per_sm,
+                                 int sm_count)
 {
     if (a.id_pos) {   // the functional frame: one scene
         if (a.n_scenes != 1) return cudaErrorInvalidValue;
-        return launch_w<WARPS, true, true>(s, a, blocks_per_sm, sm_count);
+        return launch_w<WARPS, true, true>(s, a, blocks_per_sm, solid_per_sm, sm_count);
     }
-    return a.n_scenes == 1 ? launch_w<WARPS, true, false>(s, a, blocks_per_sm, sm_count)
-                           : launch_w<WARPS, false, false>(s, a, blocks_per_sm, sm_count);
+    return a.n_scenes == 1 ? launch_w<WARPS, true, false>(s, a, blocks_per_sm, solid_per_sm, sm_count)
+                           : launch_w<WARPS, false, false>(s, a, blocks_per_sm, solid_per_sm, sm_count);
 }
 
 cudaError_t gs_launch_upsample(cudaStream_t s, const UpsampleArgs& a, int warps_per_block, int blocks_per_sm,
@@ -465,14 +463,19 @@ cudaError_t gs_launch_upsample(cudaStream_t s, const UpsampleArgs& a, int warps_
     if (a.n_warps <= 0) return cudaSuccess;
     cudaError_t e = a.clear_work ? cudaMemsetAsync(a.work, 0, sizeof(unsigned), s) : cudaSuccess;
     if (e != cudaSuccess) return e;
+    int solid_per_sm = blocks_per_sm;
     if (warps_per_block == 0) {   // by the number of items
         warps_per_block = 4;
         blocks_per_sm = a.n_warps >= kPersistentItems ? kAutoBlocks : 0;
+        // the form for solid particles as a persistent grid whatever the
+        // number, so that a frame without them pays for few empty blocks (the
+        // full grid's took 18 us on the 2 x 2 m bed)
+        solid_per_sm = 24 / warps_per_block;
     }
     switch (warps_per_block) {
-    case 4: e = launch_scenes<4>(s, a, blocks_per_sm, sm_count); break;
-    case 16: e = launch_scenes<16>(s, a, blocks_per_sm, sm_count); break;
-    default: e = launch_scenes<8>(s, a, blocks_per_sm, sm_count); break;
+    case 4: e = launch_scenes<4>(s, a, blocks_per_sm, solid_per_sm, sm_count); break;
+    case 16: e = launch_scenes<16>(s, a, blocks_per_sm, solid_per_sm, sm_count); break;
+    default: e = launch_scenes<8>(s, a, blocks_per_sm, solid_per_sm, sm_count); break;
     }
     *launches += 2;   // the two instantiations
     return e;

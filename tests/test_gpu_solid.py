@@ -3,6 +3,8 @@ inverse mass 0 under the same contact constraints; Sec. 4: they count in the
 HR weights except where no grain reaches the HR particle).  GPU against the
 FP64 oracle on a cube standing on a particle floor and on the digging bed
 with a particle bucket, plus the bitwise agreements that must hold."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -176,3 +178,87 @@ def test_reverse_modes_refuse_solid_particles():
     assert e.value.code == gs.GS_ERR_STATE
     ctx.sync()   # reported once; the context stays usable
     ctx.close()
+
+
+def _gather_grids(ctx, call):
+    """(warps per block, blocks) of the gather's two launches that call() enqueues, read from a capture of its stream."""
+    cu = ctypes.CDLL("libcuda.so.1")
+
+    class Params(ctypes.Structure):      # CUDA_KERNEL_NODE_PARAMS_v2
+        _fields_ = [("func", ctypes.c_void_p), ("grid", ctypes.c_uint * 3), ("block", ctypes.c_uint * 3),
+                    ("shared", ctypes.c_uint), ("args", ctypes.c_void_p), ("extra", ctypes.c_void_p),
+                    ("kern", ctypes.c_void_p), ("ctx", ctypes.c_void_p)]
+
+    def ok(rc):
+        assert rc == 0, rc
+
+    import torch
+    s = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    graph, n = ctypes.c_void_p(), ctypes.c_size_t()
+    ok(cu.cuStreamBeginCapture_v2(s, 1))
+    try:
+        call()
+    finally:
+        rc = cu.cuStreamEndCapture(s, ctypes.byref(graph))
+    ok(rc)
+    ok(cu.cuGraphGetNodes(graph, None, ctypes.byref(n)))
+    nodes = (ctypes.c_void_p * n.value)()
+    ok(cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n)))
+    out = []
+    for node in nodes:
+        kind = ctypes.c_int()
+        ok(cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)))
+        if kind.value != 0:              # a kernel
+            continue
+        p, name = Params(), ctypes.c_char_p()
+        ok(cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), ctypes.byref(p)))
+        if p.func:
+            ok(cu.cuFuncGetName(ctypes.byref(name), ctypes.c_void_p(p.func)))
+        else:
+            ok(cu.cuKernelGetName(ctypes.byref(name), ctypes.c_void_p(p.kern)))
+        if b"k_upsample" in name.value and b"bwd" not in name.value:
+            out.append((p.block[0] // 32, p.grid[0]))
+    ok(cu.cuGraphDestroy(graph))
+    return out
+
+
+@pytest.mark.parametrize("shape", [(8, 1), (8, 2), (4, 7), (16, 1), (4, 0), (8, 0), (16, 0)])
+def test_both_gather_forms_take_the_callers_launch_shape(shape):
+    # the form for particles of infinite mass as well as the plain one: which
+    # of the two does the frame is decided on the device
+    import torch
+
+    import paper_2308_01629_gb300 as gs
+    sc = scenes.digging(ratio=12)
+    sc["lr_pos"][::97, 3] = 0.0
+    w, per_sm = shape
+    items = (len(sc["hr_pos"]) + 31) // 32
+    need = (items + w - 1) // w
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    with torch.cuda.stream(torch.cuda.Stream()):
+        ctx = gs.Context(sc, stream="torch")
+        ctx.set_graphs(False)
+        ctx.set_tuning(*shape)
+        ctx.upsample(1.0 / 60.0)
+        ctx.sync()
+        grids = _gather_grids(ctx, lambda: ctx.upsample(1.0 / 60.0))
+        ctx.close()
+    assert grids == [(w, min(per_sm * sms, need) if per_sm else need)] * 2
+
+
+@pytest.mark.parametrize("shape", [(8, 1), (8, 0), (4, 2)])
+def test_pipelined_frames_with_a_particle_bucket_equal_sequential_frames(shape):
+    import paper_2308_01629_gb300 as gs
+    sc = scenes.digging_particle_bucket()
+    out = []
+    for pipelined in (False, True):
+        ctx = gs.Context(sc)
+        if pipelined:
+            ctx.set_pipeline(True, *shape)
+        for _ in range(5):
+            ctx.frame(DT, 4, 4)
+        out.append([ctx.read(f).view(np.uint32) for f in (gs.GS_FIELD_LR_POS, gs.GS_FIELD_LR_VEL, gs.GS_FIELD_HR_POS,
+                                                           gs.GS_FIELD_HR_VEL)])
+        ctx.close()
+    for a, b in zip(*out):
+        np.testing.assert_array_equal(a, b)
