@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 
 #include "gs.h"
@@ -159,6 +160,10 @@ extern "C" int gs_rollout_forward(gs_ctx* c, const float* lr_x0, const float* lr
         checkpoint_every < 1)
         return gs_ctx_fail(c, GS_ERR_ARG, "invalid rollout arguments");
     if (c->n_scenes != 1) return gs_ctx_fail(c, GS_ERR_STATE, "the rollout needs a single-scene context");
+    // what the LR steps and HR frames of the sequence accept as a step length
+    // (each of a rollout of no frames is accepted)
+    if (frames > 0 && (!std::isfinite(dt) || !(dt / (float)n_sub > 0.0f)))
+        return gs_ctx_fail(c, GS_ERR_ARG, "invalid rollout time step");
     const int64_t N = c->n_low, M = c->n_high;
     if (!lr_x0 || !lr_v0 || !hr_x0 || !hr_v0 || !lr_x || !lr_v || !hr_x || !hr_v)
         return gs_ctx_fail(c, GS_ERR_ARG, "null buffer");
