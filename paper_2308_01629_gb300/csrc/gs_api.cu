@@ -1205,6 +1205,8 @@ int gs_replay_or_run(gs_ctx* c, uint64_t key, int (*body)(gs_ctx*, void*), void*
     return replay_or_run(c, key, [&] { return body(c, arg); });
 }
 
+void gs_drop_graphs(gs_ctx* c) { drop_graphs(c); }
+
 uint64_t gs_sequence_key(const gs_ctx* c, char kind, float dt, int iters)
 {
     return step_key(c, kind, dt, iters);

@@ -604,6 +604,8 @@ int gs_ctx_fail(gs_ctx* c, int code, const char* msg);
 // replayed; the host-side state the body leaves is recorded at capture and
 // applied on every replay.
 int gs_replay_or_run(gs_ctx* c, uint64_t key, int (*body)(gs_ctx*, void*), void* arg);
+// Drops every captured sequence and frame (the next call captures anew).
+void gs_drop_graphs(gs_ctx* c);
 // A key of the functional sequences: kind, step length, passes and the
 // context's launch configuration.
 uint64_t gs_sequence_key(const gs_ctx* c, char kind, float dt, int iters);

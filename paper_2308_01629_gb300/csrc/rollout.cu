@@ -3,12 +3,11 @@
 // state at every checkpoint_every-th frame; its backward recomputes each
 // segment from its checkpoint with taped LR steps (the recorded passes kept
 // for their reverse) and runs the reverse modes frame by frame, last to
-// first.  The same functional entry points as a rollout driven from the
-// caller, without a host round trip per operation in the caller's language:
+// first.  The same sequences as a rollout driven from the caller through the
+// functional entry points, without a host round trip per operation:
 // with graphs enabled the whole forward, and the whole backward, of one
-// configuration are captured (on their second call; the first allocates
-// what they need) and replayed as one CUDA graph each, on the context's
-// own copies of the caller's buffers.
+// configuration are captured (on their second call) and replayed as one
+// CUDA graph each, on the context's own copies of the caller's buffers.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -20,10 +19,13 @@
 
 namespace {
 
+// Where a buffer moves, the captured sequences that hold it are dropped.
 int grow(gs_ctx* c, float4** buf, int64_t* cap, int64_t need, const char* what)
 {
     if (need <= *cap && *buf) return GS_OK;
-    if (*buf) cudaFree(*buf);
+    gs_drop_graphs(c);
+    c->ro_seen.clear();
+    if (*buf) cudaFree(*buf);   // waits for what still runs on it
     *buf = nullptr;
     *cap = 0;
     if (gs_dalloc_bytes((void**)buf, (size_t)std::max<int64_t>(need, 1) * sizeof(float4)) != cudaSuccess) {
@@ -138,8 +140,8 @@ uint64_t rollout_key(const gs_ctx* c, char kind, const RolloutCfg& g)
     return k;
 }
 
-// The first call of a configuration runs directly (it allocates what the
-// sequence needs); later calls are captured once and replayed.
+// The first call of a configuration runs directly; later calls are captured
+// once and replayed.
 int run_sequence(gs_ctx* c, uint64_t key, int (*body)(gs_ctx*, void*), void* arg)
 {
     if (std::find(c->ro_seen.begin(), c->ro_seen.end(), key) == c->ro_seen.end()) {
@@ -174,7 +176,6 @@ extern "C" int gs_rollout_forward(gs_ctx* c, const float* lr_x0, const float* lr
     int64_t cap_io = 0;
     if (c->ro_io) cap_io = 4 * rec;
     RO(grow(c, &c->ro_io, &cap_io, 4 * rec, "no memory for the rollout's buffers"));
-    if (c->ro_ckpt_cap < (int64_t)std::max(n_ckpt, 1) * rec) c->ro_seen.clear();   // buffers move: capture anew
     RO(grow(c, &c->ro_ckpt, &c->ro_ckpt_cap, (int64_t)std::max(n_ckpt, 1) * rec, "no memory for the checkpoints"));
     RO(copy(c, io(c, 0), (const float4*)lr_x0, N));
     RO(copy(c, io(c, 1), (const float4*)lr_v0, N));
@@ -208,7 +209,6 @@ extern "C" int gs_rollout_backward(gs_ctx* c, const float* g_lr_x, const float* 
     RolloutCfg g{c->ro_dt, c->ro_frames, c->ro_n_sub, c->ro_iters, c->ro_every};
     const int k_max = std::min(g.every, std::max(g.frames, 1));
     const int64_t need = (int64_t)(k_max * g.n_sub + 1) * 2 * N + (int64_t)k_max * 2 * M + 2 * 2 * N + 2 * 2 * M;
-    if (c->ro_work_cap < need) c->ro_seen.clear();   // buffers move: capture anew
     RO(grow(c, &c->ro_work, &c->ro_work_cap, need, "no memory for the rollout's backward"));
     RO(gs_rollout_buffers(c, g.iters, g.frames > 0 ? k_max * g.n_sub : 0));
     RO(copy(c, io(c, 0), (const float4*)g_lr_x, N));
