@@ -206,3 +206,35 @@ def test_crowded_cells_are_ordered_and_cost_no_more_than_the_general_sort(orc, k
     print(f"{kind}: buckets {ms[0]:.3f} ms, general sort {ms[1]:.3f} ms, {len(p)} LR, largest cell "
           f"{np.diff(ref_start).max()}")
     assert ms[0] < 2.0 * ms[1]
+
+
+@pytest.mark.parametrize("kind", ["body", "depth_friction", "solids"])
+def test_lane_forms_among_bystanders_give_the_same_bits(kind):
+    # the same grains with few and with many others far away in the same
+    # scene: on each side of both lines
+    import paper_2308_01629_gb300 as gs
+    base = scenes.cube_on_particle_floor() if kind == "solids" else scenes.cube_with_block()
+    n, r = len(base["lr_pos"]), base["r_low"]
+    hi = np.array([4.0, 1.0, 1.0])
+    side = np.arange(0.05, 0.95, 2.5 * r)
+    room = np.stack(np.meshgrid(np.arange(1.5, 3.9, 2.5 * r), side, side, indexing="ij"), -1).reshape(-1, 3)
+    states = []
+    for others in (64, 17000, 68000):
+        assert others <= len(room) and base["lr_pos"][:, 0].max() < 1.4
+        p = np.zeros((others, 4), np.float32)
+        p[:, :3], p[:, 3] = room[:others], base["lr_pos"][:, 3].max()
+        v = np.random.default_rng(23).normal(0.0, 0.5, (others, 4)).astype(np.float32)
+        v[:, 3] = 0.0
+        sc = dict(base, box_lo=(0.0, 0.0, 0.0), box_hi=tuple(hi), sdfs=[scenes.box_interior((0, 0, 0), tuple(hi))],
+                  lr_pos=np.concatenate([base["lr_pos"], p]), lr_vel=np.concatenate([base["lr_vel"], v]))
+        sc.pop("lr_body", None)
+        if kind == "body":
+            sc["lr_body"] = np.concatenate([base["lr_body"], np.zeros(others, np.uint32)])
+        ctx = gs.Context(sc, friction_mode=int(kind == "depth_friction"))
+        for _ in range(4):
+            ctx.frame(1.0 / 60.0, 2, 5)
+        states.append([ctx.read(f)[:n].view(np.uint32) for f in (gs.GS_FIELD_LR_POS, gs.GS_FIELD_LR_VEL)])
+        ctx.close()
+    for s in states[1:]:
+        for a, b in zip(s, states[0]):
+            np.testing.assert_array_equal(a, b)
