@@ -2289,10 +2289,15 @@ static int upsample_fwd_seq(gs_ctx* c, const float4* lx, const float4* lv, const
     return GS_OK;
 }
 
-// From so many HR particles on the functional frame's kernels take longer
-// than their launches, so it runs on the caller's buffers directly instead of
-// as a graph between copies of them (500,000 HR: 80 us a call against 88).
-constexpr int64_t kDirectFrame = 262144;
+// From so many HR particles on the functional frame runs on the caller's
+// buffers directly instead of as a graph between copies of them.  A call on the
+// funnel, graph / direct: one stream 256,000 HR 85 / 95 us, 384,000 102 / 109,
+// 500,000 110 / 116, 600,000 131 / 131, 1 M 274 / 268, 2 M 678 / 660; three
+// streams in turn 48 / 76, 60 / 73, 72 / 74, 86 / 82, 173 / 150, 502 / 468; a
+// context's first call at 500,000 523 / 355, which captures.  Below the line a
+// graph is faster by more than a tenth; from there to 600,000 by less, which
+// thirty calls take to win back the capture's.
+constexpr int64_t kDirectFrame = 400000;
 
 int gs_upsample_forward(gs_ctx* c, const float* lr_pos, const float* lr_vel, const float* hr_pos_in,
                         const float* hr_vel_in, float* hr_pos_out, float* hr_vel_out, float dt)

@@ -53,6 +53,35 @@ def test_functional_frame_routes(n_low, ratio, form, graphs):
     ctx.close()
 
 
+@pytest.mark.parametrize("graphs", [False, True])
+@pytest.mark.parametrize("form", ["plain", "in_place", "misaligned"])
+def test_functional_frame_routes_at_the_direct_route(form, graphs):
+    test_functional_frame_routes(16000, 25, form, graphs)      # 400,000 HR
+
+
+@pytest.mark.parametrize("n_low, copies", [(10486, 2), (15999, 2), (16000, 1)])
+def test_functional_frame_is_direct_only_above_its_line(n_low, copies):
+    # the route between copies has one launch more, that of the results
+    import torch
+
+    import paper_2308_01629_gb300 as gs
+    sc = scenes.funnel(n_low=n_low, ratio=25)
+    with torch.cuda.stream(torch.cuda.Stream()):
+        ctx = gs.Context(sc, stream="torch")
+        ctx.set_graphs(True)
+        ins = [torch.from_numpy(sc[k]).cuda() for k in ("lr_pos", "lr_vel", "hr_pos", "hr_vel")]
+        outs = [torch.zeros_like(t) for t in ins[2:]]
+        n = []
+        for off in (0, 1):      # misaligned buffers go between copies, by the driver's
+            bufs = [t if not off else torch.zeros(t.numel() + 1, device="cuda")[1:].copy_(t.reshape(-1)) for t in ins + outs]
+            k0 = ctx.launches()
+            assert gs.gs_upsample_forward(ctx.ctx, *[t.data_ptr() for t in bufs], DT) == gs.GS_OK
+            ctx.sync()
+            n.append(ctx.launches() - k0)
+        ctx.close()
+    assert n[0] - n[1] == copies
+
+
 @pytest.mark.parametrize("iters", [0, 4])
 @pytest.mark.parametrize("n_stab", [0, 2])
 def test_taped_step_and_its_reverse_equal_the_recording_ones(n_stab, iters):
