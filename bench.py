@@ -56,8 +56,8 @@ FLUSH_BYTES = 512 << 20
 # DRAM bytes of one upsampling launch on this workload, and its DRAM, SM and
 # issue utilisation, from an ncu capture of the kernel source with this hash
 # (profiles/); reported only while the source is unchanged.
-TRAFFIC_CAPTURE = {"source_sha1": "9024c95ff09a363a6c48ec63cde3b88ea4c2ac90", "bytes": 73041664,
-                   "dram_throughput_pct": 7.5, "sm_throughput_pct": 69.9, "issue_active_pct": 73.6}
+TRAFFIC_CAPTURE = {"source_sha1": "1a519aef290a2cbafaebe1117863c8275c27e8c3", "bytes": 72020480,
+                   "dram_throughput_pct": 7.3, "sm_throughput_pct": 69.5, "issue_active_pct": 73.2}
 
 
 class L2Flush:

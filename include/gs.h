@@ -179,7 +179,10 @@ void gs_default_params(gs_params* p);
  * particles); r_high: HR radius (<= 0 selects r_low * ratio^(-1/3)); ratio:
  * HR per LR (>= 1).  cuda_stream: a cudaStream_t the context enqueues on, or
  * NULL for a stream owned by the context.  The particle state starts at zero
- * and is loaded with gs_write.  Errors: GS_ERR_ARG, GS_ERR_OOM, GS_ERR_CUDA. */
+ * and is loaded with gs_write.  A grid of up to 4,194,303 cells (cells of
+ * 3 r_low over the scene box, all scenes together) takes 68 bytes per cell for
+ * the binning of the LR set, whatever its particles; a larger one none.
+ * Errors: GS_ERR_ARG, GS_ERR_OOM, GS_ERR_CUDA. */
 int gs_create(const gs_scene* scene, float r_low, float r_high, int ratio, void* cuda_stream, gs_ctx** out);
 
 /* Create one context for n_scenes independent scenes (the batched pattern
@@ -343,7 +346,7 @@ int gs_hr_slab_assemble(gs_ctx* ctx, const void* pos, const void* vel, size_t by
  * far becomes the cell's sample.  Cells are taken in 27 phases: phase
  * (cx mod 3) + 3 (cy mod 3) + 9 (cz mod 3) ascending (cells of one phase
  * never compete, so their order within the phase does not matter).  All
- * decisions in double precision.
+ * decisions are those of double precision.
  *   vertices   double[n_vertices][3];  triangles int32[n_triangles][3],
  *              counter-clockwise seen from outside, indices < n_vertices;
  *   candidates double[n_candidates][3], n_candidates < 2^31;
@@ -352,7 +355,8 @@ int gs_hr_slab_assemble(gs_ctx* ctx, const void* pos, const void* vel, size_t by
  *              cell order (at most capacity); *n_selected their number;
  *   inside     (optional) uint8[n_candidates]: 1 for candidates inside.
  * Host arrays; synchronous; uses the current device with device memory of
- * its own, freed on return.  GS_ERR_ARG (null pointers, r <= 0, a triangle
+ * its own (61 bytes per candidate, 60 per triangle, 24 per vertex, 8 per
+ * cell), freed on return.  GS_ERR_ARG (null pointers, r <= 0, a triangle
  * index out of range, more than 2^31 - 2 cells), GS_ERR_DOMAIN (a
  * non-finite coordinate), both before any device work; GS_ERR_CAPACITY when
  * more than capacity samples were chosen (*n_selected is their number);
@@ -472,7 +476,9 @@ int gs_gather_timer_ms(gs_ctx* ctx, float* ms);
 
 /* Launch shape of the upsampling kernel: warps per block (4, 8 or 16) and
  * blocks per SM of a persistent grid that pulls 32-particle work items from
- * an atomic counter (0: one warp per item, no persistent loop). */
+ * an atomic counter (0: one warp per item, no persistent loop).  A context
+ * starts with a shape chosen by its number of items; one that is set here or
+ * by gs_autotune stays. */
 int gs_set_tuning(gs_ctx* ctx, int warps_per_block, int blocks_per_sm);
 
 /* Time the upsampling kernel on the current state (written out of place,

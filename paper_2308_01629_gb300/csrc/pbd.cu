@@ -198,8 +198,10 @@ __global__ void __launch_bounds__(128) k_neighbors(const PbdArgs a, const float4
 // slightly wider test than contact_term's, which decides); then the contact
 // terms of the marked ones only.
 //   two lanes    each chain lane takes its own contacts, kContactGroup at a
-//                time.  Instruction issue bounds a large pass and the chain of
-//                dependent loads a pass of one wave.
+//                time.  A pass of one wave (50,527 LR) has its SMs active for
+//                half of its time, issuing in 53 % of those cycles: start, tail
+//                and the chain of dependent loads bound it.  At 202,112 LR they
+//                are active for two thirds and issue in 69 %.
 //   eight lanes  the marked contacts of the whole warp (four particles) are
 //                listed in shared memory and evaluated 32 at a time, one per
 //                lane, and every chain adds its own terms in order: more
@@ -220,7 +222,7 @@ constexpr int kPassBlocks = 8;     // per SM
 // Eight lanes while they fill less than one wave (152 SMs x 32 warps of four
 // particles).  At 20,000 LR they gain on a dense pile (the funnel's end, 9.2
 // against 11.9 us) and lose where grains fall without contacts (the funnel's
-// frame 363 against 342 us), so the line lies below.
+// frame 304 against 263 us), so the line lies below.
 constexpr int64_t kWideMax = 16384;
 
 // Per-warp shared memory of the eight-lane form.

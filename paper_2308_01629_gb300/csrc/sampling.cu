@@ -5,10 +5,11 @@
 // every sample taken so far.  The cells are taken in 27 phases
 // (cx mod 3, cy mod 3, cz mod 3; phase index (cx mod 3) + 3 (cy mod 3) +
 // 9 (cz mod 3) ascending): two cells of a phase are three cells apart along
-// some axis, more than 2 r, so one launch takes a whole phase, one thread per
+// some axis, more than 2 r, so one launch takes a whole phase, one warp per
 // cell, with the result of taking its cells one by one.  The decisions are
-// taken in double precision with the multiplications and additions rounded
-// one by one, so that they are those of a plain sequential evaluation.
+// those of a plain sequential evaluation in double precision: taken in single
+// precision where a bound on its error allows, and in double with the
+// multiplications and additions rounded one by one where it does not.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -62,7 +63,7 @@ struct SampleGrid {
 // plane inside it).  FP64 runs at 1/64 of the FP32 rate on sm_103a: a million
 // candidates against 344 triangles took 92 ms in double precision and take
 // 1.2 ms this way (1.1 here, 0.08 in k_sample_winding), with the same
-// decisions.  Issue of FP32 instructions (about 65 per candidate and
+// decisions (a bound as below, and every case that it does not cover left open).  Issue of FP32 instructions (about 65 per candidate and
 // triangle) bounds it.
 //
 // Coordinates are scaled to the mesh's box, q' = (q - lo) / extent, and

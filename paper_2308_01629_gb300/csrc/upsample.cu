@@ -34,11 +34,14 @@
 namespace {
 
 // Launch shape where the caller sets none: blocks of four warps, one item per
-// warp, and from about two waves on (152 SMs x 28 warps) a persistent grid
-// whose warps pull items, which balances them.  Gather of a frame (before:
+// warp, and from 8,192 items on (two waves of 152 SMs x 28 warps) a persistent
+// grid whose warps pull items, which balances them.  Gather of a frame (before:
 // eight warps, one item each): cube 250 items 25 us (25; persistent 26),
 // funnel 15,625 94 (115), digging 63,160 157 (220; one item per warp 165),
-// 2 x 2 m bed 252,640 576 (856; 619), 64 scenes 143,255 506 (609; 538).
+// 2 x 2 m bed 252,640 576 (856; 619), 64 scenes 143,255 506 (609; 538).  In
+// between the two are alike (funnels of 2,000 to 31,250 items, one per warp /
+// persistent: 43.0 / 43.0, 52.0 / 52.7, 78.8 / 80.1, 98.8 / 95.2, 312.6 /
+// 317.4), so the line is where a wave is full, not where they cross.
 constexpr int64_t kPersistentItems = 8192;
 constexpr int kAutoBlocks = 7;   // 28 warps per SM: 72 registers; 8 spill (digging 162 us), 6 are 164
 constexpr int kBuf = 64;   // staged LR per warp; flushed at >= 32
