@@ -979,6 +979,15 @@ bool capturable(const gs_ctx* c)
            c->stream != cudaStreamPerThread;
 }
 
+// Whether the caller is capturing the context's stream.
+bool caller_captures(const gs_ctx* c)
+{
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (!c->capturing && cudaStreamIsCapturing(c->stream, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return false;
+}
+
 HostAfter host_after(const gs_ctx* c)
 {
     HostAfter h;
@@ -2315,7 +2324,9 @@ int gs_upsample_forward(gs_ctx* c, const float* lr_pos, const float* lr_vel, con
     if (M == 0) return copy_all(c, {{lr_pos, c->lr_pos, N}, {lr_vel, c->lr_vel, N}});
     const bool aligned =
         (((uintptr_t)hr_pos_in | (uintptr_t)hr_vel_in | (uintptr_t)hr_pos_out | (uintptr_t)hr_vel_out) & 15u) == 0;
-    if (M >= kDirectFrame && aligned) {
+    // the copies are for the graph: without one, and in a capture of the
+    // caller's (which takes neither another capture nor an allocation), direct
+    if (aligned && (M >= kDirectFrame || !capturable(c) || caller_captures(c))) {
         st = copy_all(c, {{lr_pos, c->lr_pos, N}, {lr_vel, c->lr_vel, N}});
         if (st) return st;
         return upsample_fwd_seq(c, c->lr_pos, c->lr_vel, (const float4*)hr_pos_in, (const float4*)hr_vel_in,

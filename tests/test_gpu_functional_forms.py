@@ -82,6 +82,56 @@ def test_functional_frame_is_direct_only_above_its_line(n_low, copies):
     assert n[0] - n[1] == copies
 
 
+def test_functional_frame_is_direct_without_graphs():
+    import torch
+
+    import paper_2308_01629_gb300 as gs
+    sc = scenes.funnel(n_low=1000, ratio=7)
+    with torch.cuda.stream(torch.cuda.Stream()):
+        ctx = gs.Context(sc, stream="torch")
+        ins = [torch.from_numpy(sc[k]).cuda() for k in ("lr_pos", "lr_vel", "hr_pos", "hr_vel")]
+        outs = [torch.zeros_like(t) for t in ins[2:]]
+        n = []
+        for graphs in (False, True):
+            ctx.set_graphs(graphs)
+            k0 = ctx.launches()
+            assert gs.gs_upsample_forward(ctx.ctx, *[t.data_ptr() for t in ins + outs], DT) == gs.GS_OK
+            ctx.sync()
+            n.append(ctx.launches() - k0)
+        ctx.close()
+    assert n[1] - n[0] == 1      # the copy of the results
+
+
+@pytest.mark.parametrize("graphs", [False, True])
+@pytest.mark.parametrize("n_low, ratio", [(1000, 7), (10486, 25), (16000, 25)])
+def test_functional_frame_in_a_capture_of_the_caller(n_low, ratio, graphs):
+    import torch
+
+    import paper_2308_01629_gb300 as gs
+    sc = scenes.stir(scenes.funnel(n_low=n_low, ratio=ratio), seed=4)
+    ref = _frame_of_the_context(gs, sc)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        ctx = gs.Context(sc, stream="torch")
+        ctx.set_graphs(graphs)
+        ins = [torch.from_numpy(sc[k]).cuda() for k in ("lr_pos", "lr_vel", "hr_pos", "hr_vel")]
+        outs = [torch.zeros_like(t) for t in ins[2:]]
+        ctx.sync()
+        graph = torch.cuda.CUDAGraph()
+        graph.capture_begin(capture_error_mode="global")
+        rc = gs.gs_upsample_forward(ctx.ctx, *[t.data_ptr() for t in ins + outs], DT)
+        graph.capture_end()
+        assert rc == gs.GS_OK
+        for _ in range(2):
+            for t in outs:
+                t.zero_()
+            graph.replay()
+            stream.synchronize()
+            for t, r in zip(outs, ref):
+                np.testing.assert_array_equal(t.cpu().numpy().view(np.uint32), r.view(np.uint32))
+        ctx.close()
+
+
 @pytest.mark.parametrize("iters", [0, 4])
 @pytest.mark.parametrize("n_stab", [0, 2])
 def test_taped_step_and_its_reverse_equal_the_recording_ones(n_stab, iters):
